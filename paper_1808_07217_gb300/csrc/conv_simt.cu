@@ -1,0 +1,550 @@
+// 3x3 convolutions (zero padding 1) on the fp32 cores, G replicas per launch.
+//
+// The fp32 mode's convolutions (tensor cores cannot give fp32-exact products) and the SIMT form of
+// the bf16 ones.  All three products of a layer run as register-tiled shared-memory kernels on the
+// packed two-lane fp32 multiply-add (fma.rn.f32x2: two roundings, each that of fmaf, in one issue
+// slot), and all are bound by that pipe: per shared-memory load a thread does 8 to 12 of them.
+#include <algorithm>
+
+#include "common.cuh"
+#include "lsgd_internal.h"
+
+namespace lsgd {
+namespace {
+
+using u64 = unsigned long long;
+
+__device__ __forceinline__ u64 pack2(float lo, float hi) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(u64 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ void fma2(u64& d, u64 a, u64 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void add2(u64& d, u64 a) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a));
+}
+
+// Four consecutive elements of an activation tensor as fp32.
+__device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const uint16_t* p) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(bf2f((uint16_t)(u.x & 0xffffu)), bf2f((uint16_t)(u.x >> 16)),
+                     bf2f((uint16_t)(u.y & 0xffffu)), bf2f((uint16_t)(u.y >> 16)));
+}
+
+// A tile of pixels: ti images x th rows x tw columns (powers of two) of the output grid, chosen so
+// that images narrower than the tile still fill it.
+struct Tile {
+  int tw, th, ti;      // log2
+  int nx, ny;          // tiles across and down an image
+  int tiles;           // tiles of one replica
+};
+
+int log2_ceil(int v) {
+  int l = 0;
+  while ((1 << l) < v) ++l;
+  return l;
+}
+
+Tile tile_of(int B, int H, int W, int px_log2) {
+  Tile t;
+  t.tw = std::max(3, std::min(5, log2_ceil(W)));
+  t.th = std::min(px_log2 - t.tw, log2_ceil(H));
+  t.ti = px_log2 - t.tw - t.th;
+  t.nx = (W + (1 << t.tw) - 1) >> t.tw;
+  t.ny = (H + (1 << t.th) - 1) >> t.th;
+  t.tiles = ((B + (1 << t.ti) - 1) >> t.ti) * t.nx * t.ny;
+  return t;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Forward and data gradient: out[g][b][y][x][co] = sum over taps t and ci of
+// in[g][b][y S + t / 3 - 1][x S + t % 3 - 1][ci] w_t[co][ci].  The data gradient is this with the
+// output gradient as input and w_t[ci][co] = w[co][8 - t][ci] (flip); a stride-2 layer's reads the
+// output gradient with zeros between its pixels (up).
+//
+// A CTA computes 256 pixels x 16 channels, a thread 4 consecutive pixels x 8 channels (4 packed
+// pairs).  Eight input channels at a time, the tile's input with its halo is staged as one plane
+// per channel -- a warp's reads of its rows are then consecutive -- and their weights as
+// [channel][tap][16]; all lanes of a warp read the same weights.  Per channel and kernel row a
+// thread loads 6 inputs (9 at stride 2) in two or three loads and 24 weights in six, for 48 packed
+// multiply-adds.  The eight channels' products are summed by themselves and then added to the
+// running sum, which halves the length of the longest chain of roundings at 16 channels and keeps
+// it at 72 + Cin / 8 for any Cin.
+// The 16-channel tile over 256 pixels reads each input once per 16 outputs; wider tiles of 32
+// channels leave too few CTAs on the later, smaller stages.
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.73 ms forward and data gradients
+// (7.3 ms with one thread per pixel that loaded a weight per multiply-add).
+constexpr int kFwThreads = 128, kFwPxLog2 = 8, kFwCo = 16, kFwCi = 8;
+
+struct ConvFwArgs {
+  const void* in;
+  const void* w;
+  int64_t w_gs;
+  float* out;
+  int B, Hi, Wi, Ci, Ho, Wo, Co;
+  int up, flip;
+  Tile t;
+  int pr, pc, pitch;  // patch rows and columns per image, row pitch (floats)
+  // the block's shortcut: out += sc_dout * (sc_act > 0) at (y / sc_s, x / sc_s) where both are whole
+  const float* sc_dout;
+  const void* sc_act;
+  int sc_s, sc_H, sc_W, sc_C;
+};
+
+template <typename TA, int S>
+__global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __grid_constant__ ConvFwArgs a) {
+  pdl_begin();
+  extern __shared__ __align__(16) float fw_sm[];
+  const int plane = (a.pr * a.pitch) << a.t.ti;
+  float* patch = fw_sm;                                   // [kFwCi][ti][pr][pitch]
+  float* ws = patch + kFwCi * plane;                      // [kFwCi][9][kFwCo]
+  int2* table = reinterpret_cast<int2*>(ws + kFwCi * 9 * kFwCo);  // per patch pixel: source, place
+  const int tid = threadIdx.x, g = blockIdx.z, co0 = blockIdx.y * kFwCo;
+  int tile = blockIdx.x;
+  const int x0 = (tile % a.t.nx) << a.t.tw;
+  tile /= a.t.nx;
+  const int y0 = (tile % a.t.ny) << a.t.th;
+  const int b0 = (tile / a.t.ny) << a.t.ti;
+  const int npx = (a.pr * a.pc) << a.t.ti;
+  for (int e = tid; e < npx; e += kFwThreads) {
+    const int px = e % a.pc, r = e / a.pc, py = r % a.pr, im = r / a.pr;
+    int iy = y0 * S + py - 1, ix = x0 * S + px - 1;
+    bool in = b0 + im < a.B && iy >= 0 && ix >= 0;
+    if (a.up) {
+      in = in && !((iy | ix) & 1);
+      iy >>= 1;
+      ix >>= 1;
+    }
+    in = in && iy < a.Hi && ix < a.Wi;
+    table[e] = make_int2(in ? ((b0 + im) * a.Hi + iy) * a.Wi + ix : -1, (im * a.pr + py) * a.pitch + px);
+  }
+  const TA* in = reinterpret_cast<const TA*>(a.in) + (int64_t)g * a.B * a.Hi * a.Wi * a.Ci;
+  const TA* w = reinterpret_cast<const TA*>(a.w) + (int64_t)g * a.w_gs;
+
+  const int pg = tid & 63, cog = tid >> 6;  // pixel group (a warp's are 32 in a row), channel half
+  const int gx = (pg << 2) & ((1 << a.t.tw) - 1), gr = (pg << 2) >> a.t.tw;
+  const int gy = gr & ((1 << a.t.th) - 1), gi = gr >> a.t.th;
+  const float* prow = patch + (gi * a.pr + gy * S) * a.pitch + gx * S;
+  const float* wrow = ws + 8 * cog;
+
+  u64 sum[4][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sum[p][q] = 0ull;
+
+  for (int c0 = 0; c0 < a.Ci; c0 += kFwCi) {
+    const int nc = min(kFwCi, a.Ci - c0);
+    __syncthreads();  // the table is written; the previous channels have been read
+    if ((a.Ci & 3) == 0) {
+      for (int e = tid; e < npx; e += kFwThreads) {
+        const int2 s = table[e];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (4 * h >= nc) break;
+          const float4 v = s.x >= 0 ? load4(in + (int64_t)s.x * a.Ci + c0 + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+          float* d = patch + 4 * h * plane + s.y;
+          d[0] = v.x;
+          d[plane] = v.y;
+          d[2 * plane] = v.z;
+          d[3 * plane] = v.w;
+        }
+      }
+    } else {
+      for (int e = tid; e < npx; e += kFwThreads) {
+        const int2 s = table[e];
+        for (int c = 0; c < nc; ++c)
+          patch[c * plane + s.y] = s.x >= 0 ? Elem<TA>::load(in + (int64_t)s.x * a.Ci + c0 + c) : 0.f;
+      }
+    }
+    // weights, consecutive threads on consecutive elements of the tensor
+    for (int e = tid; e < kFwCi * 9 * kFwCo; e += kFwThreads) {
+      int co, t, c;
+      float v = 0.f;
+      if (!a.flip) {
+        c = e % kFwCi, t = (e / kFwCi) % 9, co = e / (9 * kFwCi);
+        if (c < nc && co0 + co < a.Co) v = Elem<TA>::load(w + ((int64_t)(co0 + co) * 9 + t) * a.Ci + c0 + c);
+      } else {
+        co = e % kFwCo, t = (e / kFwCo) % 9, c = e / (9 * kFwCo);
+        if (c < nc && co0 + co < a.Co) v = Elem<TA>::load(w + ((int64_t)(c0 + c) * 9 + 8 - t) * a.Co + co0 + co);
+      }
+      ws[(c * 9 + t) * kFwCo + co] = v;
+    }
+    __syncthreads();
+    u64 acc[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[p][q] = 0ull;
+    for (int c = 0; c < nc; ++c) {
+#pragma unroll
+      for (int kh = 0; kh < 3; ++kh) {
+        const float* r = prow + c * plane + kh * a.pitch;
+        constexpr int NV = 3 * S + 3;
+        u64 v[NV];
+#pragma unroll
+        for (int i = 0; i + 4 <= NV; i += 4) {
+          const float4 f = *reinterpret_cast<const float4*>(r + i);
+          v[i] = pack2(f.x, f.x);
+          v[i + 1] = pack2(f.y, f.y);
+          v[i + 2] = pack2(f.z, f.z);
+          v[i + 3] = pack2(f.w, f.w);
+        }
+        if (S == 1) {
+          const float2 f = *reinterpret_cast<const float2*>(r + 4);
+          v[4] = pack2(f.x, f.x);
+          v[5] = pack2(f.y, f.y);
+        } else {
+          v[NV - 1] = pack2(r[8], r[8]);
+        }
+#pragma unroll
+        for (int kw = 0; kw < 3; ++kw) {
+          const ulonglong2* wp = reinterpret_cast<const ulonglong2*>(wrow + (c * 9 + kh * 3 + kw) * kFwCo);
+          const ulonglong2 w0 = wp[0], w1 = wp[1];
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const u64 x = v[p * S + kw];
+            fma2(acc[p][0], x, w0.x);
+            fma2(acc[p][1], x, w0.y);
+            fma2(acc[p][2], x, w1.x);
+            fma2(acc[p][3], x, w1.y);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) add2(sum[p][q], acc[p][q]);
+  }
+
+  const int b = b0 + gi, y = y0 + gy;
+  if (b >= a.B || y >= a.Ho) return;
+  const int co = co0 + 8 * cog;
+  const int64_t img = (int64_t)g * a.B + b;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int x = x0 + gx + p;
+    if (x >= a.Wo) break;
+    float o[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 f = unpack2(sum[p][q]);
+      o[2 * q] = f.x;
+      o[2 * q + 1] = f.y;
+    }
+    if (a.sc_dout && y % a.sc_s == 0 && x % a.sc_s == 0) {
+      const int64_t e = ((img * a.sc_H + y / a.sc_s) * a.sc_W + x / a.sc_s) * a.sc_C + co;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (co + i < a.Co && Elem<TA>::load(reinterpret_cast<const TA*>(a.sc_act) + e + i) > 0.f)
+          o[i] += a.sc_dout[e + i];
+    }
+    float* dst = a.out + ((img * a.Ho + y) * a.Wo + x) * a.Co + co;
+    if ((a.Co & 3) == 0) {
+      if (co < a.Co) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+      if (co + 4 < a.Co) *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (co + i < a.Co) dst[i] = o[i];
+    }
+  }
+}
+
+template <typename TA, int S>
+cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
+  a.t = tile_of(a.B, a.Ho, a.Wo, kFwPxLog2);
+  a.pr = ((1 << a.t.th) - 1) * S + 3;
+  a.pc = ((1 << a.t.tw) - 1) * S + 3;
+  a.pitch = (a.pc + 3) / 4 * 4;  // rows start on 16 bytes
+  const size_t smem = (size_t)kFwCi * ((a.pr * a.pitch) << a.t.ti) * 4 + kFwCi * 9 * kFwCo * 4 +
+                      (size_t)((a.pr * a.pc) << a.t.ti) * sizeof(int2);
+  const dim3 grid(a.t.tiles, (a.Co + kFwCo - 1) / kFwCo, G);
+  if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
+  static int attr_dev = -1;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (attr_dev != dev) {
+    e = cudaFuncSetAttribute(conv3x3_simt_kernel<TA, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             100 * 1024);
+    if (e != cudaSuccess) return e;
+    attr_dev = dev;
+  }
+  return launch_pdl(conv3x3_simt_kernel<TA, S>, grid, dim3(kFwThreads), smem, s, a);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Weight gradient: part[g][q][co][t][ci] = sum over the pixels of range q of
+// dy[p][co] x[p S + tap t][ci]; the ranges' partials are added in order by a second kernel.
+//
+// A CTA takes 16 output x 16 input channels and a range of 128-pixel tiles, staged as they lie in
+// memory (64 bytes a pixel) by asynchronous copies, the next tile's while this one is summed.  Warp
+// w works on kernel row w % 3; its 16 lanes of a half cover 4 x 4 blocks of 4 output x 4 input
+// channels, and the four half-warps of a kernel row take rows r, r + 4, ... of the tile.  A thread
+// walks its row four pixels at a time: one load per pixel of dy and of x (two at stride 2; the
+// columns that the three kernel columns share stay in registers), 24 packed multiply-adds.  At the end
+// the four rows' sums are added in a fixed order.
+// An accumulator's chain is a tile range's pixels / 4 (a few hundred roundings; one thread used to
+// add 2,048).
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.86 ms (46.7 ms with 16 pixels staged
+// between two barriers and a shared-memory load per multiply-add).
+constexpr int kWgThreads = 192, kWgPxLog2 = 7;
+
+struct ConvWgArgs {
+  const void* x;
+  const void* dy;
+  float* part;
+  int B, Hi, Wi, Ci, Ho, Wo, Co;
+  int nq, ci_blocks;
+  Tile t;
+  int pr, pc, xpitch, dpitch;  // x patch rows and columns per image; row pitches in pixels of 16 floats
+};
+
+__device__ __forceinline__ void cp_async(float* dst, const void* src, int bytes, bool in) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  const int n = in ? bytes : 0;
+  if (bytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// One pixel's 16 channels c0 .. c0 + 15 (zeros from C on, and all zeros if !in) to dst; four lanes
+// (q = 0 .. 3) per pixel.
+template <typename TA>
+__device__ __forceinline__ void stage_px(float* dst, const TA* base, int64_t px, int C, int c0, int q,
+                                         bool in) {
+  const int c = c0 + 4 * q;
+  const TA* src = base + (in ? px * C + c : 0);
+  if constexpr (sizeof(TA) == 4) {
+    if ((C & 3) == 0) {
+      const bool ok = in && c < C;
+      cp_async(dst + 4 * q, ok ? src : base, 16, ok);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const bool ok = in && c + i < C;
+        cp_async(dst + 4 * q + i, ok ? src + i : base, 4, ok);
+      }
+    }
+  } else {
+    float v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = in && c + i < C ? Elem<TA>::load(src + i) : 0.f;
+    *reinterpret_cast<float4*>(dst + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+}
+
+template <typename TA, int S>
+__global__ void __launch_bounds__(kWgThreads, 3) conv_wgrad_simt_kernel(const __grid_constant__ ConvWgArgs a) {
+  pdl_begin();
+  extern __shared__ __align__(16) float wg_sm[];
+  const int rows = 1 << (a.t.th + a.t.ti);   // rows of the tile
+  const int dfl = rows * a.dpitch * 16, xfl = (a.pr << a.t.ti) * a.xpitch * 16;  // floats
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = blockIdx.z, q = blockIdx.x;
+  const int co0 = (blockIdx.y / a.ci_blocks) * 16, ci0 = (blockIdx.y % a.ci_blocks) * 16;
+  const int t_lo = (int)((int64_t)q * a.t.tiles / a.nq), t_hi = (int)((int64_t)(q + 1) * a.t.tiles / a.nq);
+  const TA* dy = reinterpret_cast<const TA*>(a.dy) + (int64_t)g * a.B * a.Ho * a.Wo * a.Co;
+  const TA* x = reinterpret_cast<const TA*>(a.x) + (int64_t)g * a.B * a.Hi * a.Wi * a.Ci;
+
+  auto stage = [&](int tile, float* buf) {
+    const int x0 = (tile % a.t.nx) << a.t.tw;
+    tile /= a.t.nx;
+    const int y0 = (tile % a.t.ny) << a.t.th, b0 = (tile / a.t.ny) << a.t.ti;
+    for (int e = tid; e < rows << (a.t.tw + 2); e += kWgThreads) {
+      const int p = e >> 2, c = p & ((1 << a.t.tw) - 1), r = p >> a.t.tw;
+      const int y = y0 + (r & ((1 << a.t.th) - 1)), b = b0 + (r >> a.t.th), xx = x0 + c;
+      const bool in = b < a.B && y < a.Ho && xx < a.Wo;
+      stage_px(buf + (r * a.dpitch + c) * 16, dy, ((int64_t)b * a.Ho + y) * a.Wo + xx, a.Co, co0, e & 3, in);
+    }
+    float* xb = buf + dfl;
+    for (int r = warp; r < a.pr << a.t.ti; r += kWgThreads / 32) {
+      const int im = r / a.pr, iy = y0 * S + (r - im * a.pr) - 1, b = b0 + im;
+      const bool row_in = b < a.B && iy >= 0 && iy < a.Hi;
+      for (int e = lane; e < a.pc * 4; e += 32) {
+        const int c = e >> 2, ix = x0 * S + c - 1;
+        const bool in = row_in && ix >= 0 && ix < a.Wi;
+        stage_px(xb + (r * a.xpitch + c) * 16, x, ((int64_t)b * a.Hi + iy) * a.Wi + ix, a.Ci, ci0, e & 3, in);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  const int kh = warp % 3, slice = 2 * (warp / 3) + (lane >> 4);
+  const int cob = (lane >> 2) & 3, cib = lane & 3;
+  u64 acc[3][4][2];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) acc[k][o][0] = acc[k][o][1] = 0ull;
+
+  if (t_lo < t_hi) stage(t_lo, wg_sm);
+  for (int t = t_lo; t < t_hi; ++t) {
+    float* buf = wg_sm + ((t - t_lo) & 1) * (dfl + xfl);
+    if (t + 1 < t_hi) {
+      stage(t + 1, wg_sm + ((t + 1 - t_lo) & 1) * (dfl + xfl));
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    for (int r = slice; r < rows; r += 4) {
+      const int im = r >> a.t.th, y = r & ((1 << a.t.th) - 1);
+      const float* dr = buf + r * a.dpitch * 16 + 4 * cob;
+      const float* xr = buf + dfl + (im * a.pr + y * S + kh) * a.xpitch * 16 + 4 * cib;
+      constexpr int NX = 3 * S + 3;  // columns under four pixels
+      ulonglong2 xv[NX];
+#pragma unroll
+      for (int i = 0; i < 3 - S; ++i) xv[i] = *reinterpret_cast<const ulonglong2*>(xr + i * 16);
+      for (int c = 0; c < 1 << a.t.tw; c += 4) {
+        float4 d[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) d[p] = *reinterpret_cast<const float4*>(dr + (c + p) * 16);
+#pragma unroll
+        for (int i = 3 - S; i < NX; ++i)
+          xv[i] = *reinterpret_cast<const ulonglong2*>(xr + (c * S + i) * 16);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const u64 dd[4] = {pack2(d[p].x, d[p].x), pack2(d[p].y, d[p].y), pack2(d[p].z, d[p].z),
+                             pack2(d[p].w, d[p].w)};
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+              fma2(acc[k][o][0], dd[o], xv[p * S + k].x);
+              fma2(acc[k][o][1], dd[o], xv[p * S + k].y);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 3 - S; ++i) xv[i] = xv[i + 4 * S];
+      }
+    }
+    __syncthreads();  // the buffer is free for the tile after next
+  }
+
+  // the four rows' sums: (0 + 1) + (2 + 3), across the half-warps, then through shared memory
+  float* red = wg_sm;  // [3][16 lanes][48]
+  float v[48];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 f = unpack2(acc[k][o][h]);
+        v[(k * 4 + o) * 4 + 2 * h] = f.x;
+        v[(k * 4 + o) * 4 + 2 * h + 1] = f.y;
+      }
+#pragma unroll
+  for (int i = 0; i < 48; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
+  if (warp >= 3 && lane < 16)
+#pragma unroll
+    for (int i = 0; i < 48; ++i) red[(kh * 48 + i) * 16 + lane] = v[i];
+  __syncthreads();
+  if (warp < 3 && lane < 16) {
+    float* out = a.part + ((int64_t)g * a.nq + q) * a.Co * 9 * a.Ci;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const int co = co0 + 4 * cob + o, ci = ci0 + 4 * cib;
+        if (co >= a.Co) continue;
+        float* dst = out + ((int64_t)co * 9 + kh * 3 + k) * a.Ci + ci;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int e = (k * 4 + o) * 4 + i;
+          if (ci + i < a.Ci) dst[i] = v[e] + red[(kh * 48 + e) * 16 + lane];
+        }
+      }
+  }
+}
+
+template <typename TA, int S>
+cudaError_t launch_wg(ConvWgArgs a, int G, cudaStream_t s) {
+  a.pr = ((1 << a.t.th) - 1) * S + 3;
+  a.pc = ((1 << a.t.tw) - 1) * S + 3;
+  // odd row pitches: the two half-warps of a warp, a row apart, then read different banks
+  a.xpitch = a.pc | 1;
+  a.dpitch = (1 << a.t.tw) | 1;
+  const size_t floats = (size_t)((a.dpitch << (a.t.th + a.t.ti)) + (a.pr << a.t.ti) * a.xpitch) * 16;
+  const size_t smem = std::max<size_t>(2 * floats, 3 * 48 * 16) * 4;
+  const dim3 grid(a.nq, ((a.Co + 15) / 16) * a.ci_blocks, G);
+  if (grid.y > 65535 || grid.z > 65535 || smem > 160 * 1024) return cudaErrorInvalidValue;
+  static int attr_dev = -1;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (attr_dev != dev) {
+    e = cudaFuncSetAttribute(conv_wgrad_simt_kernel<TA, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             160 * 1024);
+    if (e != cudaSuccess) return e;
+    attr_dev = dev;
+  }
+  return launch_pdl(conv_wgrad_simt_kernel<TA, S>, grid, dim3(kWgThreads), smem, s, a);
+}
+
+}  // namespace
+
+cudaError_t launch_conv3x3_simt(const ConvSimtArgs& c, cudaStream_t s) {
+  if (c.G < 1 || c.B < 1 || (c.stride != 1 && c.stride != 2) || c.cin < 1 || c.cout < 1)
+    return cudaErrorInvalidValue;
+  ConvFwArgs a{};
+  a.in = c.in;
+  a.w = c.w;
+  a.w_gs = c.w_gs;
+  a.out = c.out;
+  a.B = c.B;
+  if (!c.dgrad) {
+    a.Hi = c.hin, a.Wi = c.win, a.Ci = c.cin, a.Ho = c.hout, a.Wo = c.wout, a.Co = c.cout;
+  } else {
+    a.Hi = c.hout, a.Wi = c.wout, a.Ci = c.cout, a.Ho = c.hin, a.Wo = c.win, a.Co = c.cin;
+    a.flip = 1;
+    a.up = c.stride == 2;
+    a.sc_dout = c.sc_dout;
+    a.sc_act = c.sc_act;
+    a.sc_s = c.stride;
+    a.sc_H = c.hout, a.sc_W = c.wout, a.sc_C = c.cout;
+  }
+  if ((int64_t)a.B * a.Hi * a.Wi > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const bool two = !c.dgrad && c.stride == 2;
+  if (c.bf16) return two ? launch_fw<uint16_t, 2>(a, c.G, s) : launch_fw<uint16_t, 1>(a, c.G, s);
+  return two ? launch_fw<float, 2>(a, c.G, s) : launch_fw<float, 1>(a, c.G, s);
+}
+
+// Ranges of one replica: about four CTAs per SM over the replicas and channel blocks, at least one
+// tile each.
+int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout) {
+  const int blocks = ((cout + 15) / 16) * ((cin + 15) / 16);
+  const int tiles = tile_of(B, hout, wout, kWgPxLog2).tiles;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 4LL * kNumSMs / ((int64_t)G * blocks)));
+}
+
+cudaError_t launch_conv_wgrad_simt(const ConvSimtArgs& c, const void* dy, float* part, cudaStream_t s) {
+  if (c.G < 1 || c.B < 1 || (c.stride != 1 && c.stride != 2) || c.cin < 1 || c.cout < 1)
+    return cudaErrorInvalidValue;
+  ConvWgArgs a{};
+  a.x = c.in;
+  a.dy = dy;
+  a.part = part;
+  a.B = c.B;
+  a.Hi = c.hin, a.Wi = c.win, a.Ci = c.cin, a.Ho = c.hout, a.Wo = c.wout, a.Co = c.cout;
+  a.ci_blocks = (c.cin + 15) / 16;
+  a.t = tile_of(c.B, c.hout, c.wout, kWgPxLog2);
+  a.nq = conv_wgrad_simt_ranges(c.G, c.B, c.hout, c.wout, c.cin, c.cout);
+  if (c.bf16)
+    return c.stride == 2 ? launch_wg<uint16_t, 2>(a, c.G, s) : launch_wg<uint16_t, 1>(a, c.G, s);
+  return c.stride == 2 ? launch_wg<float, 2>(a, c.G, s) : launch_wg<float, 1>(a, c.G, s);
+}
+
+}  // namespace lsgd

@@ -252,6 +252,28 @@ bool make_tma_map_conv(CUtensorMap* map, const void* base, int ck, int win, int 
 
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t stream);
 
+// ---- 3x3 convolutions on the fp32 cores (conv_simt.cu): any channels, sizes, stride 1 or 2 ----
+// The layer [G][B][hin][win][cin] -> [G][B][hout][wout][cout], weights [cout][3][3][cin] with
+// replica stride w_gs; bf16: in, w and sc_act hold bf16, else fp32.
+struct ConvSimtArgs {
+  bool bf16;
+  int G, B, hin, win, cin, hout, wout, cout, stride;
+  const void* in;  // forward, weight gradient: the layer's input; data gradient: its output gradient
+  const void* w;
+  int64_t w_gs;
+  float* out;      // forward: the layer's output; data gradient: the gradient of its input
+  bool dgrad;
+  // data gradient: with sc_dout [G][B][hout][wout][cout], the option-A shortcut's share
+  // sc_dout (sc_act > 0) is added at the input pixels on the stride grid, channels < cin
+  const float* sc_dout;
+  const void* sc_act;
+};
+cudaError_t launch_conv3x3_simt(const ConvSimtArgs& a, cudaStream_t stream);
+// Weight-gradient partials part [G][conv_wgrad_simt_ranges()][cout][9][cin], to be added in order.
+int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout);
+cudaError_t launch_conv_wgrad_simt(const ConvSimtArgs& a, const void* dy, float* part,
+                                   cudaStream_t stream);
+
 // ---- tcgen05 / TMEM / TMA grouped GEMM (gemm_tc.cu), bf16 operands, fp32 accumulation ----
 // A is M x Kd, B is N x Kd (as stored: "K-major" = Kd contiguous, "MN-major" = M/N contiguous),
 // both described by rank-3 TMA maps whose outermost dimension is the replica (group).

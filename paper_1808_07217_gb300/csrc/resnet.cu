@@ -35,9 +35,6 @@ constexpr int kRnChunk = 256;      // the smallest chunk inside the ResNet step 
 // Pixels per reduction chunk inside the ResNet step: 1024 on large tensors, 256 on the small
 // later stages so that they still spread over many CTAs.
 int rn_chunk(int64_t P) { return P >= 65536 ? 1024 : kRnChunk; }
-constexpr int kWgradChunk = 2048;  // pixels per weight-gradient chunk
-constexpr int kWgradTile = 16;     // pixels staged per weight-gradient iteration
-constexpr int kMaxJ16 = 36;        // (9 Cin) / 16 accumulators per thread, Cin <= 64
 
 struct ConvL {
   int cin, cout, stride, hin, win, hout, wout;
@@ -50,191 +47,6 @@ int64_t rup(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 int grid_cap(int64_t items, int threads) {
   int64_t b = (items + threads - 1) / threads;
   return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)kNumSMs * 16));
-}
-
-// ------------------------------------------------------------------------------------------
-// Direct 3x3 convolution, zero padding 1: y[g][b][oh][ow][co] = sum_{kh,kw,ci}
-// in[g][b][oh s + kh - 1][ow s + kw - 1][ci] w[g][co][kh][kw][ci].  One thread per output pixel
-// and 16 output channels; the 16 channels' weights sit in shared memory.
-template <typename TA>
-__global__ void __launch_bounds__(128) conv_fwd_kernel(const TA* __restrict__ in,
-                                                       const TA* __restrict__ w, int64_t w_gs,
-                                                       float* __restrict__ y, int B, int Hin,
-                                                       int Win, int Cin, int Hout, int Wout,
-                                                       int Cout, int stride) {
-  pdl_begin();
-  extern __shared__ float ws[];  // [16][9][Cin]
-  const int g = blockIdx.z, co0 = blockIdx.y * 16;
-  const int nco = min(16, Cout - co0);
-  const TA* wg = w + (int64_t)g * w_gs;
-  const int KC = 9 * Cin;
-  for (int e = threadIdx.x; e < 16 * KC; e += blockDim.x) {
-    const int co = e / KC, r = e % KC;
-    ws[e] = co < nco ? Elem<TA>::load(wg + (int64_t)(co0 + co) * KC + r) : 0.f;
-  }
-  __syncthreads();
-  const int64_t P = (int64_t)B * Hout * Wout;
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  const int ow = (int)(p % Wout);
-  const int oh = (int)((p / Wout) % Hout);
-  const int b = (int)(p / ((int64_t)Wout * Hout));
-  float acc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-  const TA* ing = in + (int64_t)g * B * Hin * Win * Cin;
-  for (int kh = 0; kh < 3; ++kh) {
-    const int ih = oh * stride + kh - 1;
-    if (ih < 0 || ih >= Hin) continue;
-    for (int kw = 0; kw < 3; ++kw) {
-      const int iw = ow * stride + kw - 1;
-      if (iw < 0 || iw >= Win) continue;
-      const TA* src = ing + (((int64_t)b * Hin + ih) * Win + iw) * Cin;
-      const float* wk = ws + (kh * 3 + kw) * Cin;
-      for (int ci = 0; ci < Cin; ++ci) {
-        const float x = Elem<TA>::load(src + ci);
-#pragma unroll
-        for (int co = 0; co < 16; ++co) acc[co] = fmaf(x, wk[co * KC + ci], acc[co]);
-      }
-    }
-  }
-  float* dst = y + ((int64_t)g * P + p) * Cout + co0;
-  for (int co = 0; co < nco; ++co) dst[co] = acc[co];
-}
-
-// Data gradient of conv_fwd: dx[g][b][ih][iw][ci] = sum over the taps that reach (ih, iw) of
-// sum_co dy[g][b][oh][ow][co] w[g][co][kh][kw][ci], plus (option-A shortcut) the block's
-// pre-activation gradient dout * (out > 0) at (ih / s, iw / s, ci) when ih, iw are multiples of s
-// and ci < the block's input channels.
-template <typename TA>
-__global__ void __launch_bounds__(64) conv_dgrad_kernel(
-    const TA* __restrict__ dy, const TA* __restrict__ w, int64_t w_gs, float* __restrict__ dx,
-    int B, int Hin, int Win, int Cin, int Hout, int Wout, int Cout, int stride,
-    const float* __restrict__ dout, const TA* __restrict__ out_act) {
-  pdl_begin();
-  extern __shared__ float ws[];  // [Cout][9][16]
-  const int g = blockIdx.z, ci0 = blockIdx.y * 16;
-  const int nci = min(16, Cin - ci0);
-  const TA* wg = w + (int64_t)g * w_gs;
-  for (int e = threadIdx.x; e < Cout * 9 * 16; e += blockDim.x) {
-    const int ci = e % 16, tap = (e / 16) % 9, co = e / 144;
-    ws[e] = ci < nci ? Elem<TA>::load(wg + ((int64_t)co * 9 + tap) * Cin + ci0 + ci) : 0.f;
-  }
-  __syncthreads();
-  const int64_t P = (int64_t)B * Hin * Win;
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  const int iw = (int)(p % Win);
-  const int ih = (int)((p / Win) % Hin);
-  const int b = (int)(p / ((int64_t)Win * Hin));
-  float acc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-  const TA* dyg = dy + (int64_t)g * B * Hout * Wout * Cout;
-  for (int kh = 0; kh < 3; ++kh) {
-    const int on = ih + 1 - kh;
-    if (on < 0 || on % stride) continue;
-    const int oh = on / stride;
-    if (oh >= Hout) continue;
-    for (int kw = 0; kw < 3; ++kw) {
-      const int wn = iw + 1 - kw;
-      if (wn < 0 || wn % stride) continue;
-      const int ow = wn / stride;
-      if (ow >= Wout) continue;
-      const TA* src = dyg + (((int64_t)b * Hout + oh) * Wout + ow) * Cout;
-      const float* wk = ws + (kh * 3 + kw) * 16;
-      for (int co = 0; co < Cout; ++co) {
-        const float d = Elem<TA>::load(src + co);
-#pragma unroll
-        for (int ci = 0; ci < 16; ++ci) acc[ci] = fmaf(d, wk[co * 144 + ci], acc[ci]);
-      }
-    }
-  }
-  if (dout && ih % stride == 0 && iw % stride == 0) {
-    const int64_t e = ((((int64_t)g * B + b) * Hout + ih / stride) * Wout + iw / stride) * Cout;
-    for (int ci = 0; ci < nci; ++ci)
-      if (Elem<TA>::load(out_act + e + ci0 + ci) > 0.f) acc[ci] += dout[e + ci0 + ci];
-  }
-  float* dst = dx + ((int64_t)g * P + p) * Cin + ci0;
-  for (int ci = 0; ci < nci; ++ci) dst[ci] = acc[ci];
-}
-
-// Weight gradient, pass 1: part[g][q][co][j] = sum over the pixels of chunk q of
-// dy[p][co] * im2col(in)[p][j], j = (kh 3 + kw) Cin + ci.  Thread (co = t mod 16, j0 = t / 16)
-// owns j = j0 + 16 k; pixels are staged kWgradTile at a time in shared memory.
-template <typename TA>
-__global__ void __launch_bounds__(256) conv_wgrad_partial_kernel(
-    const TA* __restrict__ dy, const TA* __restrict__ in, float* __restrict__ part, int B, int Hin,
-    int Win, int Cin, int Hout, int Wout, int Cout, int stride, int nq) {
-  pdl_begin();
-  extern __shared__ float sm[];
-  const int J = 9 * Cin;
-  float* dys = sm;                     // [kWgradTile][16]
-  float* ims = sm + kWgradTile * 16;   // [kWgradTile][J]
-  const int g = blockIdx.z, co0 = blockIdx.y * 16, q = blockIdx.x;
-  const int co = threadIdx.x & 15, j0 = threadIdx.x >> 4;
-  const int64_t P = (int64_t)B * Hout * Wout;
-  const int64_t p0 = (int64_t)q * kWgradChunk, p1 = min(P, p0 + kWgradChunk);
-  const TA* dyg = dy + (int64_t)g * P * Cout;
-  const TA* ing = in + (int64_t)g * B * Hin * Win * Cin;
-  float acc[kMaxJ16];
-#pragma unroll
-  for (int k = 0; k < kMaxJ16; ++k) acc[k] = 0.f;
-  for (int64_t pb = p0; pb < p1; pb += kWgradTile) {
-    {
-      const int pp = threadIdx.x >> 4, c = threadIdx.x & 15;
-      const int64_t p = pb + pp;
-      dys[pp * 16 + c] = (p < p1 && co0 + c < Cout) ? Elem<TA>::load(dyg + p * Cout + co0 + c) : 0.f;
-    }
-    for (int e = threadIdx.x; e < kWgradTile * J; e += blockDim.x) {
-      const int pp = e / J, j = e % J;
-      const int64_t p = pb + pp;
-      float v = 0.f;
-      if (p < p1) {
-        const int tap = j / Cin, ci = j % Cin;
-        const int ow = (int)(p % Wout), oh = (int)((p / Wout) % Hout);
-        const int b = (int)(p / ((int64_t)Wout * Hout));
-        const int ih = oh * stride + tap / 3 - 1, iw = ow * stride + tap % 3 - 1;
-        if (ih >= 0 && ih < Hin && iw >= 0 && iw < Win)
-          v = Elem<TA>::load(ing + (((int64_t)b * Hin + ih) * Win + iw) * Cin + ci);
-      }
-      ims[e] = v;
-    }
-    __syncthreads();
-    for (int pp = 0; pp < kWgradTile; ++pp) {
-      const float d = dys[pp * 16 + co];
-      const float* row = ims + pp * J;
-#pragma unroll
-      for (int k = 0; k < kMaxJ16; ++k) {
-        const int j = j0 + 16 * k;
-        if (j < J) acc[k] = fmaf(d, row[j], acc[k]);
-      }
-    }
-    __syncthreads();
-  }
-  if (co0 + co < Cout) {
-    float* dst = part + (((int64_t)g * nq + q) * Cout + co0 + co) * J;
-#pragma unroll
-    for (int k = 0; k < kMaxJ16; ++k) {
-      const int j = j0 + 16 * k;
-      if (j < J) dst[j] = acc[k];
-    }
-  }
-}
-
-// Weight gradient, pass 2: G[g][w_off + e] = sum_q part[g][q][e] in chunk order.
-__global__ void sum_partials_kernel(const float* __restrict__ part, int nq, int64_t n, int G,
-                                    float* __restrict__ out, int64_t out_gs) {
-  pdl_begin();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)G * n; t += stride) {
-    const int g = (int)(t / n);
-    const int64_t e = t % n;
-    const float* p = part + (int64_t)g * nq * n + e;
-    float s = 0.f;
-    for (int q = 0; q < nq; ++q) s += p[(int64_t)q * n];
-    out[(int64_t)g * out_gs + e] = s;
-  }
 }
 
 // BatchNorm statistics, pass 1: per chunk of pixels, the chunk mean and the sum of squared
@@ -1625,6 +1437,18 @@ lsgd_status conv_dgrad_tc(const uint16_t* dy, const uint16_t* w, int64_t w_gs, f
   return LSGD_OK;
 }
 
+// Convolution c of G replicas on the fp32 cores.
+ConvSimtArgs simt_args(const ResNetPlan* p, const ConvL& c, int G) {
+  ConvSimtArgs a{};
+  a.bf16 = p->bf16;
+  a.G = G;
+  a.B = p->B;
+  a.hin = c.hin, a.win = c.win, a.cin = c.cin;
+  a.hout = c.hout, a.wout = c.wout, a.cout = c.cout;
+  a.stride = c.stride;
+  return a;
+}
+
 // stats / nparts: where the persistent implicit kernel runs, it also writes the output's
 // partial BatchNorm statistics to stats and their count per replica to *nparts (else 0).
 template <typename TA>
@@ -1729,12 +1553,12 @@ lsgd_status conv_forward(ResNetPlan* p, int i, const void* in, const void* Wop, 
     RN_CALL(launch_gemm_tc(t, s));
     return LSGD_OK;
   }
-  dim3 grid((unsigned)((P + 127) / 128), (unsigned)((c.cout + 15) / 16), (unsigned)G);
-  const size_t smem = (size_t)16 * 9 * c.cin * 4;
-  const TA* wbase = reinterpret_cast<const TA*>(Wop) + (int64_t)w_g0 * p->d_pad + c.w_off;
-  RN_LAUNCH((launch_pdl(conv_fwd_kernel<TA>, grid, 128, smem, s, reinterpret_cast<const TA*>(in),
-      wbase, (int64_t)w_gmul * p->d_pad, y, p->B, c.hin, c.win, c.cin, c.hout, c.wout, c.cout,
-      c.stride)));
+  ConvSimtArgs ca = simt_args(p, c, G);
+  ca.in = in;
+  ca.w = reinterpret_cast<const TA*>(Wop) + (int64_t)w_g0 * p->d_pad + c.w_off;
+  ca.w_gs = (int64_t)w_gmul * p->d_pad;
+  ca.out = y;
+  RN_CALL(launch_conv3x3_simt(ca, s));
   return LSGD_OK;
 }
 
@@ -1924,15 +1748,13 @@ lsgd_status conv_wgrad(ResNetPlan* p, int i, const void* in, float* Gr, cudaStre
         p->d_pad, 0, 0, s)));
     return LSGD_OK;
   }
-  const int nq = (int)((P + kWgradChunk - 1) / kWgradChunk);
+  const int nq = conv_wgrad_simt_ranges(K, p->B, c.hout, c.wout, c.cin, c.cout);
   const int J = 9 * c.cin;
-  const size_t smem = (size_t)(kWgradTile * 16 + kWgradTile * J) * 4;
-  RN_LAUNCH((launch_pdl(conv_wgrad_partial_kernel<TA>, dim3(nq, (c.cout + 15) / 16, K), 256, smem,
-      s, reinterpret_cast<const TA*>(p->dy), reinterpret_cast<const TA*>(in), p->part, p->B, c.hin,
-      c.win, c.cin, c.hout, c.wout, c.cout, c.stride, nq)));
-  const int64_t n = (int64_t)c.cout * J;
-  RN_LAUNCH((launch_pdl(sum_partials_kernel, grid_cap((int64_t)K * n, 256), 256, 0, s, p->part, nq,
-      n, K, Gr + c.w_off, p->d_pad)));
+  ConvSimtArgs ca = simt_args(p, c, K);
+  ca.in = in;
+  RN_CALL(launch_conv_wgrad_simt(ca, p->dy, p->part, s));
+  RN_LAUNCH((launch_pdl(sum_partials_crop_kernel, sum_partials_grid((int64_t)K * c.cout * J),
+      32 * kSumWarps, 0, s, p->part, nq, c.cout, J, J, K, Gr + c.w_off, p->d_pad, 0, 0)));
   return LSGD_OK;
 }
 
@@ -2087,12 +1909,15 @@ lsgd_status conv_dgrad(ResNetPlan* p, int i, const void* Wop, float* dx, const f
     }
     return LSGD_OK;
   }
-  dim3 grid((unsigned)((P + 63) / 64), (unsigned)((c.cin + 15) / 16), (unsigned)K);
-  const size_t smem = (size_t)c.cout * 9 * 16 * 4;
-  RN_LAUNCH((launch_pdl(conv_dgrad_kernel<TA>, grid, 64, smem, s,
-      reinterpret_cast<const TA*>(p->dy), reinterpret_cast<const TA*>(Wop) + c.w_off, p->d_pad, dx,
-      p->B, c.hin, c.win, c.cin, c.hout, c.wout, c.cout, c.stride, dout,
-      reinterpret_cast<const TA*>(out_act))));
+  ConvSimtArgs ca = simt_args(p, c, K);
+  ca.dgrad = true;
+  ca.in = p->dy;
+  ca.w = reinterpret_cast<const TA*>(Wop) + c.w_off;
+  ca.w_gs = p->d_pad;
+  ca.out = dx;
+  ca.sc_dout = dout;
+  ca.sc_act = out_act;
+  RN_CALL(launch_conv3x3_simt(ca, s));
   return LSGD_OK;
 }
 
@@ -2495,7 +2320,7 @@ lsgd_status resnet_alloc(ResNetPlan* p, const std::function<void*(size_t)>& allo
     p->rstd.push_back((float*)alloc((size_t)K * c.cout * 4));
     const int64_t P = (int64_t)B * c.hout * c.wout;
     const int64_t nq_s = (P + kRnChunk - 1) / kRnChunk;
-    const int64_t nq_w = (P + kWgradChunk - 1) / kWgradChunk;
+    const int64_t nq_w = conv_wgrad_simt_ranges(K, B, c.hout, c.wout, c.cin, c.cout);
     part = std::max(part, (size_t)(K * nq_s * c.cout * 2));
     part = std::max(part, (size_t)(K * nq_w * c.cout * 9 * c.cin));
     float* wp = nullptr;
