@@ -92,6 +92,26 @@ __device__ __forceinline__ float mean_of_pow2(float s, float c, float Kf, float 
   return __fadd_rn(q, __fmul_rn(r, invK));
 }
 
+// Two fp32 values in one 64-bit register pair and their packed arithmetic (each lane rounded as the
+// scalar instruction rounds it; one issue slot for two multiply-adds).
+using u64 = unsigned long long;
+__device__ __forceinline__ u64 pack2(float lo, float hi) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(u64 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ void fma2(u64& d, u64 a, u64 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void add2(u64& d, u64 a) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a));
+}
+
 // Programmatic dependent launch: kernels of the training step are launched so that the next one
 // may be scheduled while the previous one drains.  Each such kernel first waits for the previous
 // grid's completion and memory (griddepcontrol.wait) before touching global memory, and at once

@@ -12,25 +12,6 @@
 namespace lsgd {
 namespace {
 
-using u64 = unsigned long long;
-
-__device__ __forceinline__ u64 pack2(float lo, float hi) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(u64 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ void fma2(u64& d, u64 a, u64 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ void add2(u64& d, u64 a) {
-  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a));
-}
-
 // Four consecutive elements of an activation tensor as fp32.
 __device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ float4 load4(const uint16_t* p) {
