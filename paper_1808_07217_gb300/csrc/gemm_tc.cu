@@ -85,6 +85,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   return true;
 }
 
+// The TMA and MMA instructions take their operands from uniform registers.  Their issue loops are run
+// by a whole warp (the warp index broadcast, so that the compiler knows the control flow to be
+// uniform and keeps descriptors, addresses and counters in uniform registers) and one elected lane
+// issues.  A loop under "lane == 0" instead moves every operand across for every instruction: at
+// least 46 cycles per tcgen05.mma, and 90 to 150 with the descriptor arithmetic of these kernels,
+// where the tensor core takes 23 (M = 64, N = 16), 39 (M = 128, N = 16), 48 (N = 64) or 128 (N = 256).
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
+}
+
+// mbar_wait by every lane; true if all saw the phase (one that ran out cannot split the warp).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
+}
+
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
                                             int y, int z) {
   asm volatile(
@@ -1737,82 +1756,67 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
 
 
 // =============================================================================================
-// Weight gradient of a 3x3 convolution on the tensor cores, column matrix built in shared memory:
+// Weight gradient of a 3x3 convolution on the tensor cores, straight from the NHWC operands:
 //   dW[g][co][t][ci] = sum over output pixels p of dy[g][p][co] x[g][src_t(p)][ci].
-// As D[m][n] = sum_k A[m][k] B[n][k] with m = t Cin + ci (9 Cin rows in 128-row tiles), n = co
-// (one 64-wide operand, zero beyond Cout) and k = output pixels in blocks of 64: B is the output
-// gradient's 64 x 64 tile by TMA (pixel-major = MN-major, 128-byte swizzle); A is MN-major too,
-// gathered by the builder warps from a TMA-loaded strip of input rows (the halo rows above and
-// below come from out-of-bounds zero fill, the halo columns are written as zeros): one 16-byte
-// chunk = 8 channels of one tap and pixel per copy.  A CTA owns one replica and a contiguous range
-// of pixel blocks and keeps every m-tile's 128 x 64 fp32 accumulator in TMEM; it writes its
-// partial dW, and a second kernel sums the CTAs' partials in order.  Rows m >= 9 Cin of the last
-// m-tile are never written: they only reach accumulator rows that are not stored.
-// Two rings: the small TMA inputs (strip + tile) run `ni` blocks ahead, and `na` A tiles
-// (two to four) let the builders run ahead of the MMAs.
-//   warp 0      TMA producer (input strip + output-gradient tile per block)
-//   warp 1      MMA issuer: per block and m-tile, 4 x tcgen05.mma (M = 128, N = 64, K = 16)
+// As D[m][n] = sum_k A[m][k] B[n][k] with k = output pixels, n = co and, for each kernel column kw,
+// m = (kh, ci).  Both operands lie in shared memory as TMA writes them, one pixel's channels per
+// swizzled row (32, 64 or 128 bytes), i.e. pixel-major = MN-major.  A's three row groups (kh) are
+// the same strip of input rows read one image row further each: the descriptor's stride between
+// swizzle atoms along m is one strip row.  The kernel column shifts the strip by pixels: the
+// hardware swizzles address bits, so a descriptor may start at any pixel of the strip, and one
+// strip with its halo serves all nine taps -- no column matrix is ever built.  (A builder that gathered
+// it in shared memory, with single-lane issue loops, took 114 us for a first-stage layer of 16
+// workers x 128 images (134 MB, 9.7 GFLOP); the strips with such loops 111; with whole-warp loops
+// 42: 17 cycles over the tensor core's 23 per M = 64, N = 16 product.)
+//
+// Per tile of kp (128 or 64) output pixels -- whole rows of one image -- the strip holds the
+// (R - 1) S + 3 input rows under it, Wp pixels wide from column -1 on (zeros outside the image by
+// TMA's fill).  At stride 2 pixels of one parity are neighbours for the MMA, so two strips hold the
+// odd (kw = 0, 2) and the even (kw = 1) columns.  A CTA owns one replica and a contiguous range of
+// tiles and keeps the accumulators (per kw: 64 rows of 3 x 16, 128 of 3 x 32, or 128 + 64 of
+// 3 x 64 channels) in TMEM; it writes its partial dW, and a second kernel adds the CTAs' partials
+// in order.  Rows m beyond the third kernel row multiply whatever lies behind the strip and are
+// never read.
+//   warp 0      TMA producer (strip(s) + output-gradient tile per stage)
+//   warp 1      MMA issuer: per 16 pixels and kernel column one tcgen05.mma (two for 64 channels)
 //   warp 2      TMEM allocation
-//   warps 4-7   build A for each block; at the end, tcgen05.ld of the accumulators and the
-//               partial's stores
+//   warps 0-3   at the end, tcgen05.ld of the accumulators and the partial's stores
 namespace cw {
-constexpr int THREADS = 384;
-constexpr int MAX_NA = 4;   // A buffers
-constexpr int MAX_NI = 16;  // input stages
-constexpr int KB = 64;      // output pixels per block
-constexpr int BUILDERS = 8; // builder warps (warps 4-11)
-constexpr int MAX_CH = 18;  // 16-byte chunks per builder thread (9 taps x Cin / 8 / 4 parts)
-constexpr int MAX_MT = 5;   // m-tiles (9 Cin <= 640)
-constexpr uint32_t kTileA = 16384;  // one m-tile of A: two 64-row atoms x 64 pixels x 128 B
-constexpr uint32_t kTileB = 8192;   // the output-gradient tile: 64 pixels x 128 B
+constexpr int THREADS = 128;
+constexpr int MAX_ST = 8;            // stages
 constexpr uint32_t kTwoPerSm = 113 * 1024;  // shared memory that still fits two CTAs on an SM
 constexpr uint32_t kOnePerSm = 224 * 1024;
 }  // namespace cw
 
-__host__ __device__ inline int cw_rows(int stride, int wout) { return (cw::KB / wout - 1) * stride + 3; }
-__host__ __device__ inline uint32_t cw_halo_pitch(int cin, int stride, int win, int wout) {
-  return ((uint32_t)cw_rows(stride, wout) * win * cin * 2 + 1023u) & ~1023u;
-}
+namespace {
+__host__ __device__ inline uint32_t up1k(uint32_t v) { return (v + 1023u) & ~1023u; }
+}  // namespace
 
 __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
     const __grid_constant__ ConvWgradArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
-  const int cin = a.cin, cout = a.cout, mrows = 9 * cin, ni = a.ni, na = a.na;
-  const int mt_n = (mrows + 127) / 128;
-  const int rh = cw_rows(a.stride, a.wout);
-  const uint32_t halo_bytes = (uint32_t)rh * a.win * cin * 2;
-  const uint32_t in_pitch = cw_halo_pitch(cin, a.stride, a.win, a.wout) + cw::kTileB;
-  const uint32_t a_bytes = (uint32_t)mt_n * cw::kTileA;
-  uint8_t* A0 = base;                          // [na][mt_n][2][64][128 B]
-  uint8_t* I0 = A0 + na * a_bytes;             // [ni]: output-gradient tile, then the strip
-  uint64_t* full_in = reinterpret_cast<uint64_t*>(I0 + ni * in_pitch);
-  uint64_t* empty_in = full_in + cw::MAX_NI;   // arrivals: the MMAs (tile), each builder (strip)
-  uint64_t* aready = empty_in + cw::MAX_NI;
-  uint64_t* afree = aready + cw::MAX_NA;
-  uint64_t* acc_full = afree + cw::MAX_NA;
+  const ConvWgradGeom& gm = a.geom;
+  const int cin = a.cin, nst = gm.stages;
+  const uint32_t rowb = (uint32_t)cin * 2;               // bytes of one pixel
+  const uint32_t strip_bytes = (uint32_t)gm.rows * gm.wp * rowb, strip_pitch = up1k(strip_bytes);
+  const uint32_t tile_b = (uint32_t)gm.kp * a.nb * 2;
+  const uint32_t stage_pitch = gm.strips * strip_pitch + up1k(tile_b);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + nst * stage_pitch + gm.pad);
+  uint64_t* empty = full + cw::MAX_ST;
+  uint64_t* acc_full = empty + cw::MAX_ST;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int g = blockIdx.y, q = blockIdx.x, cpr = gridDim.x;
-  const int nkb = a.P / cw::KB;
-  const int kb0 = (int)((int64_t)q * nkb / cpr);
-  const int nblk = (int)((int64_t)(q + 1) * nkb / cpr) - kb0;
-  const int per_img = a.hout * a.wout;
-  const int nb = a.nb;                               // MMA N: output-gradient channels
-  const uint32_t tile_b = (uint32_t)cw::KB * nb * 2;  // bytes of the output-gradient tile
-  uint32_t tmem_cols = 32;
-  while (tmem_cols < (uint32_t)(mt_n * nb)) tmem_cols <<= 1;
+  const int ntiles = a.P / gm.kp, per_img = a.hout * a.wout;
+  const int t0 = (int)((int64_t)q * ntiles / cpr), nt = (int)((int64_t)(q + 1) * ntiles / cpr) - t0;
+  const int mt_n = cin == 64 ? 2 : 1;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < ni; ++i) {
-      mbar_init(&full_in[i], 1);
-      mbar_init(&empty_in[i], 1 + cw::BUILDERS);
-    }
-    for (int i = 0; i < na; ++i) {
-      mbar_init(&aready[i], cw::BUILDERS);
-      mbar_init(&afree[i], 1);
+    for (int i = 0; i < nst; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
     }
     mbar_init(acc_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1821,7 +1825,7 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
-                 "r"(tmem_cols)
+                 "r"(gm.tmem_cols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -1831,140 +1835,118 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
   const uint32_t tmem = *tmem_slot;
   pdl_begin();  // everything above touched only shared memory and TMEM
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- producer ----------------
-    int j = 0;
-    for (; j < nblk; ++j) {
-      const int s = j % ni;
-      if (!mbar_wait(&empty_in[s], ((j / ni) & 1) ^ 1)) break;
-      const int p0 = (kb0 + j) * cw::KB;
-      const int b = p0 / per_img, oy0 = (p0 % per_img) / a.wout;
-      uint8_t* st = I0 + s * in_pitch;
-      mbar_expect_tx(&full_in[s], halo_bytes + tile_b);
-      tma_load_3d(st, &a.dy_map, &full_in[s], 0, p0, g);
-      tma_load_5d(st + cw::kTileB, &a.x_map, &full_in[s], 0, 0, oy0 * a.stride - 1, b, g);
+    const bool el = elect_one();
+    int j = 0, s = 0;
+    uint32_t ph = 1;
+    int p0 = t0 * gm.kp, b = p0 / per_img, y = p0 % per_img / a.wout;  // the tile's image and row
+    const int R = gm.kp / a.wout;
+    for (; j < nt; ++j) {
+      if (!mbar_wait_warp(&empty[s], ph)) break;
+      uint8_t* st = base + s * stage_pitch;
+      if (el) {
+        mbar_expect_tx(&full[s], gm.strips * strip_bytes + tile_b);
+        tma_load_5d(st, &a.x_map, &full[s], 0, -1, y * a.stride - 1, b, g);
+        if (gm.strips == 2) tma_load_5d(st + strip_pitch, &a.x_map, &full[s], 0, 0, y * a.stride - 1, b, g);
+        tma_load_3d(st + gm.strips * strip_pitch, &a.dy_map, &full[s], 0, p0, g);
+      }
+      p0 += gm.kp;
+      y += R;
+      if (y == a.hout) {
+        y = 0;
+        ++b;
+      }
+      if (++s == nst) {
+        s = 0;
+        ph ^= 1;
+      }
     }
     // copies in flight land before the CTA can exit
-    for (int i = (j > ni ? j - ni : 0); i < j; ++i) mbar_wait(&full_in[i % ni], (i / ni) & 1);
-  } else if (warp == 1 && lane == 0) {
+    for (int i = (j > nst ? j - nst : 0); i < j; ++i) mbar_wait(&full[i % nst], (i / nst) & 1);
+  } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    const uint32_t idesc = make_idesc(BM, nb, true, true);
-    // descriptors of A0 and I0; a buffer / m-tile / K-step adds its byte offset / 16.  B: rows of
-    // 2 nb bytes (nb channels) swizzled at that width, 8-row groups 16 nb bytes apart, K-steps of
-    // 16 pixels 32 nb bytes apart; one swizzle atom spans all nb channels.
-    const uint64_t a_desc0 = smem_desc(smem_u32(A0), 8192, 1024);
-    const uint64_t b_desc0 = nb == 64 ? smem_desc(smem_u32(I0), 8192, 1024)
-                                      : smem_desc_swz(smem_u32(I0), 16u * nb, 16u * nb, 2u * nb);
+    const bool el = elect_one();
+    const int m0 = cin == 16 ? 64 : 128;
+    const uint32_t idesc0 = make_idesc(m0, a.nb, true, true), idesc1 = make_idesc(64, a.nb, true, true);
+    const uint32_t ux = rowb >> 4;  // one strip pixel in the descriptors' 16-byte units
+    // along k: eight pixels to the next core group (a whole output row where rows are 8 wide);
+    // along m: one strip row to the next kernel row
+    const uint32_t row_px = (uint32_t)gm.wp * a.stride;  // strip pixels from one output row to the next
+    const uint64_t a_desc0 =
+        smem_desc_swz(smem_u32(base), gm.wp * rowb, (a.wout == 8 ? row_px : 8u) * rowb, rowb);
+    const uint64_t b_desc0 = smem_desc_swz(smem_u32(base) + gm.strips * strip_pitch, 16u * a.nb,
+                                           16u * a.nb, 2u * a.nb);
+    // kernel column kw: which strip and how many pixels into it
+    const uint32_t col1 = a.stride == 1 ? ux : strip_pitch >> 4, col2 = a.stride == 1 ? 2 * ux : ux;
+    const uint32_t mt_off = 2u * gm.wp * ux;  // kernel row 2 of 64 channels
+    const uint32_t acc_kw = (uint32_t)(mt_n * a.nb);
+    const int lw = 31 - __clz(a.wout);
     bool ok = true;
-    for (int j = 0; j < nblk; ++j) {
-      const int s = j % ni, sa = j % na;
-      if (!mbar_wait(&aready[sa], (j / na) & 1) || !mbar_wait(&full_in[s], (j / ni) & 1)) {
+    int s = 0;
+    uint32_t ph = 0, acc = 0;
+    for (int j = 0; j < nt; ++j) {
+      if (!mbar_wait_warp(&full[s], ph)) {
         ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t ad = a_desc0 + ((uint32_t)sa * a_bytes >> 4);
-      const uint64_t bd = b_desc0 + ((uint32_t)s * in_pitch >> 4);
-      for (int mt = 0; mt < mt_n; ++mt)
+      const uint64_t ad0 = a_desc0 + ((uint32_t)s * stage_pitch >> 4);
+      const uint64_t bd0 = b_desc0 + ((uint32_t)s * stage_pitch >> 4);
 #pragma unroll
-        for (int kk = 0; kk < cw::KB / 16; ++kk)
-          mma_bf16(tmem + (uint32_t)(mt * nb), ad + (uint32_t)(mt * (cw::kTileA >> 4) + kk * 128),
-                   bd + (uint32_t)(kk * 2 * nb), idesc, (j > 0 || kk > 0) ? 1u : 0u);
-      mma_commit(&afree[sa]);    // A buffer reusable once these MMAs have read it
-      mma_commit(&empty_in[s]);  // and the output-gradient tile
-    }
-    if (ok && nblk > 0) mma_commit(acc_full);
-  } else if (warp >= 4) {
-    // ---------------- builders, then the epilogue ----------------
-    // Builder thread = (pixel k of the block, part p of 4): it copies chunks p, p + 4, ... of the
-    // pixel's 9 Cin / 8 sixteen-byte chunks (tap t, channels 8 cg..8 cg + 7).  Where each of them
-    // comes from in the strip and goes to in A is the same for every block, so the offsets are
-    // worked out once; per block a thread does at most MAX_CH loads and stores.  Each warp waits
-    // and signals by itself (aready and empty_in count the warps), with two warps per scheduler
-    // so that one's load latency hides behind the other's work.
-    const int bt = threadIdx.x - 128;
-    const int k = bt & (cw::KB - 1), part = bt >> 6;
-    const int cg_n = cin / 8, nchunk = 9 * cg_n;
-    const int r = k / a.wout, ox = k - r * a.wout;
-    const uint32_t swz_mask = cin == 64 ? 7u : (cin == 32 ? 3u : 1u);  // the strip's swizzle
-    uint32_t src_off[cw::MAX_CH], dst_off[cw::MAX_CH];
-    uint32_t inside = 0;
-    int nch = 0;
-#pragma unroll
-    for (int i = 0; i < cw::MAX_CH; ++i) {
-      const int c = part + 4 * i;
-      src_off[i] = dst_off[i] = 0;
-      if (c < nchunk) {
-        const int t = c / cg_n, cg = c - t * cg_n;
-        const int kh = t / 3, kw = t - 3 * kh;
-        const int ix = ox * a.stride + kw - 1;
-        if (ix >= 0 && ix < a.win) {
-          const uint32_t o = (uint32_t)(((r * a.stride + kh) * a.win + ix) * cin) * 2u + (uint32_t)cg * 16u;
-          src_off[i] = o ^ (((o >> 7) & swz_mask) << 4);
-          inside |= 1u << i;
+      for (int k = 0; k < 8; ++k) {
+        if (16 * k >= gm.kp) break;
+        // the 16 pixels from 16 k on: their output row and the column in it
+        const uint64_t ad = ad0 + (((16u * k) >> lw) * row_px + ((16u * k) & (a.wout - 1))) * ux;
+        const uint64_t bd = bd0 + (uint32_t)(2 * a.nb * k);
+        if (el) {
+          mma_bf16(tmem, ad, bd, idesc0, acc);
+          mma_bf16(tmem + acc_kw, ad + col1, bd, idesc0, acc);
+          mma_bf16(tmem + 2 * acc_kw, ad + col2, bd, idesc0, acc);
+          if (mt_n == 2) {
+            mma_bf16(tmem + a.nb, ad + mt_off, bd, idesc1, acc);
+            mma_bf16(tmem + acc_kw + a.nb, ad + col1 + mt_off, bd, idesc1, acc);
+            mma_bf16(tmem + 2 * acc_kw + a.nb, ad + col2 + mt_off, bd, idesc1, acc);
+          }
         }
-        const int m = t * cin + cg * 8;
-        dst_off[i] = (uint32_t)(m >> 7) * cw::kTileA + (uint32_t)((m >> 6) & 1) * 8192u +
-                     (uint32_t)(k >> 3) * 1024u + (uint32_t)(k & 7) * 128u +
-                     ((uint32_t)(((m >> 3) & 7) ^ (k & 7)) << 4);
-        nch = i + 1;
+        acc = 1;
+      }
+      if (el) mma_commit(&empty[s]);
+      if (++s == nst) {
+        s = 0;
+        ph ^= 1;
       }
     }
-    auto wwait = [&](uint64_t* bar, uint32_t parity) -> bool {
-      return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
-    };
-    bool ok = true;
-    for (int j = 0; j < nblk; ++j) {
-      const int s = j % ni, sa = j % na;
-      if (!wwait(&full_in[s], (j / ni) & 1) || !wwait(&afree[sa], ((j / na) & 1) ^ 1)) {
-        ok = false;
-        break;
-      }
-      const uint32_t X = smem_u32(I0 + s * in_pitch + cw::kTileB);
-      const uint32_t A = smem_u32(A0 + sa * a_bytes);
-#pragma unroll
-      for (int i = 0; i < cw::MAX_CH; ++i) {
-        if (i < nch) {
-          uint32_t v0 = 0u, v1 = 0u, v2 = 0u, v3 = 0u;
-          if (inside & (1u << i))
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3)
-                         : "r"(X + src_off[i])
-                         : "memory");
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(A + dst_off[i]), "r"(v0),
-                       "r"(v1), "r"(v2), "r"(v3)
-                       : "memory");
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the MMAs
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&aready[sa]);
-        mbar_arrive(&empty_in[s]);  // this warp has read the strip
-      }
-    }
-    if (warp >= 8) ok = false;  // the epilogue: warps 4-7, one TMEM lane quarter each
-    if (ok && nblk > 0 && wwait(acc_full, 0)) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int quarter = warp & 3;
-      float* out = a.part + ((int64_t)g * cpr + q) * cout * mrows;
+    if (ok && nt > 0 && el) mma_commit(acc_full);
+  }
+  __syncwarp();
+
+  // ---------------- epilogue ----------------
+  if (nt > 0 && __all_sync(0xffffffffu, mbar_wait(acc_full, 0) ? 1 : 0)) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    float* out = a.part + ((int64_t)g * cpr + q) * a.cout * 9 * cin;
+    for (int kw = 0; kw < 3; ++kw)
       for (int mt = 0; mt < mt_n; ++mt) {
-        const int m = mt * 128 + quarter * 32 + lane;
-        for (int c0 = 0; c0 < cout; c0 += 16) {
+        // TMEM lane -> row m: all 128 lanes of an M = 128 accumulator, the first 16 of each warp's
+        // 32 of an M = 64 one
+        const bool half = cin == 16 || mt == 1;
+        const int m = half ? warp * 16 + lane : warp * 32 + lane;
+        const int kh = 2 * mt + m / cin, ci = m % cin;
+        const bool row_ok = kh < 3 && (!half || lane < 16);
+        for (int c0 = 0; c0 < a.cout; c0 += 16) {
           float v[16];
-          tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(mt * nb + c0), v);
-          if (m < mrows) {
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((kw * mt_n + mt) * a.nb + c0), v);
+          if (row_ok) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) out[(int64_t)(c0 + i) * mrows + m] = v[i];
+            for (int i = 0; i < 16; ++i) out[((int64_t)(c0 + i) * 9 + kh * 3 + kw) * cin + ci] = v[i];
           }
         }
       }
-    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 2) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(gm.tmem_cols)
                  : "memory");
   }
 }
@@ -2299,65 +2281,62 @@ bool make_tma_map_conv(CUtensorMap* map, const void* base, int ck, int win, int 
 
 bool conv_wgrad_tc_ok(int cin, int cout, int stride, int hin, int win, int hout, int wout) {
   if ((cin != 16 && cin != 32 && cin != 64) || cout < 16 || cout > 64 || cout % 16) return false;
-  if ((stride != 1 && stride != 2) || wout < 1 || wout > cw::KB || cw::KB % wout) return false;
-  if ((hout * wout) % cw::KB || win != wout * stride || hin != hout * stride) return false;
-  return win <= 256 && cw_rows(stride, wout) <= 256;
+  if ((stride != 1 && stride != 2) || wout < 1 || wout > 64 || 64 % wout) return false;
+  return (hout * wout) % 64 == 0 && win == wout * stride && hin == hout * stride;
 }
 
-// Buffers and CTAs per SM of a shape.  Two A tiles; the input ring gets the rest of the shared
-// memory (deeper rings measured faster than more A tiles).  Two CTAs per SM whenever each still
-// gets three input stages: a CTA's blocks pass through a chain of handshakes one after another,
-// and a second CTA overlaps its chain with the first's.
-static void conv_wgrad_plan(int cin, int stride, int win, int wout, int* na, int* ni, int* per_sm,
-                            size_t* smem) {
-  const int mt_n = (9 * cin + 127) / 128;
-  const size_t bars = (2 * cw::MAX_NI + 2 * cw::MAX_NA + 1) * 8 + 16;
-  const size_t stage = cw_halo_pitch(cin, stride, win, wout) + cw::kTileB;
-  auto fixed = [&](int nA) { return 1024 + (size_t)nA * mt_n * cw::kTileA + bars; };
-  auto stages = [&](int nA, size_t budget) {
-    return budget > fixed(nA) ? (int)std::min<size_t>(cw::MAX_NI, (budget - fixed(nA)) / stage) : 0;
-  };
-  const int n2 = stages(2, cw::kTwoPerSm), n1 = stages(2, cw::kOnePerSm);
-  const int n2s = stages(1, cw::kTwoPerSm);  // one A tile: builders and MMAs take turns
-  *na = 2;
-  if (n2 >= 3 || (n2 >= 2 && 2 * n2 >= n1)) {
-    *ni = n2;
-    *per_sm = 2;
-  } else if (n2s >= 3) {
-    *na = 1;
-    *ni = n2s;
-    *per_sm = 2;
-  } else {
-    *ni = n1;
-    *per_sm = 1;
+// Outputs at least 8 wide: 16 pixels are then within a row, or two whole rows (narrower ones run
+// on the fp32 cores).
+bool conv_wgrad_geom(int cin, int cout, int stride, int hout, int wout, ConvWgradGeom* gm) {
+  if (wout < 8) return false;
+  const int nb = conv_wgrad_nb(cout);
+  gm->strips = stride;
+  gm->wp = stride == 1 ? wout + 2 : wout + 1;
+  uint32_t cols = 32;
+  while (cols < (uint32_t)(3 * (cin == 64 ? 2 : 1) * nb)) cols <<= 1;
+  gm->tmem_cols = cols;
+  // 128-pixel tiles where an image has them: fewer stage handshakes, less halo
+  for (int kp = (hout * wout) % 128 == 0 ? 128 : 64; kp >= 64; kp -= 64) {
+    gm->kp = kp;
+    gm->rows = (kp / wout - 1) * stride + 3;
+    // the unread rows of the last strip's operand end at most (fourth kernel row) one strip row
+    // behind the strip; the tile follows it, and this pad where the tile is smaller
+    gm->pad = (int)up1k((uint32_t)gm->wp * cin * 2);
+    const size_t stage = gm->strips * (size_t)up1k((uint32_t)(gm->rows * gm->wp * cin * 2)) +
+                         up1k((uint32_t)(kp * nb * 2));
+    const size_t fixed = 1024 + gm->pad + (2 * cw::MAX_ST + 1) * 8 + 16;
+    const size_t n2 = (cw::kTwoPerSm - fixed) / stage, n1 = (cw::kOnePerSm - fixed) / stage;
+    // two CTAs per SM where each still gets three stages: one's handshakes overlap the other's
+    gm->per_sm = n2 >= 3 && 2 * cols <= 512 ? 2 : 1;
+    gm->stages = (int)std::min<size_t>(cw::MAX_ST, gm->per_sm == 2 ? n2 : n1);
+    gm->smem = fixed + gm->stages * stage;
+    if (gm->stages >= 2 && gm->rows <= 256) return true;
   }
-  *smem = *ni >= 2 ? fixed(*na) + (size_t)*ni * stage : 0;
+  return false;
 }
 
-int conv_wgrad_ctas(int cin, int stride, int wout, int G, int64_t P) {
-  int na = 0, ni = 0, per_sm = 1;
-  size_t smem = 0;
-  conv_wgrad_plan(cin, stride, wout * stride, wout, &na, &ni, &per_sm, &smem);
-  const int64_t blocks = P / cw::KB;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)kNumSMs * per_sm / std::max(G, 1)));
+int conv_wgrad_ctas(int cin, int cout, int stride, int hout, int wout, int B, int G) {
+  ConvWgradGeom gm;
+  if (!conv_wgrad_geom(cin, cout, stride, hout, wout, &gm))
+    return conv_wgrad_simt_ranges(G, B, hout, wout, cin, cout);
+  const int64_t tiles = (int64_t)B * hout * wout / gm.kp;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)kNumSMs * gm.per_sm / std::max(G, 1)));
 }
 
-bool make_tma_map_halo(CUtensorMap* map, const void* base, int cin, int win, int hin, int B, int G,
-                       int stride, int wout) {
+bool make_tma_map_strip(CUtensorMap* map, const void* base, int cin, int win, int hin, int B, int G,
+                        int stride, const ConvWgradGeom& gm) {
   std::call_once(g_encode_once, load_encode);
   if (!g_encode || (cin != 16 && cin != 32 && cin != 64) || (reinterpret_cast<uintptr_t>(base) & 15))
     return false;
-  const int rh = cw_rows(stride, wout);
-  if (win > 256 || rh > 256) return false;
+  const int span = (gm.wp - 1) * stride + 1;  // columns a strip row spans
+  if (span > 256 || gm.rows > 256) return false;
   const uint64_t e = 2;
   cuuint64_t dims[5] = {(cuuint64_t)cin, (cuuint64_t)win, (cuuint64_t)hin, (cuuint64_t)B,
                         (cuuint64_t)G};
   cuuint64_t strides[4] = {(cuuint64_t)cin * e, (cuuint64_t)win * cin * e,
                            (cuuint64_t)hin * win * cin * e, (cuuint64_t)B * hin * win * cin * e};
-  cuuint32_t box[5] = {(cuuint32_t)cin, (cuuint32_t)win, (cuuint32_t)rh, 1, 1};
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  // each pixel's channels are one 32 / 64 / 128-byte row, swizzled at that width so that the
-  // builders' reads of neighbouring pixels spread over the banks
+  cuuint32_t box[5] = {(cuuint32_t)cin, (cuuint32_t)span, (cuuint32_t)gm.rows, 1, 1};
+  cuuint32_t estr[5] = {1, (cuuint32_t)stride, 1, 1, 1};
   const CUtensorMapSwizzle sw = cin == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
                                           : (cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                        : CU_TENSOR_MAP_SWIZZLE_32B);
@@ -2369,19 +2348,13 @@ bool make_tma_map_halo(CUtensorMap* map, const void* base, int cin, int win, int
 
 cudaError_t launch_conv_wgrad_tc(const ConvWgradArgs& a, cudaStream_t stream) {
   if (a.P <= 0 || a.G <= 0) return cudaSuccess;
+  ConvWgradGeom gm;
   if (!conv_wgrad_tc_ok(a.cin, a.cout, a.stride, a.hin, a.win, a.hout, a.wout) || !a.part ||
-      a.P % cw::KB || a.P % (a.hout * a.wout) || a.cpr < 1 || a.cpr > a.P / cw::KB ||
-      a.G > 65535 || (9 * a.cin + 127) / 128 > cw::MAX_MT)
-    return cudaErrorInvalidValue;
-  int na = 0, ni = 0, per_sm = 1;
-  size_t smem = 0;
-  conv_wgrad_plan(a.cin, a.stride, a.win, a.wout, &na, &ni, &per_sm, &smem);
-  if (ni < 2 || ni > cw::MAX_NI || na < 1 || na > cw::MAX_NA || smem > 232448 ||
-      (a.nb != 16 && a.nb != 32 && a.nb != 64) || a.nb < a.cout)
+      !conv_wgrad_geom(a.cin, a.cout, a.stride, a.hout, a.wout, &gm) || a.nb != conv_wgrad_nb(a.cout) ||
+      a.P % gm.kp || a.P % (a.hout * a.wout) || a.cpr < 1 || a.cpr > a.P / gm.kp || a.G > 65535)
     return cudaErrorInvalidValue;
   ConvWgradArgs la = a;
-  la.ni = ni;
-  la.na = na;
+  la.geom = gm;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -2392,8 +2365,7 @@ cudaError_t launch_conv_wgrad_tc(const ConvWgradArgs& a, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_dev = dev;
   }
-  launch_pdl(conv_wgrad_tc_kernel, dim3(a.cpr, a.G), dim3(cw::THREADS), smem, stream, la);
-  return cudaGetLastError();
+  return launch_pdl(conv_wgrad_tc_kernel, dim3(a.cpr, a.G), dim3(cw::THREADS), gm.smem, stream, la);
 }
 
 int tc_tile_n(int Kd) { return (Kd + BK - 1) / BK <= 2 ? 128 : 64; }

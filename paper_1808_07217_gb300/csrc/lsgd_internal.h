@@ -220,27 +220,39 @@ bool conv_strip_ok(int hout, int wout, int stride);
 cudaError_t launch_conv_tc(const ConvArgs& a, cudaStream_t stream, int* ctas_per_replica = nullptr);
 // The CTAs per replica launch_conv_tc will use for these arguments (0 if it would reject them).
 int conv_tc_ctas(const ConvArgs& a);
-// Weight gradient of a 3x3 convolution (zero padding 1, stride 1 or 2) on the tensor cores, the
-// column matrix built in shared memory: part[g][q][co][t Cin + ci] = the sum over CTA q's 64-pixel
-// output blocks of dy[g][p][co] x[g][src_t(p)][ci], src_t(p) the input pixel under tap t of output
-// pixel p (zero outside the image).  x_map: make_tma_map_halo over the NHWC input; dy_map: rank-3
-// bf16 map over [G][P][Cout] with box {64, 64} and a 128-byte swizzle.  Cin 16 / 32 / 64, Cout a
-// multiple of 16 up to 64, Wout dividing 64, Hout Wout a multiple of 64.  dy_map's box is
-// {nb, 64} with a 2 nb-byte swizzle.
+// Weight gradient of a 3x3 convolution (zero padding 1, stride 1 or 2) on the tensor cores:
+// part[g][q][co][t Cin + ci] = the sum over CTA q's output pixels of dy[g][p][co] x[g][src_t(p)][ci],
+// src_t(p) the input pixel under tap t of output pixel p (zero outside the image).  x_map:
+// make_tma_map_strip over the NHWC input; dy_map: rank-3 bf16 map over [G][P][Cout] with box
+// {nb, kp} and a 2 nb-byte swizzle.  Cin 16 / 32 / 64, Cout a multiple of 16 up to 64, Wout dividing
+// 64, Hout Wout a multiple of 64.
+struct ConvWgradGeom {
+  int kp;       // output pixels per tile: whole rows of one image
+  int rows, wp; // the input strip's rows and its width in pixels
+  int strips;   // 1, or 2 at stride 2 (odd and even columns)
+  int stages, per_sm, pad;
+  uint32_t tmem_cols;
+  size_t smem;
+};
+// Channels of the output-gradient tile (48 padded to 64 by the map's zero fill).
+inline int conv_wgrad_nb(int cout) { return cout == 16 || cout == 32 ? cout : 64; }
 struct ConvWgradArgs {
   CUtensorMap x_map, dy_map;
   int cin, cout, stride, hin, win, hout, wout, G, P;
   int cpr;      // CTAs (partials) per replica, from conv_wgrad_ctas
   float* part;  // [G][cpr][cout][9 cin]
-  int ni, na;   // input stages and A buffers (set by the launcher)
-  int nb;       // the MMAs' N and the output-gradient tile's channels (16, 32 or 64; dy_map's box)
+  int nb;       // the MMAs' N and the output-gradient tile's channels (conv_wgrad_nb; dy_map's box)
+  ConvWgradGeom geom;  // set by the launcher
 };
 bool conv_wgrad_tc_ok(int cin, int cout, int stride, int hin, int win, int hout, int wout);
-int conv_wgrad_ctas(int cin, int stride, int wout, int G, int64_t P);
-// The input strip of one 64-pixel output block: rank-5 map {Cin, Win, Hin, B, G} with box
-// {Cin, Win, rows, 1, 1}, rows = (64 / Wout - 1) stride + 3, swizzled at the 2 Cin-byte row.
-bool make_tma_map_halo(CUtensorMap* map, const void* base, int cin, int win, int hin, int B, int G,
-                       int stride, int wout);
+// The kernel's launch shape; false: the shape (accepted by conv_wgrad_tc_ok) runs on the fp32 cores.
+bool conv_wgrad_geom(int cin, int cout, int stride, int hout, int wout, ConvWgradGeom* gm);
+// Partials per replica of either.
+int conv_wgrad_ctas(int cin, int cout, int stride, int hout, int wout, int B, int G);
+// One tile's input strip: rank-5 map {Cin, Win, Hin, B, G}, every `stride`-th column, all rows,
+// swizzled at the 2 Cin-byte pixel.
+bool make_tma_map_strip(CUtensorMap* map, const void* base, int cin, int win, int hin, int B, int G,
+                        int stride, const ConvWgradGeom& gm);
 cudaError_t launch_conv_wgrad_tc(const ConvWgradArgs& a, cudaStream_t stream);
 // The tile geometry of an implicit convolution with an Hout x Wout output: whole output rows,
 // 128 pixels per tile.  False when the shape does not tile that way.

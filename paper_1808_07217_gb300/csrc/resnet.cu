@@ -1129,34 +1129,46 @@ cudaError_t launch_conv_wgrad_impl(const uint16_t* x, const uint16_t* dy, float*
   if (!conv_wgrad_tc_ok(cin, cout, stride, hin, win, hout, wout) || G < 1 || B < 1 ||
       P > 0x7fffffffLL || cin_out > cin)
     return cudaErrorInvalidValue;
-  ConvWgradArgs a{};
-  // the output-gradient tile: 64 pixels x nb channels (Cout of 16 / 32 / 64 exactly; 48 padded
-  // to 64 by the map's zero fill), swizzled at its 2 nb-byte row
-  const int nb = (cout == 16 || cout == 32) ? cout : 64;
-  if (!make_tma_map_halo(&a.x_map, x, cin, win, hin, B, G, stride, wout) ||
-      !make_tma_map(&a.dy_map, dy, true, cout, P, G, cout, (uint64_t)P * cout, nb, 64, 2 * nb))
-    return cudaErrorInvalidValue;
-  a.nb = nb;
-  a.cin = cin;
-  a.cout = cout;
-  a.stride = stride;
-  a.hin = hin;
-  a.win = win;
-  a.hout = hout;
-  a.wout = wout;
-  a.G = G;
-  a.P = (int)P;
-  a.cpr = conv_wgrad_ctas(cin, stride, wout, G, P);
-  a.part = part;
-  cudaError_t e = launch_conv_wgrad_tc(a, s);
+  const int cpr = conv_wgrad_ctas(cin, cout, stride, hout, wout, B, G);
+  ConvWgradGeom gm;
+  cudaError_t e;
+  if (conv_wgrad_geom(cin, cout, stride, hout, wout, &gm)) {
+    ConvWgradArgs a{};
+    a.nb = conv_wgrad_nb(cout);
+    if (!make_tma_map_strip(&a.x_map, x, cin, win, hin, B, G, stride, gm) ||
+        !make_tma_map(&a.dy_map, dy, true, cout, P, G, cout, (uint64_t)P * cout, a.nb, gm.kp, 2 * a.nb))
+      return cudaErrorInvalidValue;
+    a.cin = cin;
+    a.cout = cout;
+    a.stride = stride;
+    a.hin = hin;
+    a.win = win;
+    a.hout = hout;
+    a.wout = wout;
+    a.G = G;
+    a.P = (int)P;
+    a.cpr = cpr;
+    a.part = part;
+    e = launch_conv_wgrad_tc(a, s);
+  } else {
+    ConvSimtArgs a{};
+    a.bf16 = true;
+    a.G = G;
+    a.B = B;
+    a.hin = hin, a.win = win, a.cin = cin;
+    a.hout = hout, a.wout = wout, a.cout = cout;
+    a.stride = stride;
+    a.in = x;
+    e = launch_conv_wgrad_simt(a, dy, part, s);
+  }
   if (e != cudaSuccess) return e;
   // the partials' sum, cropped to the first cin_out channels of every tap
   if (defer && deferred && sum_partials_v4_ok(part, 9 * cin, 9 * cin_out, dW, dW_gs, cin, cin_out)) {
-    *defer = SumJob{part, dW, dW_gs, 0, a.cpr, cout, 9 * cin, 9 * cin_out, G, cin, cin_out, 0};
+    *defer = SumJob{part, dW, dW_gs, 0, cpr, cout, 9 * cin, 9 * cin_out, G, cin, cin_out, 0};
     *deferred = true;
     return cudaGetLastError();
   }
-  launch_sum_partials(part, a.cpr, cout, 9 * cin, 9 * cin_out, G, dW, dW_gs, cin, cin_out, s);
+  launch_sum_partials(part, cpr, cout, 9 * cin, 9 * cin_out, G, dW, dW_gs, cin, cin_out, s);
   return cudaGetLastError();
 }
 
@@ -2148,8 +2160,7 @@ lsgd_status conv3x3_bn_bf16(const uint16_t* in, const uint16_t* w, float* y, flo
 }
 
 size_t conv_wgrad_scratch_floats(int G, int B, int hout, int wout, int cin, int cout, int stride) {
-  const int64_t P = (int64_t)B * hout * wout;
-  return (size_t)G * conv_wgrad_ctas(cin, stride, wout, G, P) * cout * 9 * cin;
+  return (size_t)G * conv_wgrad_ctas(cin, cout, stride, hout, wout, B, G) * cout * 9 * cin;
 }
 
 cudaError_t launch_conv_wgrad_bf16(const uint16_t* x, const uint16_t* dy, float* dW, int64_t dW_gs,
@@ -2309,8 +2320,7 @@ lsgd_status resnet_alloc(ResNetPlan* p, const std::function<void*(size_t)>& allo
     p->x16 = (uint16_t*)alloc((size_t)K * B * c0.hin * c0.win * 16 * 2);
     p->wstem = (uint16_t*)alloc((size_t)K * c0.cout * 9 * 16 * 2);
     if (!p->x16 || !p->wstem) return LSGD_ENOMEM;
-    const int64_t P0 = (int64_t)B * c0.hout * c0.wout;
-    part = std::max(part, (size_t)K * conv_wgrad_ctas(16, 1, c0.wout, K, P0) * c0.cout * 9 * 16);
+    part = std::max(part, (size_t)K * conv_wgrad_ctas(16, c0.cout, 1, c0.hout, c0.wout, B, K) * c0.cout * 9 * 16);
   }
   for (const ConvL& c : p->convs) {
     const int64_t n = (int64_t)K * B * c.hout * c.wout * c.cout;
@@ -2327,7 +2337,7 @@ lsgd_status resnet_alloc(ResNetPlan* p, const std::function<void*(size_t)>& allo
     if (conv_on_tc(p, c)) {
       const int Kc = col_ld(c);
       if (wgrad_tc(p, c)) {
-        const int cpr = conv_wgrad_ctas(c.cin, c.stride, c.wout, K, P);
+        const int cpr = conv_wgrad_ctas(c.cin, c.cout, c.stride, c.hout, c.wout, B, K);
         part = std::max(part, (size_t)K * cpr * c.cout * 9 * c.cin);
         if (!(&c == &p->convs[0] && p->stem16)) {
           wp = (float*)alloc((size_t)K * cpr * c.cout * 9 * c.cin * 4);

@@ -1,4 +1,4 @@
-"""The convolution weight-gradient kernel (column matrix built in shared memory, tcgen05) against
+"""The convolution weight-gradient kernel (tcgen05, taps as shifted views of one input strip) against
 an fp64 evaluation of its definition on the same bf16 operands:
     dW[g][co][kh][kw][ci] = sum over b, oy, ox of dy[g][b][oy][ox][co] x[g][b][s oy + kh - 1][s ox + kw - 1][ci]
 (3x3 kernel, zero padding 1, stride s).  Every ResNet-20 shape (16 / 32 / 64 channels, both
@@ -95,3 +95,11 @@ def test_conv_wgrad_rejects_unsupported_shapes(P):
         kw.update(bad)
         with pytest.raises(P.LsgdError):
             P.lsgd_conv_wgrad_bf16(x, dy, dW, **kw)
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 2, 64, 16, 16, 1), (1, 2, 4, 64, 64, 64, 2),   # widest rows
+                                   (2, 3, 2, 32, 32, 16, 1), (1, 5, 4, 16, 64, 32, 2),   # 64-pixel tiles
+                                   (3, 2, 16, 8, 16, 48, 1), (1, 9, 16, 8, 32, 64, 2),   # two rows per step
+                                   (2, 3, 16, 4, 16, 32, 1), (1, 2, 32, 2, 32, 16, 2)])  # narrower than 8
+def test_conv_wgrad_tile_edges(P, shape):
+    test_conv_wgrad_matches_fp64(P, shape)
