@@ -195,6 +195,34 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15},"
+      " [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+
+// Three groups of 16 columns, all loads in flight before the one wait (which the registers pass
+// through, so that no use of them moves above it).
+__device__ __forceinline__ void tmem_ld16x3(uint32_t t0, uint32_t t1, uint32_t t2, float (&v0)[16],
+                                            float (&v1)[16], float (&v2)[16]) {
+  uint32_t r0[16], r1[16], r2[16];
+  tmem_ld16_nowait(t0, r0);
+  tmem_ld16_nowait(t1, r1);
+  tmem_ld16_nowait(t2, r2);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    asm volatile("" : "+r"(r0[i]), "+r"(r1[i]), "+r"(r2[i]));
+    v0[i] = __uint_as_float(r0[i]);
+    v1[i] = __uint_as_float(r1[i]);
+    v2[i] = __uint_as_float(r2[i]);
+  }
+}
+
 // Sums 16 values per lane over the 32 lanes of a warp in four halving exchanges and one final
 // exchange: afterwards lane l holds the warp's sum of value l / 2 (lanes 2 j and 2 j + 1 agree).
 __device__ __forceinline__ float warp_colsum16(float (&v)[16], int lane) {
@@ -1395,10 +1423,10 @@ __global__ void __launch_bounds__(wu::THREADS, 1) wgrad_update_kernel(
 //   per kernel row: three stages per tile, stage kh holds the three kw-shifted boxes of the
 //     tile's rows under kernel row kh (stride 2, and tiles that span several images).
 //   warp 0      TMA producer (weights once, then one stage per tap)
-//   warp 1      MMA issuer: per tap ck / 16 tcgen05.mma (M = 128, N = NP, K = 16), descriptors
-//               from precomputed bases (the issuing thread is on the critical path); with
-//               nsplit = 3 the taps of column kw accumulate into partial kw, consecutive MMAs
-//               into different partials (small-N MMAs into one accumulator wait on each other)
+//   warp 1      MMA issuer (the whole warp, one lane issuing: 72 -> 65 us for a first-stage forward
+//               of 16 workers x 128 images): per tap ck / 16 tcgen05.mma (M = 128, N = NP, K = 16),
+//               descriptors from precomputed bases; with nsplit = 3 the taps of column kw
+//               accumulate into partial kw
 //   warp 2      TMEM allocation
 //   warps 4-7   epilogue: tcgen05.ld of the tile row's NP columns (the partials' sum), fp32
 //               stores
@@ -1442,7 +1470,7 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
   float* bw_mu = reinterpret_cast<float*>(tmem_slot + 4);  // [64]
   float* bw_rs = bw_mu + 64;                                // [64]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int g = blockIdx.y, cpr = gridDim.x;
   const int tiles = a.P / BM;  // per replica
   const int per_img = a.hout * a.wout;
@@ -1476,34 +1504,52 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
   const uint32_t tmem = *tmem_slot;
   pdl_begin();  // everything above touched only shared memory and TMEM
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- producer ----------------
-    mbar_expect_tx(w_full, 9 * wtap);
-    for (int t = 0; t < 9; ++t) tma_load_3d(wsm + t * wtap, &a.w_map, w_full, t * ck, 0, g);
-    int q = 0;
+    const bool el = elect_one();
+    if (el) {
+      mbar_expect_tx(w_full, 9 * wtap);
+      for (int t = 0; t < 9; ++t) tma_load_3d(wsm + t * wtap, &a.w_map, w_full, t * ck, 0, g);
+    }
+    // a tile's first image and row; the next one is cpr tiles on
+    const int rows_img = a.hout, row_step = cpr * (BM / a.wout);
+    int b0 = (int)blockIdx.x * BM / per_img, y = (int)blockIdx.x * BM % per_img / a.wout;
+    int q = 0, sl = 0;
+    uint32_t ph = 1;
     bool ok = true;
     for (int tile = blockIdx.x; tile < tiles && ok; tile += cpr) {
-      const int p0 = tile * BM, b0 = p0 / per_img, oy0 = (p0 / a.wout) % a.hout;
       for (int sp = 0; sp < spt; ++sp, ++q) {
-        const int sl = q % nst;
-        if (!mbar_wait(&empty[sl], ((q / nst) & 1) ^ 1)) {
+        if (!mbar_wait_warp(&empty[sl], ph)) {
           ok = false;
           break;
         }
-        mbar_expect_tx(&full[sl], stage_bytes);
-        // strip: rows oy0 - 1 .. oy0 + rows (the halo rows out of the image read as zeros);
+        // strip: rows y - 1 .. y + rows (the halo rows out of the image read as zeros);
         // per kernel row sp: the rows under kernel row sp
-        const int y0 = a.strip ? oy0 - 1 : oy0 * a.stride + sp - 1;
-        for (int kw = 0; kw < 3; ++kw)
-          tma_load_5d(ring + sl * stage_bytes + kw * box_bytes, &a.in_map, &full[sl], 0, kw - 1,
-                      y0, b0, g);
+        const int y0 = a.strip ? y - 1 : y * a.stride + sp - 1;
+        if (el) {
+          mbar_expect_tx(&full[sl], stage_bytes);
+          uint8_t* st = ring + sl * stage_bytes;
+          tma_load_5d(st, &a.in_map, &full[sl], 0, -1, y0, b0, g);
+          tma_load_5d(st + box_bytes, &a.in_map, &full[sl], 0, 0, y0, b0, g);
+          tma_load_5d(st + 2 * box_bytes, &a.in_map, &full[sl], 0, 1, y0, b0, g);
+        }
+        if (++sl == nst) {
+          sl = 0;
+          ph ^= 1;
+        }
+      }
+      y += row_step;
+      while (y >= rows_img) {
+        y -= rows_img;
+        ++b0;
       }
     }
     // copies in flight land before the CTA can exit
     mbar_wait(w_full, 0);
     for (int j = (q > nst ? q - nst : 0); j < q; ++j) mbar_wait(&full[j % nst], (j / nst) & 1);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
+    const bool el = elect_one();
     const uint32_t idesc = make_idesc(BM, np, false, false);
     const uint32_t swz = (uint32_t)ck * 2;
     // descriptors of the ring's start and of tap 0's weights: the address field is in 16-byte
@@ -1512,43 +1558,56 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
     const uint64_t b_desc0 = smem_desc_kmajor(smem_u32(wsm), swz);
     const uint32_t kw_step = box_bytes >> 4, kh_step = (a.strip ? row_bytes : 0u) >> 4;
     const uint32_t tap_step = wtap >> 4;
-    bool ok = mbar_wait(w_full, 0);
+    const bool split3 = nsplit == 3;
+    const uint32_t acc_kw = split3 ? (uint32_t)np : 0u;
+    bool ok = mbar_wait_warp(w_full, 0);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    int q = 0, i = 0;
-    for (int tile = blockIdx.x; tile < tiles && ok; tile += cpr, ++i) {
-      const int ab = i % nacc;
-      if (!mbar_wait(&acc_empty[ab], ((i / nacc) & 1) ^ 1)) break;
+    int sl = 0, ab = 0;
+    uint32_t ph = 0, ph_acc = 1;
+    for (int tile = blockIdx.x; tile < tiles && ok; tile += cpr) {
+      if (!mbar_wait_warp(&acc_empty[ab], ph_acc)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t acc = tmem + (uint32_t)ab * acc_cols;
-      for (int sp = 0; sp < spt; ++sp, ++q) {
-        const int sl = q % nst;
-        if (!mbar_wait(&full[sl], (q / nst) & 1)) {
+      for (int sp = 0; sp < spt; ++sp) {
+        if (!mbar_wait_warp(&full[sl], ph)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t st_desc = a_desc0 + ((uint32_t)sl * stage_bytes >> 4);
-        for (int kh = a.strip ? 0 : sp; kh < (a.strip ? 3 : sp + 1); ++kh) {
+#pragma unroll
+        for (int kh = 0; kh < 3; ++kh) {
+          if (!a.strip && kh != sp) continue;
           const uint64_t row_desc = st_desc + (uint32_t)kh * kh_step;
-          for (int kk = 0; kk < ck / 16; ++kk) {
+          const uint64_t tap_desc = b_desc0 + (uint32_t)(3 * kh) * tap_step;
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            if (16 * kk >= ck) break;
 #pragma unroll
             for (int kw = 0; kw < 3; ++kw) {
-              const int t = kh * 3 + kw;
               // partial kw (nsplit = 3) starts at its first kernel row; a single accumulator at
               // the first tap
-              const bool first = kk == 0 && (nsplit == 3 ? kh == 0 : t == 0);
-              mma_bf16(acc + (nsplit == 3 ? (uint32_t)(kw * np) : 0u),
-                       row_desc + (uint32_t)kw * kw_step + (uint32_t)(2 * kk),
-                       b_desc0 + (uint32_t)t * tap_step + (uint32_t)(2 * kk), idesc,
-                       first ? 0u : 1u);
+              const bool first = kk == 0 && kh == 0 && (kw == 0 || split3);
+              if (el)
+                mma_bf16(acc + kw * acc_kw, row_desc + (uint32_t)kw * kw_step + (uint32_t)(2 * kk),
+                         tap_desc + (uint32_t)kw * tap_step + (uint32_t)(2 * kk), idesc,
+                         first ? 0u : 1u);
             }
           }
         }
         // strip form: the epilogue releases the stage once it sees the tile's accumulator (one
         // commit per tile); per kernel row: the stage is released as soon as its MMAs complete
-        if (!a.strip) mma_commit(&empty[sl]);
+        if (!a.strip && el) mma_commit(&empty[sl]);
+        if (++sl == nst) {
+          sl = 0;
+          ph ^= 1;
+        }
       }
-      if (ok) mma_commit(&acc_full[ab]);
+      if (ok && el) mma_commit(&acc_full[ab]);
+      if (++ab == nacc) {
+        ab = 0;
+        ph_acc ^= 1;
+      }
     }
   } else if (warp >= 4) {
     // ---------------- epilogue ----------------
@@ -1556,10 +1615,6 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
     // itself (every lane polls; the warp goes on only if all lanes saw the phase, so a wait that
     // runs out never splits a warp-wide tensor-memory load) and gives it back with one arrival.
     const int quarter = warp & 3, r = quarter * 32 + lane;
-    auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-      const bool okl = mbar_wait(bar, parity);
-      return __all_sync(0xffffffffu, okl);
-    };
     // per-channel BatchNorm statistics of the output pixels (forward convolutions), per
     // epilogue warp: lanes 2 j, 2 j + 1 keep channel 16 ci + j's running count, mean and M2 over
     // the warp's 32 rows of every tile
@@ -1579,13 +1634,14 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
     }
-    int i = 0;
-    for (int tile = blockIdx.x; tile < tiles; tile += cpr, ++i) {
-      const int ab = i % nacc;
-      if (!warp_wait(&acc_full[ab], (i / nacc) & 1)) break;
+    int ab = 0, sl = 0;  // the tile's accumulator and (strip form) input stage
+    uint32_t ph = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += cpr) {
+      if (!mbar_wait_warp(&acc_full[ab], ph)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       // strip form: this tile's MMAs (and so its reads of its input stage) are complete
-      if (a.strip && quarter == 0 && lane == 0) mbar_arrive(&empty[i % nst]);
+      if (a.strip && quarter == 0 && lane == 0) mbar_arrive(&empty[sl]);
+      if (++sl == nst) sl = 0;
       int64_t dst = (int64_t)tile * BM + r;
       if (a.dst_h > 0) {
         const int pp = tile * BM + r, img = pp / per_img, rem = pp - img * per_img;
@@ -1634,16 +1690,14 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
         if (c0 >= a.N) break;
         float v[16];
         const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)ab * acc_cols + c0;
-        tmem_ld16(tl, v);
         if (nsplit == 3) {
           // the three column partials, added in column order
+          float u1[16], u2[16];
+          tmem_ld16x3(tl, tl + (uint32_t)np, tl + (uint32_t)(2 * np), v, u1, u2);
 #pragma unroll
-          for (int kw = 1; kw < 3; ++kw) {
-            float u[16];
-            tmem_ld16(tl + (uint32_t)(kw * np), u);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] += u[j];
-          }
+          for (int j = 0; j < 16; ++j) v[j] = (v[j] + u1[j]) + u2[j];
+        } else {
+          tmem_ld16(tl, v);
         }
         if (with_bwd) {
           // dx (+ the shortcut's share) masked by the layer below's ReLU, and that layer's
@@ -1727,6 +1781,10 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      if (++ab == nacc) {
+        ab = 0;
+        ph ^= 1;
+      }
     }
     if (with_bwd && !(lane & 1)) {
 #pragma unroll
