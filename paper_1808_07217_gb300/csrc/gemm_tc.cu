@@ -1814,6 +1814,490 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
 
 
 // =============================================================================================
+// The 3x3 convolutions of images whose rows are 512 channel values (32 x 16, 16 x 32 or 8 x 64
+// channels: every ResNet-20 stage), persistent, 64 / ck neighbouring pixels as one 64-channel
+// "super-pixel": an image row is then eight 128-byte rows -- one row group of a K-major operand --
+// and the next image row the next group.  A tile is TR = 16 or 8 image rows (M = 128 or 64 rows of
+// super-pixels) and its whole input, halo included, is ONE box of (TR - 1) S + 3 rows of ten
+// super-pixels: tap rows are a row further, and the 16-channel slices from the pixel left of the
+// super-pixel to the one right of it follow one another in memory, so a product's operand is the
+// box read from a shifted start (the hardware swizzles address bits).  The weights are laid out per
+// slice as [output pixel, output channel][16] with zeros where the slice is not under the tap (a
+// block Toeplitz matrix), by every CTA from the packed weights.
+// What it buys at 16 channels over one pixel per row (conv_tc_kernel): a product has N = 64 columns
+// (48 cycles) for four pixels instead of N = 16 (39) for one; the box has 180 128-byte rows per 512
+// pixels instead of 2,304 32-byte ones, whose TMA rate bound that kernel; a thread owns four
+// pixels (256 contiguous bytes), so the statistics' warp sums run once per four.
+// A stride-2 data gradient's four parity phases are one such product: output row parity = 64-column
+// segment, column parity = alternate pixels, taps of kernel rows 1 and 2 of the phase weights.
+//   warp 0      TMA producer           warp 1      MMA issuer
+//   warp 2      TMEM allocation        warps 1-7   weight layout at the start
+//   warps 4-7   epilogue
+// The epilogue reads TMEM in the 16 x 256-bit shape, which gives a row to four lanes, and the weight
+// rows (= columns) are laid out so that each of them gets two runs of eight consecutive outputs: the
+// four write (and read, for the BatchNorm backward) whole 128-byte lines.  With a row per lane every
+// 32-byte access of a warp touched 32 lines, and the L1's line rate bound the BatchNorm-backward
+// epilogue at 107 us (141 with the shortcut) for a first-stage layer of 16 workers x 128 images.
+// A lane then also holds few channels (8, or 16 of 64), so running moments and sums stay in its
+// registers until the end of the kernel: no exchange per tile.
+// Measured there: forward with statistics 35 us, data gradient 32 (201 MB: 6.3 TB/s), with the
+// BatchNorm-backward epilogue 59 (402 MB: 6.8 TB/s), 90 with the shortcut, where conv_tc_kernel took
+// 65, 55, 102 and 135.
+// The BatchNorm-backward epilogue reads up to 192 bytes for every 64 it writes, and four warps that
+// went through a tile's rows one after another were bound by the latency of those reads (102 us, 158
+// with the shortcut): its sixteen warps (eight of an M = 64 tile) take 16 rows x 32 columns each, on
+// one CTA per SM, and request all they read of a tile before they wait for its accumulator.
+namespace sp {
+template <int M, int MODE>
+constexpr int kEpq = MODE == 2 ? M / 32 : 1;  // epilogue warps per TMEM lane quarter
+template <int M, int MODE>
+constexpr int kThreads = 128 + 128 * kEpq<M, MODE>;
+constexpr int MAX_ST = 6;
+constexpr size_t kTwoPerSm = 113 * 1024, kOnePerSm = 224 * 1024;
+constexpr int BOX_W = 10;                    // super-pixels of a box row
+constexpr uint32_t ROWB = BOX_W * 128;       // bytes of a box row
+constexpr size_t AUX = (2 * MAX_ST + 2 * cv::MAX_ACC + 1) * 8 + 16;
+}  // namespace sp
+
+// Eight consecutive values (32-byte aligned) in one access.
+__device__ __forceinline__ void ld8(const float* p, float* v) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+                 "=f"(v[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void st8(float* p, const float* v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]),
+               "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+// Sixteen TMEM lanes x 64 columns: lane l of the warp gets, of rows l / 4 and l / 4 + 8, columns
+// 8 k + 2 (l mod 4) and the next for k < 8: v[4 k .. 4 k + 3] = row l / 4's two, then row l / 4 + 8's.
+__device__ __forceinline__ void tmem_ld_16x256_x8(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
+        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+// The same for 32 columns.
+__device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ bool bf_positive(const uint32_t (&w)[4], int k) {
+  return bf2f((uint16_t)(k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu)) > 0.f;
+}
+
+template <int M, int MODE>  // MODE 0: plain, 1: BatchNorm statistics, 2: BatchNorm-backward epilogue
+__global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv_sp_kernel(
+    const __grid_constant__ ConvSpArgs a) {
+  constexpr int EPQ = sp::kEpq<M, MODE>, THREADS = sp::kThreads<M, MODE>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~uintptr_t(1023));
+  const int ck = a.ck, ks = ck / 16, nst = a.nst, nacc = a.nacc;
+  const int np = 64 * a.nseg;                        // accumulator columns
+  const int per_row = a.nj * ks, nmma = a.nkh * per_row;
+  const uint32_t box_bytes = (uint32_t)a.box_rows * sp::ROWB, pitch = (box_bytes + 1023u) & ~1023u;
+  const uint32_t slice_bytes = (uint32_t)np * 32u;   // one slice's weights
+  uint8_t* wsm = base + nst * pitch;
+  uint64_t* full = reinterpret_cast<uint64_t*>(wsm + nmma * slice_bytes);
+  uint64_t* empty = full + sp::MAX_ST;
+  uint64_t* acc_full = empty + sp::MAX_ST;
+  uint64_t* acc_empty = acc_full + cv::MAX_ACC;
+  uint64_t* w_full = acc_empty + cv::MAX_ACC;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
+  const int g = blockIdx.y, cpr = gridDim.x;
+  const int tpi = a.hg / a.tr, tiles = a.B * tpi;  // tiles per image, per replica
+  const uint32_t tmem_cols = conv_tmem_cols(nacc, np);
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < nst; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < nacc; ++i) {
+      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_empty[i], 4 * EPQ);
+    }
+    mbar_init(w_full, THREADS / 32 - 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+  pdl_begin();  // everything above touched only shared memory and TMEM
+
+  if (warp > 0) {
+    // the weights: 16-byte chunk e = (slice, column n, half of its 16 channels)
+    const uint16_t* w = a.w + (int64_t)g * a.w_gs;
+    for (int e = threadIdx.x - 32; e < nmma * np * 2; e += THREADS - 32) {
+      const int h = e & 1, n = (e >> 1) & (np - 1), sl = (e >> 1) / np;
+      const int khi = sl / per_row, r = sl - khi * per_row, jj = r / ks, kq = r - jj * ks;
+      // column n of a segment is output o of its 64: lane m = (n mod 8) / 2 of a row's four holds
+      // columns 8 k + 2 m, + 1, which are to be outputs 32 i + 8 m + r, r = 2 (k mod 4) + n mod 2
+      const int seg = n >> 6, o = (n & 32) + ((n & 6) << 2) + ((n >> 2) & 6) + (n & 1);
+      const int px = o / a.N, ch = o - px * a.N;
+      // segment and pixel of a column -> source pixel p and (phases) which phase's weights
+      const int p = a.nseg == 2 ? px >> 1 : px, phase = a.nseg == 2 ? 2 * seg + (px & 1) : 0;
+      const int d = a.j0 + jj - p * a.S;  // kernel column
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (d >= 0 && d <= 2)
+        v = __ldg(reinterpret_cast<const uint4*>(
+            w + phase * a.w_ps + (int64_t)(ch * 9 + (a.kh0 + khi) * 3 + d) * ck + kq * 16 + h * 8));
+      *reinterpret_cast<uint4*>(wsm + sl * slice_bytes + n * 32 + ((h ^ ((n >> 2) & 1)) << 4)) = v;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(w_full);
+  }
+
+  if (warp == 0) {
+    // ---------------- producer ----------------
+    const bool el = elect_one();
+    int b = (int)blockIdx.x / tpi, t = (int)blockIdx.x % tpi;
+    int q = 0, sl = 0;
+    uint32_t ph = 1;
+    for (int tile = blockIdx.x; tile < tiles; tile += cpr, ++q) {
+      if (!mbar_wait_warp(&empty[sl], ph)) break;
+      if (el) {
+        mbar_expect_tx(&full[sl], box_bytes);
+        tma_load_5d(base + sl * pitch, &a.in_map, &full[sl], 0, -1, t * a.tr * a.S + a.kh0 - 1, b, g);
+      }
+      if (++sl == nst) {
+        sl = 0;
+        ph ^= 1;
+      }
+      t += cpr;
+      while (t >= tpi) {
+        t -= tpi;
+        ++b;
+      }
+    }
+    // copies in flight land before the CTA can exit
+    for (int j = (q > nst ? q - nst : 0); j < q; ++j) mbar_wait(&full[j % nst], (j / nst) & 1);
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    const bool el = elect_one();
+    const uint32_t idesc = make_idesc(M, np, false, false);
+    // slice j0 of box row 0: the pixels before it in the super-pixel left of the tile's first
+    const uint64_t a_desc0 =
+        smem_desc_swz(smem_u32(base) + 128 - 2 * ck + a.j0 * 2 * ck, 16, (uint32_t)a.S * sp::ROWB, 128);
+    const uint64_t b_desc0 = smem_desc_kmajor(smem_u32(wsm), 32);
+    const uint32_t b_step = slice_bytes >> 4;
+    bool ok = mbar_wait_warp(w_full, 0);
+    int sl = 0, ab = 0;
+    uint32_t ph = 0, ph_acc = 1;
+    for (int tile = blockIdx.x; tile < tiles && ok; tile += cpr) {
+      if (!mbar_wait_warp(&acc_empty[ab], ph_acc) || !mbar_wait_warp(&full[sl], ph)) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t acc = tmem + (uint32_t)(ab * np);
+      const uint64_t st = a_desc0 + ((uint32_t)sl * pitch >> 4);
+      uint64_t bd = b_desc0;
+      uint32_t on = 0;
+      for (int kh = 0; kh < a.nkh; ++kh) {
+        uint64_t ad = st + (uint32_t)kh * (sp::ROWB >> 4);
+#pragma unroll 4
+        for (int r = 0; r < per_row; ++r) {
+          if (el) mma_bf16(acc, ad, bd, idesc, on);
+          on = 1;
+          ad += 2;
+          bd += b_step;
+        }
+      }
+      if (el) {
+        mma_commit(&empty[sl]);
+        mma_commit(&acc_full[ab]);
+      }
+      if (++sl == nst) {
+        sl = 0;
+        ph ^= 1;
+      }
+      if (++ab == nacc) {
+        ab = 0;
+        ph_acc ^= 1;
+      }
+    }
+  } else if (MODE == 2 && warp >= 4) {
+    // ---------------- BatchNorm-backward epilogue ----------------
+    // Warp (h, i) of a quarter: rows 16 h .. 16 h + 15 (two image rows) and outputs 32 i .. 32 i + 31 of
+    // a segment; lane = (super-pixel sx, part m) with outputs 32 i + 8 m + r of both image rows.
+    const int quarter = warp & 3, hi = (warp - 4) >> 2, h = hi >> 1, i = hi & 1;
+    const int sx = lane >> 2, m = lane & 3;
+    const int N = a.N, ps = 64 / N;  // pixels of a segment
+    const ConvBwdFuse& bw = a.bwd;
+    const int o = 32 * i + 8 * m, px = o / N, ch = o & (N - 1);  // this lane's pixel and first channel
+    float sg[8], sgx[8], mu[8];  // sums of g and g (y - mean); the mean
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      sg[r] = sgx[r] = 0.f;
+      mu[r] = bw.mean[g * N + ch + r];
+    }
+    int b = (int)blockIdx.x / tpi, t = (int)blockIdx.x % tpi;
+    int ab = 0;
+    uint32_t ph = 0;
+    // this lane's first output of image row `row` (0, 1) and segment seg of tile (b, t), in pixels
+    auto pixel = [&](int bb, int tt, int row, int seg) -> int64_t {
+      return ((int64_t)bb * a.ho + (tt * a.tr + quarter * (M / 32) + 2 * h + row) * a.rs + seg) * a.wo +
+             sx * ps;
+    };
+    for (int tile = blockIdx.x; tile < tiles; tile += cpr) {
+      const int img = b, tt = t;
+      t += cpr;
+      while (t >= tpi) {
+        t -= tpi;
+        ++b;
+      }
+      bool ok = true;
+      for (int seg = 0; seg < a.nseg; ++seg) {
+        uint4 mk[2], so[2];
+        float yv[2][8], sd[2][8];
+        bool has = false;
+#pragma unroll
+        for (int row = 0; row < 2; ++row) {
+          const int64_t pix = pixel(img, tt, row, seg);
+          const int64_t e = (int64_t)g * a.out_gs + pix * N + o;
+          mk[row] = *reinterpret_cast<const uint4*>(bw.mask + e);
+          ld8(bw.y + e, yv[row]);
+          if (bw.sc_dout) {
+            // the shortcut's source pixel: the same one (stride 1) or, in even rows, every other
+            // pixel's (stride 2: segment 0 is the even row)
+            int64_t src = pix + px;
+            has = true;
+            if (bw.sc_stride == 2) {
+              has = seg == 0 && !(px & 1);
+              src = ((int64_t)img * (a.ho / 2) + tt * a.tr + quarter * (M / 32) + 2 * h + row) * (a.wo / 2) +
+                    (sx * ps + px) / 2;
+            }
+            if (has) {
+              const int64_t se = (int64_t)g * bw.sc_gs + src * bw.sc_C + ch;
+              so[row] = *reinterpret_cast<const uint4*>(bw.sc_out + se);
+              ld8(bw.sc_dout + se, sd[row]);
+            }
+          }
+        }
+        if (tile + cpr < tiles) {
+          // the next tile's into L2
+#pragma unroll
+          for (int row = 0; row < 2; ++row) {
+            const int64_t pix = pixel(b, t, row, seg);
+            const int64_t e = (int64_t)g * a.out_gs + pix * N + o;
+            if (m == 0) {
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(bw.y + e));
+              if (i == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(bw.mask + e));
+              if (bw.sc_dout && bw.sc_stride == 1) {
+                const int64_t se = (int64_t)g * bw.sc_gs + (pix + px) * bw.sc_C + ch;
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(bw.sc_dout + se));
+                if (i == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(bw.sc_out + se));
+              }
+            }
+          }
+        }
+        if (seg == 0) {
+          ok = mbar_wait_warp(&acc_full[ab], ph);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        float v[16];  // v[4 k + 2 row + b]: column 32 i + 8 k + 2 m + b
+        tmem_ld_16x256_x4(
+            tmem + ((uint32_t)(quarter * 32 + 16 * h) << 16) + (uint32_t)(ab * np + 64 * seg + 32 * i), v);
+#pragma unroll
+        for (int row = 0; row < 2; ++row) {
+          // dx (+ the shortcut's share) masked by the layer below's ReLU, and that layer's sums
+          const uint32_t mw[4] = {mk[row].x, mk[row].y, mk[row].z, mk[row].w};
+          const uint32_t ow[4] = {so[row].x, so[row].y, so[row].z, so[row].w};
+          float x[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            x[r] = v[4 * (r >> 1) + 2 * row + (r & 1)];
+            if (has) x[r] += bf_positive(ow, r) ? sd[row][r] : 0.f;
+            x[r] = bf_positive(mw, r) ? x[r] : 0.f;
+            sg[r] += x[r];
+            sgx[r] = fmaf(x[r], yv[row][r] - mu[r], sgx[r]);
+          }
+          st8(a.out + (int64_t)g * a.out_gs + pixel(img, tt, row, seg) * N + o, x);
+        }
+      }
+      if (!ok) break;
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      if (++ab == nacc) {
+        ab = 0;
+        ph ^= 1;
+      }
+    }
+    // one partial per warp: the lanes of a channel added in a fixed order (zeros for the channels
+    // of the other i)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+#pragma unroll
+      for (int d = 4; d <= 16; d <<= 1) {
+        sg[r] += __shfl_xor_sync(0xffffffffu, sg[r], d);
+        sgx[r] += __shfl_xor_sync(0xffffffffu, sgx[r], d);
+      }
+      if (N == 16) {
+        sg[r] += __shfl_xor_sync(0xffffffffu, sg[r], 2);
+        sgx[r] += __shfl_xor_sync(0xffffffffu, sgx[r], 2);
+      }
+    }
+    float2* out = bw.part + ((int64_t)g * bw.part_gs + (int64_t)4 * EPQ * blockIdx.x + (warp - 4)) * N;
+    if (sx == 0 && 8 * m < N) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        out[ch + r] = make_float2(sg[r], sgx[r] * bw.rstd[g * N + ch + r]);
+        if (N == 64) out[(ch ^ 32) + r] = make_float2(0.f, 0.f);
+      }
+    }
+  } else if (MODE != 2 && warp >= 4) {
+    // ---------------- epilogue ----------------
+    // A warp reads 16 rows of its TMEM lane quarter at a time: two image rows of eight super-pixels
+    // each; lane = (super-pixel sx, part m), and m's outputs of a 64-output segment are 32 i + 8 m + r,
+    // i < 2, r < 8.  The warps wait for accumulators and return them by themselves.
+    const int quarter = warp & 3, sx = lane >> 2, m = lane & 3;
+    const int N = a.N, ps = 64 / N;  // pixels of a segment
+    // statistics: running mean and sum of squared deviations of the lane's outputs (i, r)
+    float mean[2][8], m2[2][8];
+    float run_n = 0.f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) mean[i][r] = m2[i][r] = 0.f;
+    int b = (int)blockIdx.x / tpi, t = (int)blockIdx.x % tpi;
+    int ab = 0;
+    uint32_t ph = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += cpr) {
+      const int img = b, y_first = t * a.tr + quarter * (M / 32);  // this warp's first group row
+      t += cpr;
+      while (t >= tpi) {
+        t -= tpi;
+        ++b;
+      }
+      if (!mbar_wait_warp(&acc_full[ab], ph)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+      for (int hs = 0; hs < (M / 64) * a.nseg; ++hs) {
+        const int h = a.nseg == 2 ? hs >> 1 : hs, seg = a.nseg == 2 ? hs & 1 : 0;
+        float v[32];  // v[4 k + 2 row + b]: column 8 k + 2 m + b of image row `row`
+        tmem_ld_16x256_x8(tmem + ((uint32_t)(quarter * 32 + 16 * h) << 16) + (uint32_t)(ab * np + 64 * seg), v);
+        const int64_t pix0 = ((int64_t)img * a.ho + (y_first + 2 * h) * a.rs + seg) * a.wo + sx * ps;
+#pragma unroll
+        for (int row = 0; row < 2; ++row) {
+          float* orow = a.out + (int64_t)g * a.out_gs + (pix0 + (int64_t)row * a.rs * a.wo) * N + 8 * m;
+          float f = 0.f;
+          if (MODE == 1) {
+            run_n += 1.f;
+            f = 1.f / run_n;
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            float x[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) x[r] = v[4 * (4 * i + (r >> 1)) + 2 * row + (r & 1)];
+            st8(orow + 32 * i, x);
+            if (MODE == 1) {
+              // Welford's update of the running moments
+#pragma unroll
+              for (int r = 0; r < 8; ++r) {
+                const float d = x[r] - mean[i][r];
+                mean[i][r] = fmaf(d, f, mean[i][r]);
+                m2[i][r] = fmaf(d, x[r] - mean[i][r], m2[i][r]);
+              }
+            }
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      if (++ab == nacc) {
+        ab = 0;
+        ph ^= 1;
+      }
+    }
+    if (MODE == 1) {
+      // one partial per warp: the lanes that hold the same channel combined in a fixed order, all of
+      // them with the same count
+      float cnt = run_n;
+      auto merge = [&](float& ma, float& sa, float mb, float sb) {
+        const float d = ma - mb;
+        ma = 0.5f * (ma + mb);
+        sa = (sa + sb) + d * d * (0.5f * cnt);
+      };
+      for (int o = 4; o <= 16; o <<= 1) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+            merge(mean[i][r], m2[i][r], __shfl_xor_sync(0xffffffffu, mean[i][r], o),
+                  __shfl_xor_sync(0xffffffffu, m2[i][r], o));
+        cnt *= 2.f;
+      }
+      if (N <= 32) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) merge(mean[0][r], m2[0][r], mean[1][r], m2[1][r]);
+        cnt *= 2.f;
+      }
+      if (N == 16) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          merge(mean[0][r], m2[0][r], __shfl_xor_sync(0xffffffffu, mean[0][r], 2),
+                __shfl_xor_sync(0xffffffffu, m2[0][r], 2));
+        cnt *= 2.f;
+      }
+      if (sx == 0 && 8 * m < N)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (32 * i + 8 * m >= N) break;
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+            a.stats[((int64_t)g * cpr * 4 + 4 * blockIdx.x + quarter) * N + 32 * i + 8 * m + r] =
+                make_float4(cnt, mean[i][r], m2[i][r], 0.f);
+        }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 2) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols)
+                 : "memory");
+  }
+}
+
+// =============================================================================================
 // Weight gradient of a 3x3 convolution on the tensor cores, straight from the NHWC operands:
 //   dW[g][co][t][ci] = sum over output pixels p of dy[g][p][co] x[g][src_t(p)][ci].
 // As D[m][n] = sum_k A[m][k] B[n][k] with k = output pixels, n = co and, for each kernel column kw,
@@ -2245,6 +2729,96 @@ cudaError_t launch_conv_tc(const ConvArgs& a, cudaStream_t stream, int* ctas_per
   }
   if (ctas_per_replica) *ctas_per_replica = 4 * cpr;  // statistics partials: one per epilogue warp
   return launch_pdl(conv_tc_kernel, dim3(cpr, a.G), dim3(cv::THREADS), smem, stream, la);
+}
+
+// The launch shape of conv_sp_kernel; false if it does not take the convolution.
+namespace {
+bool conv_sp_plan(ConvSpArgs& a, int sms, int* cpr, size_t* smem) {
+  if ((a.ck != 16 && a.ck != 32 && a.ck != 64) || (a.N != 16 && a.N != 32 && a.N != 64) || a.wi * a.ck != 512 ||
+      (a.stride != 1 && a.stride != 2) || a.B < 1 || a.G < 1 || a.G > 65535)
+    return false;
+  const int s = 64 / a.ck;  // pixels per super-pixel
+  if (a.phases) {
+    if (2 * s * a.N != 64 || a.stride != 1) return false;
+    a.nseg = 2, a.rs = 2, a.S = 1, a.kh0 = 1, a.nkh = 2, a.j0 = 1, a.nj = s + 1;
+    a.hg = a.hi, a.ho = 2 * a.hi, a.wo = 2 * a.wi;
+  } else {
+    if (a.hi % a.stride || s % a.stride || (s / a.stride) * a.N != 64) return false;
+    a.nseg = 1, a.rs = 1, a.S = a.stride, a.kh0 = 0, a.nkh = 3, a.j0 = 0, a.nj = s + 3 - a.stride;
+    a.hg = a.ho = a.hi / a.stride, a.wo = a.wi / a.stride;
+  }
+  if (a.hg % 8) return false;
+  // 16 image rows a tile (one M = 128 product costs 1.5 of M = 64) where every SM still gets two
+  a.tr = a.hg % 16 == 0 && a.S == 1 && (int64_t)a.G * a.B * (a.hg / 16) >= 2 * sms ? 16 : 8;
+  a.box_rows = (a.tr - 1) * a.S + a.nkh;
+  const size_t pitch = ((size_t)a.box_rows * sp::ROWB + 1023) / 1024 * 1024;
+  const size_t fixed = 1024 + (size_t)a.nkh * a.nj * (a.ck / 16) * 64 * a.nseg * 32 + sp::AUX;
+  a.nacc = a.nseg == 2 ? 2 : 4;
+  int per_sm = 2;
+  size_t st = sp::kTwoPerSm > fixed ? (sp::kTwoPerSm - fixed) / pitch : 0;
+  if (st < 2 || a.bwd.y) {
+    per_sm = 1;
+    st = (sp::kOnePerSm - fixed) / pitch;
+  }
+  if (st < 2) return false;
+  a.nst = (int)std::min<size_t>(st, sp::MAX_ST);
+  *smem = fixed + a.nst * pitch;
+  *cpr = std::max(1, std::min(a.B * (a.hg / a.tr), per_sm * sms / a.G));
+  return true;
+}
+}  // namespace
+
+int conv_sp_parts(const ConvSpArgs& a) {
+  int sms = 0, cpr = 0;
+  size_t smem = 0;
+  ConvSpArgs t = a;
+  if (device_sms(&sms) < 0) return 0;
+  if (!conv_sp_plan(t, sms, &cpr, &smem)) return 0;
+  // one per epilogue warp
+  return 4 * (!a.bwd.y ? 1 : t.tr == 16 ? sp::kEpq<128, 2> : sp::kEpq<64, 2>) * cpr;
+}
+
+cudaError_t launch_conv_sp(const ConvSpArgs& a, const void* in, cudaStream_t stream) {
+  int sms = 0, cpr = 0;
+  size_t smem = 0;
+  ConvSpArgs la = a;
+  const int dev = device_sms(&sms);
+  if (dev < 0) return cudaErrorInvalidDevice;
+  if (!conv_sp_plan(la, sms, &cpr, &smem) || !la.out || !la.w || (reinterpret_cast<uintptr_t>(la.out) & 31) ||
+      la.out_gs % 8 || (reinterpret_cast<uintptr_t>(la.w) & 15) || la.w_gs % 8 || la.w_ps % 8 ||
+      (la.stats && la.bwd.y))
+    return cudaErrorInvalidValue;
+  std::call_once(g_encode_once, load_encode);
+  if (!g_encode || (reinterpret_cast<uintptr_t>(in) & 15)) return cudaErrorInvalidValue;
+  // the NHWC input with 64 channel values (64 / ck pixels) innermost
+  const cuuint64_t H = la.hi, B = la.B, G = la.G;
+  cuuint64_t dims[5] = {64, 8, H, B, G};
+  cuuint64_t strides[4] = {128, 1024, 1024 * H, 1024 * H * B};
+  cuuint32_t box[5] = {64, (cuuint32_t)sp::BOX_W, (cuuint32_t)la.box_rows, 1, 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  if (g_encode(&la.in_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(in), dims, strides, box,
+               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  const int mode = la.stats ? 1 : (la.bwd.y ? 2 : 0);
+  static int attr_dev[2][3] = {{-1, -1, -1}, {-1, -1, -1}};
+  auto run = [&](auto kernel, int threads) -> cudaError_t {
+    int& ad = attr_dev[la.tr == 16][mode];
+    if (ad != dev) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp::kOnePerSm);
+      if (e != cudaSuccess) return e;
+      ad = dev;
+    }
+    return launch_pdl(kernel, dim3(cpr, la.G), dim3(threads), smem, stream, la);
+  };
+  if (la.tr == 16)
+    return mode == 1   ? run(conv_sp_kernel<128, 1>, sp::kThreads<128, 1>)
+           : mode == 2 ? run(conv_sp_kernel<128, 2>, sp::kThreads<128, 2>)
+                       : run(conv_sp_kernel<128, 0>, sp::kThreads<128, 0>);
+  return mode == 1   ? run(conv_sp_kernel<64, 1>, sp::kThreads<64, 1>)
+         : mode == 2 ? run(conv_sp_kernel<64, 2>, sp::kThreads<64, 2>)
+                     : run(conv_sp_kernel<64, 0>, sp::kThreads<64, 0>);
 }
 
 cudaError_t launch_wgrad_update(const WgradUpdateArgs& a, cudaStream_t stream) {

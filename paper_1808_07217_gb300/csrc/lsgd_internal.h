@@ -220,6 +220,30 @@ bool conv_strip_ok(int hout, int wout, int stride);
 cudaError_t launch_conv_tc(const ConvArgs& a, cudaStream_t stream, int* ctas_per_replica = nullptr);
 // The CTAs per replica launch_conv_tc will use for these arguments (0 if it would reject them).
 int conv_tc_ctas(const ConvArgs& a);
+// The same convolutions where an image row is 512 channel values (wi ck = 512) and the output's
+// pixels over one 64-value super-pixel of it give 64 columns (conv_sp_kernel): input [G][B][hi][wi][ck]
+// bf16, weights w [N][9][ck] bf16 per replica (stride w_gs), output [G][B][ho][wo][N] fp32, 32-byte
+// aligned.  phases: the input is the output gradient of a stride-2 layer and w its four parity
+// phases' weights (stride w_ps between phases, flip_phase_weights_kernel); the output has twice the
+// rows and columns.  stats and bwd as in ConvArgs (part_off unused; bwd.sc_stride 2 only with phases).
+struct ConvSpArgs {
+  CUtensorMap in_map;  // set by the launcher
+  const uint16_t* w;
+  int64_t w_gs, w_ps;
+  int ck, N, stride, phases, hi, wi, B, G;
+  float* out;
+  int64_t out_gs;
+  float4* stats;
+  ConvBwdFuse bwd;
+  // set by the launcher: columns / 64; output rows per input row group; row stride; first kernel row
+  // and their number; first pixel (0 = the one left of the super-pixel) and their number; group
+  // rows, output size; tile rows, box rows; ring stages and accumulators
+  int nseg, rs, S, kh0, nkh, j0, nj, hg, ho, wo, tr, box_rows, nst, nacc;
+};
+// The partials per replica that launch_conv_sp writes to stats or bwd.part (a number > 0 without
+// either), or 0 if it does not take the convolution.
+int conv_sp_parts(const ConvSpArgs& a);
+cudaError_t launch_conv_sp(const ConvSpArgs& a, const void* in, cudaStream_t stream);
 // Weight gradient of a 3x3 convolution (zero padding 1, stride 1 or 2) on the tensor cores:
 // part[g][q][co][t Cin + ci] = the sum over CTA q's output pixels of dy[g][p][co] x[g][src_t(p)][ci],
 // src_t(p) the input pixel under tap t of output pixel p (zero outside the image).  x_map:

@@ -1305,6 +1305,17 @@ size_t conv_wt_elems(int G, int cin, int cout, int stride) {
   return (size_t)(stride == 2 ? 4 : 1) * G * cin * 9 * cout;
 }
 
+// The partials per replica of a convolution on conv_sp_kernel (conv_sp_parts), 0 where it does not take it (its
+// shape, or buffers that its 32-byte accesses of the output and 16-byte ones of the weights reject).
+int conv_sp_takes(const ConvSpArgs& a) {
+  auto al = [](const void* p, uintptr_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; };
+  if (!al(a.out, 32) || a.out_gs % 8 || !al(a.w, 16) || a.w_gs % 8 || a.w_ps % 8) return 0;
+  if (a.bwd.y && (!al(a.bwd.y, 32) || !al(a.bwd.mask, 32) || (a.bwd.sc_dout && (!al(a.bwd.sc_dout, 32) ||
+                                                                               !al(a.bwd.sc_out, 32)))))
+    return 0;
+  return conv_sp_parts(a);
+}
+
 lsgd_status conv_fwd_tc(const uint16_t* x, const uint16_t* w, int64_t w_gs, float* y, int G, int B,
                         int hin, int win, int cin, int cout, int stride, uint16_t* x16,
                         uint16_t* wstem, cudaStream_t s, std::string& err, int64_t* launches,
@@ -1315,6 +1326,22 @@ lsgd_status conv_fwd_tc(const uint16_t* x, const uint16_t* w, int64_t w_gs, floa
   }
   const int hout = conv_out_size(hin, stride), wout = conv_out_size(win, stride);
   const int64_t P = (int64_t)B * hout * wout;
+  auto sp_args = [&](const uint16_t* wt, int64_t wt_gs, int ck) {
+    ConvSpArgs sa{};
+    sa.w = wt;
+    sa.w_gs = wt_gs;
+    sa.ck = ck;
+    sa.N = cout;
+    sa.stride = stride;
+    sa.hi = hin;
+    sa.wi = win;
+    sa.B = B;
+    sa.G = G;
+    sa.out = y;
+    sa.out_gs = P * cout;
+    sa.stats = stats;
+    return sa;
+  };
   ConvArgs ca{};
   bool okc;
   if (cin < 16) {
@@ -1323,12 +1350,24 @@ lsgd_status conv_fwd_tc(const uint16_t* x, const uint16_t* w, int64_t w_gs, floa
     CV_LAUNCH(launch_pdl(pad_input16_kernel, grid_cap(npix, 256), 256, 0, s, x, x16, npix, cin));
     CV_LAUNCH(launch_pdl(pad_stem_weights_kernel, grid_cap((int64_t)G * cout * 144, 256), 256, 0, s,
                          w, w_gs, (int64_t)0, wstem, G, cout, cin));
+    const ConvSpArgs sa = sp_args(wstem, (int64_t)cout * 9 * 16, 16);
+    if (const int n = conv_sp_takes(sa)) {
+      if (nparts && stats) *nparts = n;
+      CV_CALL(launch_conv_sp(sa, x16, s));
+      return LSGD_OK;
+    }
     ca.strip = conv_strip_ok(hout, wout, 1);
     okc = make_tma_map_conv(&ca.in_map, x16, 16, win, hin, B, G, wout, hout, 1, ca.strip);
     okc &= make_tma_map(&ca.w_map, wstem, true, 9 * 16, cout, G, 9 * 16, (uint64_t)cout * 9 * 16, 16,
                         cout, 32);
     ca.ck = 16;
   } else {
+    const ConvSpArgs sa = sp_args(w, w_gs, cin);
+    if (const int n = conv_sp_takes(sa)) {
+      if (nparts && stats) *nparts = n;
+      CV_CALL(launch_conv_sp(sa, x, s));
+      return LSGD_OK;
+    }
     ca.strip = conv_strip_ok(hout, wout, stride);
     okc = make_tma_map_conv(&ca.in_map, x, cin, win, hin, B, G, wout, hout, stride, ca.strip);
     okc &= make_tma_map(&ca.w_map, w, true, 9 * cin, cout, G, 9 * cin, w_gs, cin, cout, 2 * cin);
@@ -1369,6 +1408,25 @@ lsgd_status conv_dgrad_tc(const uint16_t* dy, const uint16_t* w, int64_t w_gs, f
     if (!flipped)
       CV_LAUNCH((launch_pdl(flip_weights_kernel, dim3((unsigned)((cin * 9 * cout + 255) / 256), (unsigned)G),
                             256, 0, s, w, w_gs, (int64_t)0, wt, G, cin, cout)));
+    ConvSpArgs sa{};
+    sa.w = wt;
+    sa.w_gs = (int64_t)cin * 9 * cout;
+    sa.ck = cout;
+    sa.N = cin;
+    sa.stride = 1;
+    sa.hi = hin;
+    sa.wi = win;
+    sa.B = B;
+    sa.G = G;
+    sa.out = dx;
+    sa.out_gs = P * cin;
+    if (bf) sa.bwd = *bf;
+    if (const int n = conv_sp_takes(sa)) {
+      sa.bwd.part_gs = n;
+      if (nparts && bf) *nparts = n;
+      CV_CALL(launch_conv_sp(sa, dy, s));
+      return LSGD_OK;
+    }
     ConvArgs ca{};
     ca.strip = conv_strip_ok(hin, win, 1);
     bool okc = make_tma_map_conv(&ca.in_map, dy, cout, win, hin, B, G, win, hin, 1, ca.strip);
@@ -1408,6 +1466,27 @@ lsgd_status conv_dgrad_tc(const uint16_t* dy, const uint16_t* w, int64_t w_gs, f
   if (!flipped)
     CV_LAUNCH(launch_pdl(flip_phase_weights_kernel, grid_cap(4 * (int64_t)G * per, 256), 256, 0, s,
                          w, w_gs, (int64_t)0, wt, G, cin, cout));
+  ConvSpArgs sa{};
+  sa.w = wt;
+  sa.w_gs = per;
+  sa.w_ps = G * per;
+  sa.ck = cout;
+  sa.N = cin;
+  sa.stride = 1;
+  sa.phases = 1;
+  sa.hi = hout;
+  sa.wi = wout;
+  sa.B = B;
+  sa.G = G;
+  sa.out = dx;
+  sa.out_gs = P * cin;
+  if (bf) sa.bwd = *bf;
+  if (const int n = conv_sp_takes(sa)) {  // all four in one launch
+    sa.bwd.part_gs = n;
+    if (nparts && bf) *nparts = n;
+    CV_CALL(launch_conv_sp(sa, dy, s));
+    return LSGD_OK;
+  }
   const int64_t Pq = (int64_t)B * hout * wout;
   for (int ph = 0; ph < 4; ++ph) {
     ConvArgs ca{};

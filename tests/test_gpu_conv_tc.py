@@ -86,6 +86,10 @@ FORWARD = [  # (G, B, Hin, Win, Cin, Cout, stride): ResNet-20's forward convolut
     (2, 6, 8, 8, 64, 64, 1),       # stage 3
     (16, 16, 32, 32, 16, 16, 1),   # many groups, several tiles per CTA
     (16, 4, 32, 32, 3, 16, 1),     # stem with many groups
+    (16, 20, 16, 16, 32, 32, 1),   # sixteen-row tiles of whole images
+    (5, 7, 16, 16, 32, 32, 1),     # eight-row tiles, CTAs with unequal shares
+    (2, 3, 32, 64, 16, 16, 1),     # rows wider than eight super-pixels: the tap kernel
+    (2, 4, 8, 32, 16, 16, 1),      # eight image rows
 ]
 
 
@@ -113,6 +117,9 @@ DGRAD = [  # (G, B, Hin, Win, Cin, Cout, stride): ResNet-20's input gradients
     (2, 6, 8, 8, 64, 64, 1),       # stage 3
     (16, 16, 32, 32, 16, 16, 1),   # many groups, several tiles per CTA
     (16, 8, 32, 32, 16, 32, 2),    # parity phases with many groups
+    (16, 20, 32, 32, 16, 32, 2),   # phases in sixteen-row tiles
+    (16, 10, 32, 32, 16, 16, 1),
+    (3, 2, 16, 16, 32, 64, 2),     # phases over 64 channels
 ]
 
 
