@@ -1528,6 +1528,21 @@ lsgd_status conv_dgrad_tc(const uint16_t* dy, const uint16_t* w, int64_t w_gs, f
   return LSGD_OK;
 }
 
+// Layer c's data gradient runs on conv_sp_kernel (the step's buffers are all 256-byte aligned).
+bool dgrad_on_sp(const ResNetPlan* p, const ConvL& c) {
+  if (!conv_dgrad_tc_route(p->B, c.hin, c.win, c.cin, c.cout, c.stride)) return false;
+  ConvSpArgs a{};
+  a.ck = c.cout;
+  a.N = c.cin;
+  a.stride = 1;
+  a.phases = c.stride == 2;
+  a.hi = c.hout;
+  a.wi = c.wout;
+  a.B = p->B;
+  a.G = p->K;
+  return conv_sp_parts(a) > 0;
+}
+
 // Convolution c of G replicas on the fp32 cores.
 ConvSimtArgs simt_args(const ResNetPlan* p, const ConvL& c, int G) {
   ConvSimtArgs a{};
@@ -1863,10 +1878,12 @@ lsgd_status conv_dgrad(ResNetPlan* p, int i, const void* Wop, float* dx, const f
   const int64_t P = (int64_t)p->B * c.hin * c.win;
   if (fused_parts) *fused_parts = 0;
   ConvBwdFuse bf{};
-  // measured per layer in the ResNet-20 step: the fused epilogue's extra loads pay for themselves
-  // on the 16-channel data gradients (the largest tensors) but not on the 32 / 64-channel ones,
-  // where the separate passes are cheaper than the epilogue's added latency
-  const bool fuse = bn_t >= 0 && fused_parts && p->bpart && sizeof(TA) == 2 && c.cin <= 16;
+  // The fused epilogue replaces the BatchNorm backward's sums pass and the shortcut pass.  Measured
+  // in the ResNet-20 step (16 workers x 128 images): on conv_sp_kernel it pays at every stage (8.13 ->
+  // 7.48 ms for two steps with the 32- and 64-channel layers fused too); conv_tc_kernel's four
+  // epilogue warps hide its loads only beside the 16-channel layers' larger products.
+  const bool fuse = bn_t >= 0 && fused_parts && p->bpart && sizeof(TA) == 2 && conv_on_tc(p, c) &&
+                    (c.cin <= 16 || dgrad_on_sp(p, c));
   if (fuse) {
     bf.mask = reinterpret_cast<const uint16_t*>(p->act[bn_t]);
     bf.y = p->y[bn_t];
