@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   Smem<BN, STAGES>& sm = *reinterpret_cast<Smem<BN, STAGES>*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int splits = args.splits > 1 ? args.splits : 1;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM, g = blockIdx.z / splits;
   // implicit convolution: the tile's 128 output pixels are rows of whole images (TW = Wout) from
@@ -510,13 +510,13 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   pdl_begin();  // everything above touched only shared memory and TMEM
 
   bool ok = true;
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- TMA producer ----------------
-    int issued = 0;
-    for (int kb = 0; kb < nk && ok; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (kb / STAGES) & 1;
-      if (!mbar_wait(&sm.empty[s], ph ^ 1)) {
+    const bool el = elect_one();
+    int issued = 0, s = 0;
+    uint32_t ph = 1;
+    for (int kb = 0; kb < nk; ++kb) {
+      if (!mbar_wait_warp(&sm.empty[s], ph)) {
         ok = false;
         break;
       }
@@ -525,80 +525,90 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
         // image, stride by the map's element strides) and the weights' tap-t slice [N][Ck]
         const int ck = args.cv_ck, tps = 64 / ck;
         const int t0 = (kb_first + kb) * tps, t1 = min(9, t0 + tps);
-        mbar_expect_tx(&sm.full[s], (uint32_t)(t1 - t0) * (BM + BN) * ck * 2);
-        for (int t = t0; t < t1; ++t) {
-          const int kh = t / 3, kw = t % 3, j = t - t0;
-          tma_load_5d(sm.a[s] + j * BM * ck * 2, &args.A.map, &sm.full[s], 0, kw - 1,
-                      cv_oy0 * args.cv_stride + kh - 1, cv_b0, g);
-          tma_load_3d(sm.b[s] + j * BN * ck * 2, &args.B.map, &sm.full[s], t * ck, n0, g);
+        if (el) {
+          mbar_expect_tx(&sm.full[s], (uint32_t)(t1 - t0) * (BM + BN) * ck * 2);
+          for (int t = t0; t < t1; ++t) {
+            const int kh = t / 3, kw = t % 3, j = t - t0;
+            tma_load_5d(sm.a[s] + j * BM * ck * 2, &args.A.map, &sm.full[s], 0, kw - 1,
+                        cv_oy0 * args.cv_stride + kh - 1, cv_b0, g);
+            tma_load_3d(sm.b[s] + j * BN * ck * 2, &args.B.map, &sm.full[s], t * ck, n0, g);
+          }
         }
-        issued = kb + 1;
-        continue;
-      }
-      mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
-      const int k0 = (kb_first + kb) * BK;
-      if (!a_mn) {
-        tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
-      } else {
+      } else if (el) {
+        mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
+        const int k0 = (kb_first + kb) * BK;
+        if (!a_mn) {
+          tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
+        } else {
 #pragma unroll
-        for (int i = 0; i < BM / 64; ++i)
-          tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
-      }
-      const int gb = args.b_shared ? 0 : g;  // identical replicas: group 0's copy for all
-      if (!b_mn) {
-        // K-major B: BN / box_rows boxes stacked along N (8-row swizzle atoms, rows contiguous)
-        const int brows = args.B.box_rows;
-        for (int i = 0; i < BN / brows; ++i)
-          tma_load_3d(sm.b[s] + i * brows * BK * 2, &args.B.map, &sm.full[s], k0, n0 + i * brows, gb);
-      } else {
+          for (int i = 0; i < BM / 64; ++i)
+            tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+        }
+        const int gb = args.b_shared ? 0 : g;  // identical replicas: group 0's copy for all
+        if (!b_mn) {
+          // K-major B: BN / box_rows boxes stacked along N (8-row swizzle atoms, rows contiguous)
+          const int brows = args.B.box_rows;
+          for (int i = 0; i < BN / brows; ++i)
+            tma_load_3d(sm.b[s] + i * brows * BK * 2, &args.B.map, &sm.full[s], k0, n0 + i * brows, gb);
+        } else {
 #pragma unroll
-        for (int i = 0; i < BN / 64; ++i)
-          tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
+          for (int i = 0; i < BN / 64; ++i)
+            tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
+        }
       }
       issued = kb + 1;
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1;
+      }
     }
     if (!ok) {
       // let copies already in flight land before the CTA can exit
       for (int kb = (issued > STAGES ? issued - STAGES : 0); kb < issued; ++kb)
         mbar_wait(&sm.full[kb % STAGES], (kb / STAGES) & 1);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
+    const bool el = elect_one();
     constexpr uint32_t idesc_kk = make_idesc(BM, BN, false, false);
     const uint32_t idesc = idesc_kk | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16);
+    // descriptors of stage 0; a stage and a 16-deep slice add their byte offsets / 16
+    const uint64_t a_desc0 = a_mn ? smem_desc(smem_u32(sm.a[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.a[0]), 16, 1024);
+    const uint64_t b_desc0 = b_mn ? smem_desc(smem_u32(sm.b[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.b[0]), 16, 1024);
+    const uint32_t a_step = a_mn ? 2048 >> 4 : 32 >> 4, b_step = b_mn ? 2048 >> 4 : 32 >> 4;
+    int s = 0;
+    uint32_t ph = 0;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (kb / STAGES) & 1;
-      if (!mbar_wait(&sm.full[s], ph)) {
+      if (!mbar_wait_warp(&sm.full[s], ph)) {
         ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_base = smem_u32(sm.a[s]), b_base = smem_u32(sm.b[s]);
       if (args.conv) {
         // each tap's sub-tiles: rows of Ck bf16 = swz bytes; K = 16 per MMA, 32 bytes further
+        const uint32_t a_base = smem_u32(sm.a[s]), b_base = smem_u32(sm.b[s]);
         const int ck = args.cv_ck, tps = 64 / ck;
         const int nt = min(9, (kb_first + kb + 1) * tps) - (kb_first + kb) * tps;
         const uint32_t swz = (uint32_t)ck * 2;
-        for (int j = 0; j < nt; ++j)
-          for (int kk = 0; kk < ck / 16; ++kk)
-            mma_bf16(tmem, smem_desc_kmajor(a_base + j * BM * ck * 2 + kk * 32, swz),
-                     smem_desc_kmajor(b_base + j * BN * ck * 2 + kk * 32, swz), idesc,
-                     (kb > 0 || j > 0 || kk > 0) ? 1u : 0u);
-        mma_commit(&sm.empty[s]);
-        continue;
-      }
+        if (el)
+          for (int j = 0; j < nt; ++j)
+            for (int kk = 0; kk < ck / 16; ++kk)
+              mma_bf16(tmem, smem_desc_kmajor(a_base + j * BM * ck * 2 + kk * 32, swz),
+                       smem_desc_kmajor(b_base + j * BN * ck * 2 + kk * 32, swz), idesc,
+                       (kb > 0 || j > 0 || kk > 0) ? 1u : 0u);
+      } else {
+        const uint64_t ad = a_desc0 + (uint32_t)s * (kBytesA >> 4), bd = b_desc0 + (uint32_t)s * (kBytesB >> 4);
 #pragma unroll
-      for (int kk = 0; kk < BK / 16; ++kk) {
-        const uint64_t ad = a_mn ? smem_desc(a_base + kk * 2048, 64 * BK * 2, 1024)
-                                 : smem_desc(a_base + kk * 32, 16, 1024);
-        const uint64_t bd = b_mn ? smem_desc(b_base + kk * 2048, 64 * BK * 2, 1024)
-                                 : smem_desc(b_base + kk * 32, 16, 1024);
-        mma_bf16(tmem, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < BK / 16; ++kk)
+          if (el) mma_bf16(tmem, ad + kk * a_step, bd + kk * b_step, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
       }
-      mma_commit(&sm.empty[s]);  // stage reusable once these MMAs have read it
+      if (el) mma_commit(&sm.empty[s]);  // stage reusable once these MMAs have read it
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1;
+      }
     }
-    if (ok) mma_commit(&sm.accum);  // accumulator complete
+    if (ok && el) mma_commit(&sm.accum);  // accumulator complete
   } else if (warp >= 2 && args.epi == EPI_MASK && args.mask) {
     // warps 2-3 idle through the mainloop: they bring the tile's ReLU-mask rows (the stored
     // activation) into L1, so that the epilogue's mask loads hit L1 instead of waiting on DRAM
@@ -675,7 +685,7 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
   PtSmem& sm = *reinterpret_cast<PtSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                           ~uintptr_t(1023));
   constexpr int PBN = pt::PBN, PST = pt::PST;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int tiles_n = (args.N + PBN - 1) / PBN, tiles_m = (args.M + BM - 1) / BM;
   const int tiles = tiles_n * tiles_m * args.G;
   const int nk = (args.Kd + BK - 1) / BK;
@@ -715,37 +725,44 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
   const uint32_t tmem = sm.tmem_base;
   pdl_begin();  // everything above touched only shared memory and TMEM
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- TMA producer ----------------
-    int it = 0;
+    const bool el = elect_one();
+    int it = 0, s = 0;
+    uint32_t ph = 1;
     bool ok = true;
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       int g, m0, n0;
       coords(t, g, m0, n0);
       const int gb = args.b_shared ? 0 : g;  // identical replicas: replica 0's copy for all
       for (int kb = 0; kb < nk; ++kb, ++it) {
-        const int s = it % PST;
-        if (!mbar_wait(&sm.empty[s], ((it / PST) & 1) ^ 1)) {
+        if (!mbar_wait_warp(&sm.empty[s], ph)) {
           ok = false;
           break;
         }
-        mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
-        const int k0 = kb * BK;
-        if (!a_mn) {
-          tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
-        } else {
+        if (el) {
+          mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
+          const int k0 = kb * BK;
+          if (!a_mn) {
+            tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
+          } else {
 #pragma unroll
-          for (int i = 0; i < BM / 64; ++i)
-            tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+            for (int i = 0; i < BM / 64; ++i)
+              tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+          }
+          if (!b_mn) {
+            const int brows = args.B.box_rows;  // 64-row boxes stacked along N
+            for (int i = 0; i < PBN / brows; ++i)
+              tma_load_3d(sm.b[s] + i * brows * BK * 2, &args.B.map, &sm.full[s], k0, n0 + i * brows, gb);
+          } else {
+#pragma unroll
+            for (int i = 0; i < PBN / 64; ++i)
+              tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
+          }
         }
-        if (!b_mn) {
-          const int brows = args.B.box_rows;  // 64-row boxes stacked along N
-          for (int i = 0; i < PBN / brows; ++i)
-            tma_load_3d(sm.b[s] + i * brows * BK * 2, &args.B.map, &sm.full[s], k0, n0 + i * brows, gb);
-        } else {
-#pragma unroll
-          for (int i = 0; i < PBN / 64; ++i)
-            tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
+        if (++s == PST) {
+          s = 0;
+          ph ^= 1;
         }
       }
     }
@@ -753,36 +770,40 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
       for (int j = (it > PST ? it - PST : 0); j < it; ++j)
         mbar_wait(&sm.full[j % PST], (j / PST) & 1);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
+    const bool el = elect_one();
     constexpr uint32_t idesc_kk = make_idesc(BM, PBN, false, false);
     const uint32_t idesc = idesc_kk | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16);
-    int it = 0, i = 0;
+    // descriptors of stage 0; a stage and a 16-deep slice add their byte offsets / 16
+    const uint64_t a_desc0 = a_mn ? smem_desc(smem_u32(sm.a[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.a[0]), 16, 1024);
+    const uint64_t b_desc0 = b_mn ? smem_desc(smem_u32(sm.b[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.b[0]), 16, 1024);
+    const uint32_t a_step = a_mn ? 2048 >> 4 : 32 >> 4, b_step = b_mn ? 2048 >> 4 : 32 >> 4;
+    int i = 0, s = 0;
+    uint32_t ph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
       const int ab = i & 1;
-      if (!mbar_wait(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1)) break;
+      if (!mbar_wait_warp(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t acc = tmem + (uint32_t)(ab * PBN);
-      for (int kb = 0; kb < nk; ++kb, ++it) {
-        const int s = it % PST;
-        if (!mbar_wait(&sm.full[s], (it / PST) & 1)) {
+      for (int kb = 0; kb < nk; ++kb) {
+        if (!mbar_wait_warp(&sm.full[s], ph)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a_base = smem_u32(sm.a[s]), b_base = smem_u32(sm.b[s]);
+        const uint64_t ad = a_desc0 + (uint32_t)s * (kBytesA >> 4), bd = b_desc0 + (uint32_t)s * (kBytesB >> 4);
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-          const uint64_t ad = a_mn ? smem_desc(a_base + kk * 2048, 64 * BK * 2, 1024)
-                                   : smem_desc(a_base + kk * 32, 16, 1024);
-          const uint64_t bd = b_mn ? smem_desc(b_base + kk * 2048, 64 * BK * 2, 1024)
-                                   : smem_desc(b_base + kk * 32, 16, 1024);
-          mma_bf16(acc, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < BK / 16; ++kk)
+          if (el) mma_bf16(acc, ad + kk * a_step, bd + kk * b_step, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+        if (el) mma_commit(&sm.empty[s]);
+        if (++s == PST) {
+          s = 0;
+          ph ^= 1;
         }
-        mma_commit(&sm.empty[s]);
       }
-      if (ok) mma_commit(&sm.acc_full[ab]);
+      if (ok && el) mma_commit(&sm.acc_full[ab]);
     }
   } else if (warp >= 4) {
     // ---------------- epilogue ----------------
@@ -1061,7 +1082,7 @@ __global__ void __launch_bounds__(wu::THREADS, 1) wgrad_update_kernel(
   extern __shared__ uint8_t smem_raw[];
   WuSmem& sm = *reinterpret_cast<WuSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                           ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   // the layers' tiles one layer after another (operand layouts are the same in all): layer l's
   // tiles follow uc_l tile positions (uc_l G tiles) of the layers before it (scalars, so that
   // nothing needs local memory)
@@ -1157,35 +1178,42 @@ __global__ void __launch_bounds__(wu::THREADS, 1) wgrad_update_kernel(
     g = avg ? gi : (gi + 1) % args.G;
   };
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- operand producer ----------------
-    int it = 0;
+    const bool el = elect_one();
+    int it = 0, s = 0;
+    uint32_t ph = 1;
     bool ok = true;
     for (int j = 0; j < my_count && ok; ++j) {
       const WgradUpdateLayer* ly;
       int g, m0, n0, gi;
       tile_at(j, ly, g, m0, n0, gi);
       for (int kb = 0; kb < nk; ++kb, ++it) {
-        const int s = it % wu::ST;
-        if (!mbar_wait(&sm.op_empty[s], ((it / wu::ST) & 1) ^ 1)) {
+        if (!mbar_wait_warp(&sm.op_empty[s], ph)) {
           ok = false;
           break;
         }
-        mbar_expect_tx(&sm.op_full[s], kBytesA + kBytesB);
-        const int k0 = kb * BK;
-        if (!a_mn) {
-          tma_load_3d(sm.a[s], &ly->A.map, &sm.op_full[s], k0, m0, g);
-        } else {
+        if (el) {
+          mbar_expect_tx(&sm.op_full[s], kBytesA + kBytesB);
+          const int k0 = kb * BK;
+          if (!a_mn) {
+            tma_load_3d(sm.a[s], &ly->A.map, &sm.op_full[s], k0, m0, g);
+          } else {
 #pragma unroll
-          for (int i = 0; i < BM / 64; ++i)
-            tma_load_3d(sm.a[s] + i * 64 * BK * 2, &ly->A.map, &sm.op_full[s], m0 + 64 * i, k0, g);
+            for (int i = 0; i < BM / 64; ++i)
+              tma_load_3d(sm.a[s] + i * 64 * BK * 2, &ly->A.map, &sm.op_full[s], m0 + 64 * i, k0, g);
+          }
+          if (!b_mn) {
+            tma_load_3d(sm.b[s], &ly->B.map, &sm.op_full[s], k0, n0, g);
+          } else {
+#pragma unroll
+            for (int i = 0; i < wu::TN / 64; ++i)
+              tma_load_3d(sm.b[s] + i * 64 * BK * 2, &ly->B.map, &sm.op_full[s], n0 + 64 * i, k0, g);
+          }
         }
-        if (!b_mn) {
-          tma_load_3d(sm.b[s], &ly->B.map, &sm.op_full[s], k0, n0, g);
-        } else {
-#pragma unroll
-          for (int i = 0; i < wu::TN / 64; ++i)
-            tma_load_3d(sm.b[s] + i * 64 * BK * 2, &ly->B.map, &sm.op_full[s], n0 + 64 * i, k0, g);
+        if (++s == wu::ST) {
+          s = 0;
+          ph ^= 1;
         }
       }
     }
@@ -1194,39 +1222,45 @@ __global__ void __launch_bounds__(wu::THREADS, 1) wgrad_update_kernel(
       for (int j = (it > wu::ST ? it - wu::ST : 0); j < it; ++j)
         mbar_wait(&sm.op_full[j % wu::ST], (j / wu::ST) & 1);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
+    const bool el = elect_one();
     const uint32_t idesc = make_idesc(BM, wu::TN, a_mn, b_mn);
-    int it = 0, i = 0;
+    // descriptors of stage 0; a stage and a 16-deep slice add their byte offsets / 16
+    const uint64_t a_desc0 = a_mn ? smem_desc(smem_u32(sm.a[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.a[0]), 16, 1024);
+    const uint64_t b_desc0 = b_mn ? smem_desc(smem_u32(sm.b[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.b[0]), 16, 1024);
+    const uint32_t a_step = a_mn ? 2048 >> 4 : 32 >> 4, b_step = b_mn ? 2048 >> 4 : 32 >> 4;
+    int i = 0, s = 0;
+    uint32_t ph = 0;
     bool ok = true;
     for (; i < my_count && ok; ++i) {
       const int ab = i & 1;
-      if (!mbar_wait(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1)) break;
+      if (!mbar_wait_warp(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t acc = tmem + (uint32_t)(ab * wu::TN);
-      for (int kb = 0; kb < nk; ++kb, ++it) {
-        const int s = it % wu::ST;
-        if (!mbar_wait(&sm.op_full[s], (it / wu::ST) & 1)) {
+      for (int kb = 0; kb < nk; ++kb) {
+        if (!mbar_wait_warp(&sm.op_full[s], ph)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a_base = smem_u32(sm.a[s]), b_base = smem_u32(sm.b[s]);
+        const uint64_t ad = a_desc0 + (uint32_t)s * (kBytesA >> 4), bd = b_desc0 + (uint32_t)s * (kBytesB >> 4);
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-          const uint64_t ad = a_mn ? smem_desc(a_base + kk * 2048, 64 * BK * 2, 1024)
-                                   : smem_desc(a_base + kk * 32, 16, 1024);
-          const uint64_t bd = b_mn ? smem_desc(b_base + kk * 2048, 64 * BK * 2, 1024)
-                                   : smem_desc(b_base + kk * 32, 16, 1024);
-          mma_bf16(acc, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < BK / 16; ++kk)
+          if (el) mma_bf16(acc, ad + kk * a_step, bd + kk * b_step, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+        if (el) mma_commit(&sm.op_empty[s]);
+        if (++s == wu::ST) {
+          s = 0;
+          ph ^= 1;
         }
-        mma_commit(&sm.op_empty[s]);
       }
-      if (ok) mma_commit(&sm.acc_full[ab]);
+      if (ok && el) mma_commit(&sm.acc_full[ab]);
     }
-  } else if (warp == 2 && lane == 0) {
+  } else if (warp == 2) {
     // ---------------- w / u chunk producer ----------------
-    int q = 0;
+    const bool el = elect_one();
+    int q = 0, sl = 0;
+    uint32_t ph = 1;
     bool ok = true;
     const uint32_t bytes = wu::kChunkF32 * (has_u ? 2u : 1u);
     for (int j = 0; j < my_count && ok; ++j) {
@@ -1236,27 +1270,35 @@ __global__ void __launch_bounds__(wu::THREADS, 1) wgrad_update_kernel(
       const int gw = args.w_rep0 ? 0 : g;  // identical replicas: read replica 0's
       const int nc = wu_chunks(ly->N, n0);
       for (int c = 0; c < nc; ++c, ++q) {
-        const int sl = q % wu::NS;
-        if (!mbar_wait(&sm.wu_empty[sl], ((q / wu::NS) & 1) ^ 1)) {
+        if (!mbar_wait_warp(&sm.wu_empty[sl], ph)) {
           ok = false;
           break;
         }
-        mbar_expect_tx(&sm.wu_full[sl], bytes);
-        tma_load_3d(sm.w[sl], &ly->wmap, &sm.wu_full[sl], n0 + c * wu::CW, m0, gw);
-        if (has_u) tma_load_3d(sm.u[sl], &ly->umap, &sm.wu_full[sl], n0 + c * wu::CW, m0, g);
+        if (el) {
+          mbar_expect_tx(&sm.wu_full[sl], bytes);
+          tma_load_3d(sm.w[sl], &ly->wmap, &sm.wu_full[sl], n0 + c * wu::CW, m0, gw);
+          if (has_u) tma_load_3d(sm.u[sl], &ly->umap, &sm.wu_full[sl], n0 + c * wu::CW, m0, g);
+        }
+        if (++sl == wu::NS) {
+          sl = 0;
+          ph ^= 1;
+        }
       }
     }
     if (!ok) {
       for (int j = (q > wu::NS ? q - wu::NS : 0); j < q; ++j)
         mbar_wait(&sm.wu_full[j % wu::NS], (j / wu::NS) & 1);
     }
-  } else if (warp == 3 && lane == 0) {
+  } else if (warp == 3) {
     // ---------------- store issuer ----------------
     // Each finished chunk leaves by TMA stores (u; the updated w and its bf16 shadow, or in
     // averaging mode at the unit's last replica the mean to replica 0); once they have read the
     // slot it goes back to the w / u producer.  Issuing stores here keeps their cost (a few
-    // hundred cycles each) off the epilogue threads.
-    int q = 0;
+    // hundred cycles each) off the epilogue threads.  One and the same elected lane issues, commits
+    // and waits for the store groups (they are a thread's own).
+    const bool el = elect_one();
+    int q = 0, sl = 0, back = 0;  // chunks stored; their slot; the slot to hand back next
+    uint32_t ph = 0;
     bool ok = true;
     for (int j = 0; j < my_count && ok; ++j) {
       const WgradUpdateLayer* ly;
@@ -1265,32 +1307,40 @@ __global__ void __launch_bounds__(wu::THREADS, 1) wgrad_update_kernel(
       const bool last = gi == per_unit - 1;
       const int nc = wu_chunks(ly->N, n0);
       for (int c = 0; c < nc; ++c, ++q) {
-        const int sl = q % wu::NS;
-        if (!mbar_wait(&sm.st_full[sl], (q / wu::NS) & 1)) {
+        if (!mbar_wait_warp(&sm.st_full[sl], ph)) {
           ok = false;
           break;
         }
-        const int x = n0 + c * wu::CW;
-        if (has_u) tma_store_3d(&ly->umap, sm.u[sl], x, m0, g);
-        if (!avg) {
-          tma_store_3d(&ly->wmap, sm.w[sl], x, m0, g);
-          if (args.sgd.wb) tma_store_3d(&ly->wbmap, sm.wb[sl], x, m0, g);
-        } else if (last) {
-          // the mean goes to replica 0 only; the runtime copies it to the other replicas when
-          // something needs them (every consumer of the next step reads replica 0)
-          tma_store_3d(&ly->wmap, sm.w[sl], x, m0, 0);
-          if (args.sgd.wb) tma_store_3d(&ly->wbmap, sm.wb[sl], x, m0, 0);
+        if (el) {
+          const int x = n0 + c * wu::CW;
+          if (has_u) tma_store_3d(&ly->umap, sm.u[sl], x, m0, g);
+          if (!avg) {
+            tma_store_3d(&ly->wmap, sm.w[sl], x, m0, g);
+            if (args.sgd.wb) tma_store_3d(&ly->wbmap, sm.wb[sl], x, m0, g);
+          } else if (last) {
+            // the mean goes to replica 0 only; the runtime copies it to the other replicas when
+            // something needs them (every consumer of the next step reads replica 0)
+            tma_store_3d(&ly->wmap, sm.w[sl], x, m0, 0);
+            if (args.sgd.wb) tma_store_3d(&ly->wbmap, sm.wb[sl], x, m0, 0);
+          }
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          // SD chunks' store groups in flight: once at most SD - 1 are still reading shared
+          // memory, the oldest one's slot goes back to the w / u producer
+          asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(wu::SD - 1) : "memory");
+          if (q >= wu::SD - 1) mbar_arrive(&sm.wu_empty[back]);
         }
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        // SD chunks' store groups in flight: once at most SD - 1 are still reading shared
-        // memory, the oldest one's slot goes back to the w / u producer
-        asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(wu::SD - 1) : "memory");
-        if (q >= wu::SD - 1) mbar_arrive(&sm.wu_empty[(q - (wu::SD - 1)) % wu::NS]);
+        if (q >= wu::SD - 1 && ++back == wu::NS) back = 0;
+        if (++sl == wu::NS) {
+          sl = 0;
+          ph ^= 1;
+        }
       }
     }
-    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-    // the last SD - 1 chunks' slots (their stores have now completed)
-    for (int j = (q > wu::SD - 1 ? q - (wu::SD - 1) : 0); j < q; ++j) mbar_arrive(&sm.wu_empty[j % wu::NS]);
+    if (el) {
+      asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+      // the last SD - 1 chunks' slots (their stores have now completed)
+      for (int j = (q > wu::SD - 1 ? q - (wu::SD - 1) : 0); j < q; ++j) mbar_arrive(&sm.wu_empty[j % wu::NS]);
+    }
   } else if (warp >= 4) {
     // ---------------- epilogue ----------------
     // The epilogue warps do not wait for one another: each waits for the accumulator and for
