@@ -104,6 +104,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
 }
 
+// A tensor map into the descriptor cache (maps are kernel parameters: no dependency on other kernels).
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
                                             int y, int z) {
   asm volatile(
@@ -239,61 +244,16 @@ __device__ __forceinline__ float warp_colsum16(float (&v)[16], int lane) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-template <int BN, int STAGES>
-struct Smem {
-  // stage buffers first (1024-byte aligned for the 128-byte swizzle)
-  uint8_t a[STAGES][BM * BK * 2];
-  uint8_t b[STAGES][BN * BK * 2];
-  uint64_t full[STAGES];
-  uint64_t empty[STAGES];
+constexpr int kTcMaxStages = 16;
+// Barriers of the one-tile kernel, behind its ring: `stages` A tiles (a_bytes each), then as many B
+// tiles, all 1024-byte aligned for the 128-byte swizzle.
+struct TcSync {
+  uint64_t full[kTcMaxStages], empty[kTcMaxStages];
   uint64_t accum;
   uint32_t tmem_base;
 };
 
 // ---- GEMM epilogue (one-tile and persistent kernels) ----
-// One thread's 32 consecutive accumulator columns of its TMEM lane, one wait.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// One thread's 64 consecutive accumulator columns of its TMEM lane: two 32-column loads, one wait.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
-  uint32_t r[64];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%64];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,"
-      "%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%65];\n"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]),
-        "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]),
-        "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]),
-        "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]),
-        "=r"(r[63])
-      : "r"(taddr), "r"(taddr + 32u)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // Sixteen consecutive outputs of one row: 32-byte stores where the row is aligned and whole, 16-byte
 // ones where it is aligned to that (a bf16 row of an odd multiple of 8 elements), else element by
 // element up to the matrix edge.  The 16-byte form took four EF-sign steps of MLP 776-520-264-17, K =
@@ -343,87 +303,94 @@ __device__ __forceinline__ void store_row16(void* C, bool c_bf16, int64_t off, i
 }
 
 // The GEMM epilogue of one 128 x BN tile for one epilogue thread: tile row et (TMEM lane et)
-// leaves TMEM CW (32 or 64) columns at a time and is written straight from registers, 16 columns
-// per store: C(m, n) at C + c_base + m c_rs + n, with bias (+ ReLU) or the ReLU mask of the stored
-// activation applied (the row's CW mask values requested before the accumulator loads).  With
-// hs_warp (bias_colsum) the stored values -- rounded to bf16 when C is bf16 -- are also summed
-// over the warp's 32 rows, per column, by a fixed butterfly (rows past M add nothing); hs_warp[c]
-// gets column c's partial.
-template <int BN, int CW>
+// leaves TMEM 16 columns at a time and is written straight from registers: C(m, n) at
+// C + c_base + m c_rs + n, with bias (+ ReLU) or the ReLU mask of the stored activation applied (the
+// next 16 mask values requested while these are used).  With hs_warp (bias_colsum) the stored values
+// -- rounded to bf16 when C is bf16 -- are also summed over the warp's 32 rows, per column, by a fixed
+// butterfly (rows past M add nothing); hs_warp[c] gets column c's partial.
+// One loop of one 16-column body: the one-tile kernel's CTAs run it once, and unrolled over a tile its
+// instructions came from memory (column sums of 128 columns: 22,000 cycles for 50 x 264, K = 5;
+// 64 columns of MLP 3072-512-512-10: 10,000; the persistent data gradients of MLP-4096 77 -> 58 us).
+template <int BN>
 __device__ __forceinline__ void epilogue_rows(const TcGemmArgs& args, int et, int lane,
                                               uint32_t tmem_acc, int g, int m0, int n0,
                                               int64_t c_base, float* hs_warp) {
-  static_assert(CW == 32 || CW == 64, "chunk width");
   const int m = m0 + et;
   const bool row_ok = m < args.M;
   const int epi = args.epi;
   const bool has_bias = epi == EPI_BIAS || epi == EPI_BIAS_RELU;
   const float* bias = has_bias ? args.bias + (int64_t)g * args.bias_gs : nullptr;
+  const bool bias_al = has_bias && (reinterpret_cast<uintptr_t>(bias + n0) & 15) == 0;
   const int64_t coff = c_base + (int64_t)m * args.c_rs;
   const int64_t moff = (int64_t)g * args.mask_gs + (int64_t)m * args.mask_rs;
-  const uint32_t lane_base = (uint32_t)(et & ~31) << 16;
-  for (int cc = 0; cc < BN; cc += CW) {
-    if (n0 + cc >= args.N) break;  // uniform over the CTA
-    const int nc = n0 + cc;
-    // the chunk's bf16 mask words (two values each) when the row is whole and 16-byte aligned
-    uint32_t mw[CW / 2];
-    const uint16_t* mrow = epi == EPI_MASK && args.mask_bf16
-                               ? reinterpret_cast<const uint16_t*>(args.mask) + moff + nc
-                               : nullptr;
-    const bool mfast = mrow && row_ok && nc + CW <= args.N &&
-                       (reinterpret_cast<uintptr_t>(mrow) & 15) == 0;
-    if (mfast) {
-#pragma unroll
-      for (int i = 0; i < CW / 8; ++i) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4*>(mrow) + i);
-        mw[4 * i] = t.x;
-        mw[4 * i + 1] = t.y;
-        mw[4 * i + 2] = t.z;
-        mw[4 * i + 3] = t.w;
-      }
+  const uint16_t* mrow = epi == EPI_MASK && args.mask_bf16
+                             ? reinterpret_cast<const uint16_t*>(args.mask) + moff + n0
+                             : nullptr;
+  const bool mal = mrow && row_ok && (reinterpret_cast<uintptr_t>(mrow) & 15) == 0;
+  const uint32_t tl = tmem_acc + ((uint32_t)(et & ~31) << 16);
+  // the mask values of 16 columns (two per word) where they are whole and aligned
+  auto load_mask = [&](int cc, uint4 (&mk)[2]) {
+    if (mal && cc < BN && n0 + cc + 16 <= args.N) {
+      mk[0] = __ldg(reinterpret_cast<const uint4*>(mrow + cc));
+      mk[1] = __ldg(reinterpret_cast<const uint4*>(mrow + cc) + 1);
     }
-    float v[CW];
-    if constexpr (CW == 64)
-      tmem_ld64(tmem_acc + lane_base + (uint32_t)cc, v);
-    else
-      tmem_ld32(tmem_acc + lane_base + (uint32_t)cc, v);
+  };
+  uint4 mk[2] = {};
+  load_mask(0, mk);
+#pragma unroll 1
+  for (int cc = 0; cc < BN; cc += 16) {
+    const int nb = n0 + cc;
+    if (nb >= args.N) break;  // uniform over the CTA
+    const bool whole = nb + 16 <= args.N;
+    float4 bv[4];
+    if (bias_al && whole) {
 #pragma unroll
-    for (int q = 0; q < CW / 16; ++q) {
-      const int nb = nc + 16 * q;
-      float x[16];
+      for (int j = 0; j < 4; ++j) bv[j] = __ldg(reinterpret_cast<const float4*>(bias + nb) + j);
+    }
+    const uint32_t mw[8] = {mk[0].x, mk[0].y, mk[0].z, mk[0].w, mk[1].x, mk[1].y, mk[1].z, mk[1].w};
+    load_mask(cc + 16, mk);
+    float x[16];
+    tmem_ld16(tl + (uint32_t)cc, x);
+    if (has_bias) {
+      if (bias_al && whole) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) x[i] = v[16 * q + i];
-      if (has_bias) {
+        for (int j = 0; j < 4; ++j) {
+          x[4 * j] += bv[j].x;
+          x[4 * j + 1] += bv[j].y;
+          x[4 * j + 2] += bv[j].z;
+          x[4 * j + 3] += bv[j].w;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] += nb + i < args.N ? __ldg(bias + nb + i) : 0.f;
+      }
+      if (epi == EPI_BIAS_RELU) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = fmaxf(x[i], 0.f);
+      }
+    } else if (epi == EPI_MASK) {
+      if (mal && whole) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          x[i] = bf2f((uint16_t)((i & 1) ? (mw[i >> 1] >> 16) : (mw[i >> 1] & 0xffffu))) > 0.f ? x[i] : 0.f;
+      } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int n = nb + i;
-          const float t = x[i] + (n < args.N ? __ldg(bias + n) : 0.f);
-          x[i] = (epi == EPI_BIAS_RELU) ? fmaxf(t, 0.f) : t;
-        }
-      } else if (epi == EPI_MASK) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float mv;
-          if (mfast) {
-            const uint32_t w = mw[8 * q + (i >> 1)];
-            mv = bf2f((uint16_t)((i & 1) ? (w >> 16) : (w & 0xffffu)));
-          } else {
-            const int n = nb + i;
-            mv = !(row_ok && n < args.N) ? 0.f
-                 : args.mask_bf16 ? bf2f(reinterpret_cast<const uint16_t*>(args.mask)[moff + n])
-                                  : reinterpret_cast<const float*>(args.mask)[moff + n];
-          }
+          const float mv = !(row_ok && n < args.N) ? 0.f
+                           : args.mask_bf16 ? bf2f(reinterpret_cast<const uint16_t*>(args.mask)[moff + n])
+                                            : reinterpret_cast<const float*>(args.mask)[moff + n];
           x[i] = mv > 0.f ? x[i] : 0.f;
         }
       }
-      if (row_ok && nb < args.N) store_row16(args.C, args.c_bf16, coff + nb, nb, args.N, x);
-      if (hs_warp) {
-        float t[16];
+    }
+    if (row_ok) store_row16(args.C, args.c_bf16, coff + nb, nb, args.N, x);
+    if (hs_warp) {
+      float t[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) t[i] = !row_ok ? 0.f : (args.c_bf16 ? bf2f(f2bf(x[i])) : x[i]);
-        const float sum = warp_colsum16(t, lane);
-        if (!(lane & 1)) hs_warp[cc + 16 * q + (lane >> 1)] = sum;
-      }
+      for (int i = 0; i < 16; ++i) t[i] = !row_ok ? 0.f : (args.c_bf16 ? bf2f(f2bf(x[i])) : x[i]);
+      const float sum = warp_colsum16(t, lane);
+      if (!(lane & 1)) hs_warp[cc + (lane >> 1)] = sum;
     }
   }
 }
@@ -479,11 +446,20 @@ __device__ __forceinline__ void bias_update(const TcGemmArgs& args, int et, int 
   }
 }
 
-template <int BN, int STAGES>
+// The ring is as deep as the reduction and the shared memory of the CTAs that share an SM allow
+// (launch_one_tile): a TMA load takes 500 (L2) to 2,400 cycles to land, so a k-block costs 2,400 / stages
+// of them.
+template <int BN>
 __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__ TcGemmArgs args) {
   extern __shared__ uint8_t smem_raw[];
-  Smem<BN, STAGES>& sm = *reinterpret_cast<Smem<BN, STAGES>*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int STAGES = args.stages;
+  // K-major A: the box's rows (a mini-batch of fewer than 128); the product reads on into what
+  // follows for the tile's other rows, which are not stored
+  const uint32_t a_bytes = args.A.mn_major ? (uint32_t)BM * BK * 2 : (uint32_t)args.A.box_rows * BK * 2;
+  constexpr uint32_t kBytesB = BN * BK * 2;
+  uint8_t* ring_b = ring + STAGES * a_bytes;
+  TcSync& sm = *reinterpret_cast<TcSync*>(ring_b + STAGES * kBytesB);
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int splits = args.splits > 1 ? args.splits : 1;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM, g = blockIdx.z / splits;
@@ -498,9 +474,10 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   const int nk = min(nk_all - kb_first, per_split);  // >= 1 (the host makes every split nonempty)
   const int64_t c_base = (int64_t)g * args.c_gs + (int64_t)split * args.c_split_stride;
   const bool a_mn = args.A.mn_major, b_mn = args.B.mn_major;
-  constexpr uint32_t kBytesA = BM * BK * 2, kBytesB = BN * BK * 2;
 
   if (threadIdx.x == 0) {
+    prefetch_map(&args.A.map);
+    prefetch_map(&args.B.map);
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], 1);
@@ -542,31 +519,28 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
           mbar_expect_tx(&sm.full[s], (uint32_t)(t1 - t0) * (BM + BN) * ck * 2);
           for (int t = t0; t < t1; ++t) {
             const int kh = t / 3, kw = t % 3, j = t - t0;
-            tma_load_5d(sm.a[s] + j * BM * ck * 2, &args.A.map, &sm.full[s], 0, kw - 1,
+            tma_load_5d(ring + s * a_bytes + j * BM * ck * 2, &args.A.map, &sm.full[s], 0, kw - 1,
                         cv_oy0 * args.cv_stride + kh - 1, cv_b0, g);
-            tma_load_3d(sm.b[s] + j * BN * ck * 2, &args.B.map, &sm.full[s], t * ck, n0, g);
+            tma_load_3d(ring_b + s * kBytesB + j * BN * ck * 2, &args.B.map, &sm.full[s], t * ck, n0, g);
           }
         }
       } else if (el) {
-        mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
+        mbar_expect_tx(&sm.full[s], a_bytes + kBytesB);
         const int k0 = (kb_first + kb) * BK;
         if (!a_mn) {
-          tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
+          tma_load_3d(ring + s * a_bytes, &args.A.map, &sm.full[s], k0, m0, g);
         } else {
 #pragma unroll
           for (int i = 0; i < BM / 64; ++i)
-            tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+            tma_load_3d(ring + s * a_bytes + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
         }
         const int gb = args.b_shared ? 0 : g;  // identical replicas: group 0's copy for all
         if (!b_mn) {
-          // K-major B: BN / box_rows boxes stacked along N (8-row swizzle atoms, rows contiguous)
-          const int brows = args.B.box_rows;
-          for (int i = 0; i < BN / brows; ++i)
-            tma_load_3d(sm.b[s] + i * brows * BK * 2, &args.B.map, &sm.full[s], k0, n0 + i * brows, gb);
+          tma_load_3d(ring_b + s * kBytesB, &args.B.map, &sm.full[s], k0, n0, gb);  // one box of BN rows
         } else {
 #pragma unroll
           for (int i = 0; i < BN / 64; ++i)
-            tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
+            tma_load_3d(ring_b + s * kBytesB + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
         }
       }
       issued = kb + 1;
@@ -586,8 +560,8 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
     constexpr uint32_t idesc_kk = make_idesc(BM, BN, false, false);
     const uint32_t idesc = idesc_kk | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16);
     // descriptors of stage 0; a stage and a 16-deep slice add their byte offsets / 16
-    const uint64_t a_desc0 = a_mn ? smem_desc(smem_u32(sm.a[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.a[0]), 16, 1024);
-    const uint64_t b_desc0 = b_mn ? smem_desc(smem_u32(sm.b[0]), 64 * BK * 2, 1024) : smem_desc(smem_u32(sm.b[0]), 16, 1024);
+    const uint64_t a_desc0 = a_mn ? smem_desc(smem_u32(ring), 64 * BK * 2, 1024) : smem_desc(smem_u32(ring), 16, 1024);
+    const uint64_t b_desc0 = b_mn ? smem_desc(smem_u32(ring_b), 64 * BK * 2, 1024) : smem_desc(smem_u32(ring_b), 16, 1024);
     const uint32_t a_step = a_mn ? 2048 >> 4 : 32 >> 4, b_step = b_mn ? 2048 >> 4 : 32 >> 4;
     int s = 0;
     uint32_t ph = 0;
@@ -599,7 +573,7 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (args.conv) {
         // each tap's sub-tiles: rows of Ck bf16 = swz bytes; K = 16 per MMA, 32 bytes further
-        const uint32_t a_base = smem_u32(sm.a[s]), b_base = smem_u32(sm.b[s]);
+        const uint32_t a_base = smem_u32(ring + s * a_bytes), b_base = smem_u32(ring_b + s * kBytesB);
         const int ck = args.cv_ck, tps = 64 / ck;
         const int nt = min(9, (kb_first + kb + 1) * tps) - (kb_first + kb) * tps;
         const uint32_t swz = (uint32_t)ck * 2;
@@ -610,7 +584,7 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
                        smem_desc_kmajor(b_base + j * BN * ck * 2 + kk * 32, swz), idesc,
                        (kb > 0 || j > 0 || kk > 0) ? 1u : 0u);
       } else {
-        const uint64_t ad = a_desc0 + (uint32_t)s * (kBytesA >> 4), bd = b_desc0 + (uint32_t)s * (kBytesB >> 4);
+        const uint64_t ad = a_desc0 + (uint32_t)s * (a_bytes >> 4), bd = b_desc0 + (uint32_t)s * (kBytesB >> 4);
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk)
           if (el) mma_bf16(tmem, ad + kk * a_step, bd + kk * b_step, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
@@ -647,9 +621,9 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   bias_prefetch<BN>(args, (int)threadIdx.x, g, n0, bsw, bsu);
   const bool have_acc = mbar_wait(&sm.accum, 0);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  float(*hs)[BN] = reinterpret_cast<float(*)[BN]>(sm.a[0]);
+  float(*hs)[BN] = reinterpret_cast<float(*)[BN]>(ring);
   if (have_acc)
-    epilogue_rows<BN, 32>(args, (int)threadIdx.x, lane, tmem, g, m0, n0, c_base,
+    epilogue_rows<BN>(args, (int)threadIdx.x, lane, tmem, g, m0, n0, c_base,
                           args.bias_colsum ? hs[warp] : nullptr);
   if (args.bias_colsum) {
     __syncthreads();  // every thread passes it, so a wait that ran out cannot split the CTA
@@ -764,9 +738,9 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
               tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
           }
           if (!b_mn) {
-            const int brows = args.B.box_rows;  // 64-row boxes stacked along N
-            for (int i = 0; i < PBN / brows; ++i)
-              tma_load_3d(sm.b[s] + i * brows * BK * 2, &args.B.map, &sm.full[s], k0, n0 + i * brows, gb);
+#pragma unroll
+            for (int i = 0; i < PBN / 64; ++i)  // 64-row boxes stacked along N
+              tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], k0, n0 + 64 * i, gb);
           } else {
 #pragma unroll
             for (int i = 0; i < PBN / 64; ++i)
@@ -851,11 +825,11 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
       if (!colsum) {
         if (!okw) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        epilogue_rows<PBN, 64>(args, et, lane, acc, g, m0, n0, (int64_t)g * args.c_gs, nullptr);
+        epilogue_rows<PBN>(args, et, lane, acc, g, m0, n0, (int64_t)g * args.c_gs, nullptr);
       } else {
         if (okw) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          epilogue_rows<PBN, 64>(args, et, lane, acc, g, m0, n0, (int64_t)g * args.c_gs,
+          epilogue_rows<PBN>(args, et, lane, acc, g, m0, n0, (int64_t)g * args.c_gs,
                                  sm.hs[ab][quarter]);
         } else if (lane == 0) {
           sm.fail = 1;
@@ -2570,23 +2544,36 @@ void load_encode() {
     cudaGetLastError();
 }
 
-template <int BN, int STAGES>
-constexpr size_t smem_bytes() {
-  return sizeof(Smem<BN, STAGES>) + 1024;
+int device_sms(int* sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  return e == cudaSuccess ? dev : -1;
 }
 
-template <int BN, int STAGES>
-cudaError_t launch_cfg(const TcGemmArgs& a, dim3 grid, cudaStream_t stream) {
-  constexpr size_t smem = smem_bytes<BN, STAGES>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, STAGES>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int BN>
+cudaError_t launch_one_tile(const TcGemmArgs& a, dim3 grid, int nk, cudaStream_t stream) {
+  int sms = 0;
+  const int dev = device_sms(&sms);
+  if (dev < 0) return cudaErrorInvalidDevice;
+  static int attr_dev = -1;
+  if (attr_dev != dev) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
     if (e != cudaSuccess) return e;
-    attr_set = true;
+    attr_dev = dev;
   }
-  launch_pdl(gemm_tc_kernel<BN, STAGES>, grid, dim3(128), smem, stream, a);
-  return cudaGetLastError();
+  // shared memory for one, two or three CTAs per SM, by what the grid gives an SM; the ring takes
+  // what it needs of it, two to sixteen stages.  (Two CTAs of four 24 KB stages whatever the grid:
+  // 64 CTAs, one per SM, took 27,700 cycles for 48 k-blocks.)
+  const int64_t ctas = (int64_t)grid.x * grid.y * grid.z;
+  const size_t budget = ctas <= sms ? 220 * 1024 : ctas <= 2 * (int64_t)sms || nk > 2 ? 112 * 1024 : 72 * 1024;
+  const size_t stage = (a.A.mn_major ? (size_t)BM : (size_t)a.A.box_rows) * BK * 2 + (size_t)BN * BK * 2;
+  const size_t fixed = 1024 + sizeof(TcSync);
+  TcGemmArgs la = a;
+  la.stages = (int)std::min<size_t>({(budget - fixed) / stage, (size_t)std::max(2, nk), (size_t)kTcMaxStages});
+  // the product's reads past a short A box stay inside the ring: B tiles follow (two at least)
+  static_assert(2 * BN * BK * 2 >= BM * BK * 2, "reads past the last A box end inside the B tiles");
+  return launch_pdl(gemm_tc_kernel<BN>, grid, dim3(128), fixed + la.stages * stage, stream, la);
 }
 
 }  // namespace
@@ -2732,12 +2719,6 @@ bool conv_tc_plan(const ConvArgs& a, int sms, int* per_sm, size_t* ring, size_t*
   return true;
 }
 
-int device_sms(int* sms) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-  return e == cudaSuccess ? dev : -1;
-}
 }  // namespace
 
 int conv_tc_ctas(const ConvArgs& a) {
@@ -3109,7 +3090,11 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
   // The TMA boxes must deliver exactly the tiles the kernel expects (expect-tx byte counts and
   // shared-memory extents depend on it).
   const int bn = tc_tile_n(a.Kd);
-  if (a.A.mn_major ? a.A.box_rows != 64 : a.A.box_rows != BM) return cudaErrorInvalidValue;
+  // (a K-major A of at most box_rows rows may come in a shorter box of whole 8-row swizzle atoms)
+  if (a.A.mn_major ? a.A.box_rows != 64
+                   : a.A.box_rows != BM && (a.A.box_rows < 8 || a.A.box_rows > BM || a.A.box_rows % 8 ||
+                                            a.M > a.A.box_rows || a.conv))
+    return cudaErrorInvalidValue;
   if (a.B.mn_major ? a.B.box_rows != 64 : a.B.box_rows != bn) return cudaErrorInvalidValue;
   if ((a.epi == EPI_BIAS || a.epi == EPI_BIAS_RELU) && !a.bias) return cudaErrorInvalidValue;
   if (a.epi == EPI_MASK && !a.mask) return cudaErrorInvalidValue;
@@ -3124,7 +3109,7 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
     if (a.M % (a.cv_hout * a.cv_wout)) return cudaErrorInvalidValue;  // whole images
     dim3 gridc((a.N + 63) / 64, (a.M + BM - 1) / BM, a.G);
     if (gridc.y > 65535) return cudaErrorInvalidValue;
-    return launch_cfg<64, 4>(a, gridc, stream);
+    return launch_one_tile<64>(a, gridc, 9, stream);
   }
   // the bias column sums need the whole mini-batch in one tile, and the masked data gradient
   if (a.bias_colsum && (a.M > BM || a.epi != EPI_MASK || (!a.bsgd.w && !a.bias_grad)))
@@ -3141,19 +3126,20 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
   static_assert(BM == kTcTileM, "tile height");
   // Short reductions (the weight gradient's k = B_loc) need only two stages; the smaller shared
   // footprint lets three CTAs share an SM so one CTA's epilogue overlaps the others' loads.
-  if ((a.Kd + BK - 1) / BK <= 2) return launch_cfg<BN, 2>(a, grid, stream);
+  if ((a.Kd + BK - 1) / BK <= 2) return launch_one_tile<BN>(a, grid, (a.Kd + BK - 1) / BK, stream);
   // Wide products (at least 2048 output columns, no split): the persistent kernel -- the forward
   // (K-major weights) and, since its epilogue prefetches the tile's ReLU mask, the data gradient
   // (MN-major weights).  Narrower layers give it too few 128 x 256 tiles to fill the SMs
   // (measured: MLP 3072-4096x3-100 forward 0.36 -> 0.27 ms per step, backward 0.333 -> 0.322 ms;
   // MLP 3072-1024-1024-10 0.29 -> 0.35 ms per step, so it stays on the one-tile kernel).
-  if (splits == 1 && a.N >= 2048 && a.B.box_rows == 64 && !gemm_pt_off())
+  if (splits == 1 && a.N >= 2048 && a.B.box_rows == 64 && (a.A.mn_major || a.A.box_rows == BM) && !gemm_pt_off())
     return launch_pt(a, stream);
   // Other long reductions: 64-wide N tiles with four stages (96 KB) so two CTAs share an SM and
   // twice as many tiles stream weights at once.
   constexpr int BN2 = 64;
   dim3 grid2((a.N + BN2 - 1) / BN2, (a.M + BM - 1) / BM, a.G * splits);
-  return launch_cfg<BN2, 4>(a, grid2, stream);
+  const int nk_all = (a.Kd + BK - 1) / BK;
+  return launch_one_tile<BN2>(a, grid2, (nk_all + splits - 1) / splits, stream);
 }
 
 }  // namespace lsgd

@@ -353,7 +353,12 @@ struct TcGemmArgs {
   // b_shared = 1 (not with conv): every group reads B from group 0 -- the replicas' weights are
   // identical (the step follows an average), so one copy serves all, mostly from L2
   int b_shared;
+  int stages;  // ring depth of the one-tile kernel (set by the launcher)
 };
+// Rows of a K-major A operand's TMA box for a product of m rows and n columns: the rows themselves
+// where they are fewer than a tile's, so that a stage of the one-tile kernel holds no padding (the
+// persistent kernel, from 2048 columns on, takes whole tiles).
+inline int tc_a_box_rows(int m, int n) { return m >= 128 || n >= 2048 ? 128 : (m + 7) / 8 * 8; }
 
 // The weight gradient of one dense layer fused with the local update, for G replicas: W[g] (M x
 // N, row stride N) -= update(dZ[g]^T act[g]) with the momentum and bf16 shadow of SgdParams.

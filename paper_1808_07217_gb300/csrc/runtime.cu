@@ -309,11 +309,11 @@ lsgd_status make_tc_maps(lsgd_ctx* c) {
     bool ok = true;
     // forward: A = act [K][B][ld_in] (K-major), B = W [K][out][in] (K-major)
     const int bn = lsgd::tc_tile_n(L.in);
+    L.fwdA.box_rows = lsgd::tc_a_box_rows(B, L.out);
     ok &= lsgd::make_tma_map_bf16(&L.fwdA.map, a_in, L.in, B, K, L.ld_in, (uint64_t)B * L.ld_in, 64,
-                                  lsgd::kTcTileM);
+                                  L.fwdA.box_rows);
     ok &= lsgd::make_tma_map_bf16(&L.fwdB.map, Wb_l, L.in, L.out, K, L.in, c->d_pad, 64, bn);
     L.fwdA.mn_major = false;
-    L.fwdA.box_rows = lsgd::kTcTileM;
     L.fwdB.mn_major = false;
     L.fwdB.box_rows = bn;
     // weight gradient: A = dZ as [K][B][out] read MN-major (M = out), B = act read MN-major (N = in)
@@ -556,12 +556,12 @@ lsgd_status dense_backward(lsgd_ctx* c, bool avg) {
         t.N = Ly.in;
         t.Kd = Ly.out;
         t.G = K;
+        t.A.box_rows = lsgd::tc_a_box_rows(B, Ly.in);
         bool ok = lsgd::make_tma_map_bf16(&t.A.map, dz, Ly.out, B, K, c->ld_dz, (uint64_t)B * c->ld_dz,
-                                          64, lsgd::kTcTileM);
+                                          64, t.A.box_rows);
         ok &= lsgd::make_tma_map_bf16(&t.B.map, c->Wb + Ly.w_off, Ly.in, Ly.out, K, Ly.in, c->d_pad, 64, 64);
         if (!ok) return fail(c, LSGD_ECUDA, "TMA map encoding failed (dgrad)");
         t.A.mn_major = false;
-        t.A.box_rows = lsgd::kTcTileM;
         t.B.mn_major = true;
         t.B.box_rows = 64;
         t.b_shared = (c->synced && K > 1) ? 1 : 0;  // identical replicas: one weight copy
@@ -1705,8 +1705,8 @@ lsgd_status lsgd_grouped_gemm_bf16(const uint16_t* A, int a_mn, const uint16_t* 
       ok = lsgd::make_tma_map_bf16(&t.A.map, A, M, Kd, G, M, (uint64_t)M * Kd, 64, 64);
       t.A.box_rows = 64;
     } else {
-      ok = lsgd::make_tma_map_bf16(&t.A.map, A, Kd, M, G, Kd, (uint64_t)M * Kd, 64, lsgd::kTcTileM);
-      t.A.box_rows = lsgd::kTcTileM;
+      t.A.box_rows = lsgd::tc_a_box_rows(M, N);
+      ok = lsgd::make_tma_map_bf16(&t.A.map, A, Kd, M, G, Kd, (uint64_t)M * Kd, 64, t.A.box_rows);
     }
     const int bn = lsgd::tc_tile_n(Kd);
     if (b_mn) {
