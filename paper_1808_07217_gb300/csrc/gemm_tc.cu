@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
     prefetch_map(&args.A.map);
     prefetch_map(&args.B.map);
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.full[s], args.conv ? 1 : 2);  // both producers
       mbar_init(&sm.empty[s], 1);
     }
     mbar_init(&sm.accum, 1);
@@ -500,13 +500,16 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   pdl_begin();  // everything above touched only shared memory and TMEM
 
   bool ok = true;
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
+  if (warp == 0 || (warp == 3 && !args.conv)) {
+    // ---------------- TMA producers: warp 0 A (of a convolution both), warp 3 B ----------------
+    // Issuing a load takes its warp about 100 cycles and a wait 150, so the operands have a warp each
+    // (with one, a k-block took 380 cycles, twice the products), and the ring's first lap no waits.
     const bool el = elect_one();
     int issued = 0, s = 0;
-    uint32_t ph = 1;
+    uint32_t ph = 1;  // of the lap before: the second lap waits for phase 0
+    const int gb = args.b_shared ? 0 : g;  // identical replicas: group 0's copy for all
     for (int kb = 0; kb < nk; ++kb) {
-      if (!mbar_wait_warp(&sm.empty[s], ph)) {
+      if (kb >= STAGES && !mbar_wait_warp(&sm.empty[s], ph)) {
         ok = false;
         break;
       }
@@ -525,22 +528,27 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
           }
         }
       } else if (el) {
-        mbar_expect_tx(&sm.full[s], a_bytes + kBytesB);
         const int k0 = (kb_first + kb) * BK;
-        if (!a_mn) {
-          tma_load_3d(ring + s * a_bytes, &args.A.map, &sm.full[s], k0, m0, g);
-        } else {
+        if (warp == 0) {
+          mbar_expect_tx(&sm.full[s], a_bytes);
+          if (!a_mn) {
+            tma_load_3d(ring + s * a_bytes, &args.A.map, &sm.full[s], k0, m0, g);
+          } else {
 #pragma unroll
-          for (int i = 0; i < BM / 64; ++i)
-            tma_load_3d(ring + s * a_bytes + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
-        }
-        const int gb = args.b_shared ? 0 : g;  // identical replicas: group 0's copy for all
-        if (!b_mn) {
-          tma_load_3d(ring_b + s * kBytesB, &args.B.map, &sm.full[s], k0, n0, gb);  // one box of BN rows
+            for (int i = 0; i < BM / 64; ++i)
+              tma_load_3d(ring + s * a_bytes + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+          }
         } else {
+          mbar_expect_tx(&sm.full[s], kBytesB);
+          if (!b_mn && args.B.box_rows == BN) {
+            tma_load_3d(ring_b + s * kBytesB, &args.B.map, &sm.full[s], k0, n0, gb);
+          } else {
+            // 64-row boxes stacked along N (K-major) or 64-wide ones (MN-major)
 #pragma unroll
-          for (int i = 0; i < BN / 64; ++i)
-            tma_load_3d(ring_b + s * kBytesB + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
+            for (int i = 0; i < BN / 64; ++i)
+              tma_load_3d(ring_b + s * kBytesB + i * 64 * BK * 2, &args.B.map, &sm.full[s],
+                          b_mn ? n0 + 64 * i : k0, b_mn ? k0 : n0 + 64 * i, gb);
+          }
         }
       }
       issued = kb + 1;
@@ -596,8 +604,8 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
       }
     }
     if (ok && el) mma_commit(&sm.accum);  // accumulator complete
-  } else if (warp >= 2 && args.epi == EPI_MASK && args.mask) {
-    // warps 2-3 idle through the mainloop: they bring the tile's ReLU-mask rows (the stored
+  } else if (warp == 2 && args.epi == EPI_MASK && args.mask) {
+    // warp 2 idles through the mainloop: it brings the tile's ReLU-mask rows (the stored
     // activation) into L1, so that the epilogue's mask loads hit L1 instead of waiting on DRAM
     // (the TMA operand loads bypass L1).  Every line prefetched starts inside the tile.
     const int esz = args.mask_bf16 ? 2 : 4;
@@ -606,7 +614,7 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
     const int rows = min(BM, args.M - m0);
     const char* base = reinterpret_cast<const char*>(args.mask) +
                        ((int64_t)g * args.mask_gs + (int64_t)m0 * args.mask_rs + n0) * esz;
-    for (int t = (int)threadIdx.x - 64; t < rows * lines; t += 64) {
+    for (int t = lane; t < rows * lines; t += 32) {
       const int r = t / lines, l = t % lines;
       asm volatile("prefetch.global.L1 [%0];" ::"l"(base + (int64_t)r * args.mask_rs * esz + l * 128));
     }
@@ -688,7 +696,7 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < PST; ++s) {
-      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.full[s], 2);  // both producers
       mbar_init(&sm.empty[s], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -712,8 +720,8 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
   const uint32_t tmem = sm.tmem_base;
   pdl_begin();  // everything above touched only shared memory and TMEM
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
+  if (warp == 0 || warp == 3) {
+    // ---------------- TMA producers: warp 0 A and the first 64 of B's columns, warp 3 the others ----------------
     const bool el = elect_one();
     int it = 0, s = 0;
     uint32_t ph = 1;
@@ -728,24 +736,23 @@ __global__ void __launch_bounds__(pt::THREADS, 1) gemm_pt_kernel(const __grid_co
           break;
         }
         if (el) {
-          mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
           const int k0 = kb * BK;
-          if (!a_mn) {
-            tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
+          if (warp == 0) {
+            mbar_expect_tx(&sm.full[s], kBytesA + kBytesB / 4);
+            if (!a_mn) {
+              tma_load_3d(sm.a[s], &args.A.map, &sm.full[s], k0, m0, g);
+            } else {
+#pragma unroll
+              for (int i = 0; i < BM / 64; ++i)
+                tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+            }
           } else {
-#pragma unroll
-            for (int i = 0; i < BM / 64; ++i)
-              tma_load_3d(sm.a[s] + i * 64 * BK * 2, &args.A.map, &sm.full[s], m0 + 64 * i, k0, g);
+            mbar_expect_tx(&sm.full[s], kBytesB / 4 * 3);
           }
-          if (!b_mn) {
-#pragma unroll
-            for (int i = 0; i < PBN / 64; ++i)  // 64-row boxes stacked along N
-              tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], k0, n0 + 64 * i, gb);
-          } else {
-#pragma unroll
-            for (int i = 0; i < PBN / 64; ++i)
-              tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], n0 + 64 * i, k0, gb);
-          }
+          // 64-row boxes stacked along N (K-major) or 64-wide ones (MN-major)
+          for (int i = warp == 0 ? 0 : 1; i < (warp == 0 ? 1 : PBN / 64); ++i)
+            tma_load_3d(sm.b[s] + i * 64 * BK * 2, &args.B.map, &sm.full[s], b_mn ? n0 + 64 * i : k0,
+                        b_mn ? k0 : n0 + 64 * i, gb);
         }
         if (++s == PST) {
           s = 0;
@@ -3095,7 +3102,7 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
                    : a.A.box_rows != BM && (a.A.box_rows < 8 || a.A.box_rows > BM || a.A.box_rows % 8 ||
                                             a.M > a.A.box_rows || a.conv))
     return cudaErrorInvalidValue;
-  if (a.B.mn_major ? a.B.box_rows != 64 : a.B.box_rows != bn) return cudaErrorInvalidValue;
+  if (a.B.mn_major ? a.B.box_rows != 64 : a.B.box_rows != bn) return cudaErrorInvalidValue;  // 64 or, short, 128
   if ((a.epi == EPI_BIAS || a.epi == EPI_BIAS_RELU) && !a.bias) return cudaErrorInvalidValue;
   if (a.epi == EPI_MASK && !a.mask) return cudaErrorInvalidValue;
   if (!a.C) return cudaErrorInvalidValue;
@@ -3134,11 +3141,12 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
   // MLP 3072-1024-1024-10 0.29 -> 0.35 ms per step, so it stays on the one-tile kernel).
   if (splits == 1 && a.N >= 2048 && a.B.box_rows == 64 && (a.A.mn_major || a.A.box_rows == BM) && !gemm_pt_off())
     return launch_pt(a, stream);
-  // Other long reductions: 64-wide N tiles with four stages (96 KB) so two CTAs share an SM and
-  // twice as many tiles stream weights at once.
+  // Other long reductions: 64-wide N tiles, one or two CTAs per SM.  (128-wide ones read the
+  // activations half as often and were no faster where they leave three SMs in four a CTA: 31.6, 16.5
+  // and 13.2 us against 31.6, 14.5 and 12.4 for the products of MLP 3072-1024-1024-10, K = 16.)
   constexpr int BN2 = 64;
-  dim3 grid2((a.N + BN2 - 1) / BN2, (a.M + BM - 1) / BM, a.G * splits);
   const int nk_all = (a.Kd + BK - 1) / BK;
+  dim3 grid2((a.N + BN2 - 1) / BN2, (a.M + BM - 1) / BM, a.G * splits);
   return launch_one_tile<BN2>(a, grid2, (nk_all + splits - 1) / splits, stream);
 }
 
