@@ -283,6 +283,8 @@ __global__ void bn_act_fwd_kernel(const float* __restrict__ y, const float* __re
   }
 }
 
+constexpr int kMergeBatch = 8;  // partials per lane requested together
+
 // The convolution epilogue's statistics partials (count, mean, M2; one per epilogue warp and CTA)
 // merged by Chan et al.'s formula: one warp per (replica, channel); lane l merges partials l,
 // l + 32, ... in order, then the fixed butterfly of bn_stats_finalize_kernel combines the lanes.
@@ -294,9 +296,16 @@ __global__ void bn_merge_partials_kernel(const float4* __restrict__ stats, int n
   const int g = wid / C, c = wid % C;
   const float4* src = stats + (int64_t)g * nparts * C + c;
   float n = 0.f, mu = 0.f, M2 = 0.f;
-  for (int q = lane; q < nparts; q += 32) {
-    const float4 v = __ldg(src + (int64_t)q * C);
-    chan_merge(n, mu, M2, v.x, v.y, v.z);
+  // a batch of loads at a time, merged in order (one after another, eight round trips took 7.3 us
+  // for 240 partials)
+  for (int q0 = lane; q0 < nparts; q0 += 32 * kMergeBatch) {
+    float4 v[kMergeBatch];
+#pragma unroll
+    for (int i = 0; i < kMergeBatch; ++i)
+      v[i] = q0 + 32 * i < nparts ? __ldg(src + (int64_t)(q0 + 32 * i) * C) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kMergeBatch; ++i)
+      if (q0 + 32 * i < nparts) chan_merge(n, mu, M2, v[i].x, v[i].y, v[i].z);
   }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -525,10 +534,18 @@ __global__ void bn_bwd_merge_kernel(const float2* __restrict__ part, int nparts,
   if (wid >= G * C) return;
   const int g = wid / C, c = wid % C;
   float a = 0.f, b = 0.f;
-  for (int q = lane; q < nparts; q += 32) {
-    const float2 v = part[((int64_t)g * nparts + q) * C + c];
-    a += v.x;
-    b += v.y;
+  for (int q0 = lane; q0 < nparts; q0 += 32 * kMergeBatch) {
+    float2 v[kMergeBatch];
+#pragma unroll
+    for (int i = 0; i < kMergeBatch; ++i)
+      v[i] = q0 + 32 * i < nparts ? __ldg(part + ((int64_t)g * nparts + q0 + 32 * i) * C + c)
+                                  : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kMergeBatch; ++i)
+      if (q0 + 32 * i < nparts) {
+        a += v[i].x;
+        b += v[i].y;
+      }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -829,8 +846,31 @@ unsigned sum_partials_grid(int64_t n) { return (unsigned)((n + 31) / 32); }
 
 // The same sum for four consecutive outputs per thread (float4 loads and store), partials added in
 // split order q = 0, 1, ...: for column counts, leading dimensions, tap widths and destinations
-// that keep every group of four outputs contiguous and 16-byte aligned (sum_partials_v4_ok).
-__global__ void __launch_bounds__(256) sum_partials_v4_kernel(
+// that keep every group of four outputs contiguous and 16-byte aligned (sum_partials_v4_ok).  One
+// layer's sum has sixteen loads in flight and small CTAs, so that few outputs still use many SMs (7.8 ->
+// 7.0 us for 60 partials of 23,040 outputs); the whole network's (below) has the threads, and four
+// loads each are faster there (44 against 56 us).
+constexpr int kSumThreads = 64;
+template <int kSumBatch>
+__device__ __forceinline__ float4 sum_in_order(const float* p, int64_t qs, int nq) {
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int q0 = 0; q0 < nq; q0 += kSumBatch) {
+    float4 v[kSumBatch];
+#pragma unroll
+    for (int i = 0; i < kSumBatch; ++i)
+      if (q0 + i < nq) v[i] = __ldg(reinterpret_cast<const float4*>(p + (int64_t)(q0 + i) * qs));
+#pragma unroll
+    for (int i = 0; i < kSumBatch; ++i)
+      if (q0 + i < nq) {
+        acc.x += v[i].x;
+        acc.y += v[i].y;
+        acc.z += v[i].z;
+        acc.w += v[i].w;
+      }
+  }
+  return acc;
+}
+__global__ void __launch_bounds__(kSumThreads) sum_partials_v4_kernel(
     const float* __restrict__ part, int nq, int rows, int ldc, int cols, int G,
     float* __restrict__ out, int64_t out_gs, int tap_src, int tap_dst) {
   pdl_begin();
@@ -842,16 +882,7 @@ __global__ void __launch_bounds__(256) sum_partials_v4_kernel(
   const int g = (int)(t / ((int64_t)rows * (cols / 4)));
   const int js = tap_dst > 0 ? (j / tap_dst) * tap_src + j % tap_dst : j;
   const float* p = part + (int64_t)g * nq * rows * ldc + (int64_t)r * ldc + js;
-  const int64_t qs = (int64_t)rows * ldc;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-  for (int q = 0; q < nq; ++q) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p + q * qs));
-    acc.x += v.x;
-    acc.y += v.y;
-    acc.z += v.z;
-    acc.w += v.w;
-  }
+  const float4 acc = sum_in_order<16>(p, (int64_t)rows * ldc, nq);
   *reinterpret_cast<float4*>(out + (int64_t)g * out_gs + (int64_t)r * cols + j) = acc;
 }
 
@@ -893,16 +924,7 @@ __global__ void __launch_bounds__(256) sum_partials_jobs_v4_kernel(const __grid_
   const int g = (int)(t / ((int64_t)jb.rows * c4));
   const int js_ = jb.tap_dst > 0 ? (j / jb.tap_dst) * jb.tap_src + j % jb.tap_dst : j;
   const float* pp = jb.part + (int64_t)g * jb.nq * jb.rows * jb.ldc + (int64_t)r * jb.ldc + js_;
-  const int64_t qs = (int64_t)jb.rows * jb.ldc;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-  for (int q = 0; q < jb.nq; ++q) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(pp + q * qs));
-    acc.x += v.x;
-    acc.y += v.y;
-    acc.z += v.z;
-    acc.w += v.w;
-  }
+  const float4 acc = sum_in_order<4>(pp, (int64_t)jb.rows * jb.ldc, jb.nq);
   *reinterpret_cast<float4*>(jb.out + (int64_t)g * jb.out_gs + (int64_t)r * jb.cols + j) = acc;
 }
 
@@ -911,7 +933,7 @@ void launch_sum_partials(const float* part, int nq, int rows, int ldc, int cols,
                          int64_t out_gs, int tap_src, int tap_dst, cudaStream_t s) {
   if (sum_partials_v4_ok(part, ldc, cols, out, out_gs, tap_src, tap_dst)) {
     const int64_t n4 = (int64_t)G * rows * (cols / 4);
-    launch_pdl(sum_partials_v4_kernel, (unsigned)((n4 + 255) / 256), 256, 0, s, part, nq, rows, ldc,
+    launch_pdl(sum_partials_v4_kernel, (unsigned)((n4 + kSumThreads - 1) / kSumThreads), kSumThreads, 0, s, part, nq, rows, ldc,
                cols, G, out, out_gs, tap_src, tap_dst);
   } else {
     launch_pdl(sum_partials_crop_kernel, sum_partials_grid((int64_t)G * rows * cols),
@@ -1004,31 +1026,39 @@ struct FlipJobs {
   FlipJob j[kMaxFlipJobs];
 };
 
-__global__ void flip_jobs_kernel(const uint16_t* __restrict__ Wb, int64_t d_pad, int G,
-                                 const __grid_constant__ FlipJobs js, int64_t total) {
+// One 16-byte group of eight output channels per thread, consecutive threads on consecutive input
+// channels (one element per thread with 64-bit divisions: 60 us for ResNet-20 x 16 workers, 11 so).
+__global__ void __launch_bounds__(256) flip_jobs_kernel(const uint16_t* __restrict__ Wb, int64_t d_pad, int G,
+                                                        const __grid_constant__ FlipJobs js, int total8) {
   pdl_begin();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total8; t += gridDim.x * blockDim.x) {
     int k = 0;
-    while (k + 1 < js.n && t >= js.j[k + 1].begin) ++k;
+    while (k + 1 < js.n && (int64_t)t * 8 >= js.j[k + 1].begin) ++k;
     const FlipJob& jb = js.j[k];
-    const int64_t e = t - jb.begin;
-    const int Cin = jb.cin, Cout = jb.cout;
-    const int64_t per = (int64_t)Cin * 9 * Cout;
-    const int co = (int)(e % Cout), tp = (int)((e / Cout) % 9), ci = (int)((e / (9 * Cout)) % Cin);
-    const int64_t gp = e / per;
-    if (!jb.phases) {
-      const int g = (int)gp;
-      jb.dst[e] = Wb[(int64_t)g * d_pad + jb.w_off + ((int64_t)co * 9 + (8 - tp)) * Cin + ci];
-    } else {
-      const int g = (int)(gp % G), ph = (int)(gp / G);
-      const int dr = tp / 3 - 1, dc = tp % 3 - 1;
-      const int kh = (ph >> 1) + 1 - 2 * dr, kw = (ph & 1) + 1 - 2 * dc;
-      uint16_t v = 0;
-      if (kh >= 0 && kh <= 2 && kw >= 0 && kw <= 2)
-        v = Wb[(int64_t)g * d_pad + jb.w_off + (((int64_t)co * 3 + kh) * 3 + kw) * Cin + ci];
-      jb.dst[e] = v;
+    int e = t - (int)(jb.begin / 8);  // (phase, replica, tap, channel group, input channel)
+    const int Cin = jb.cin, c8 = jb.cout / 8;
+    const int ci = e % Cin;
+    e /= Cin;
+    const int co = (e % c8) * 8;
+    e /= c8;
+    const int tp = e % 9, gp = e / 9;
+    const int g = jb.phases ? gp % G : gp, ph = jb.phases ? gp / G : 0;
+    const uint16_t* src = Wb + (int64_t)g * d_pad + jb.w_off;
+    int tap = 8 - tp;
+    bool any = true;
+    if (jb.phases) {
+      const int kh = (ph >> 1) + 1 - 2 * (tp / 3 - 1), kw = (ph & 1) + 1 - 2 * (tp % 3 - 1);
+      any = kh >= 0 && kh <= 2 && kw >= 0 && kw <= 2;
+      tap = 3 * kh + kw;
     }
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (any) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        w[i >> 1] |= (uint32_t)__ldg(src + ((co + i) * 9 + tap) * Cin + ci) << (16 * (i & 1));
+    }
+    *reinterpret_cast<uint4*>(jb.dst + (((int64_t)gp * Cin + ci) * 9 + tp) * jb.cout + co) =
+        make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -2052,16 +2082,16 @@ lsgd_status flip_all(ResNetPlan* p, const void* Wop, cudaStream_t s, int64_t* la
   int64_t total = 0;
   auto flush = [&]() -> lsgd_status {
     if (total > 0)
-      RN_LAUNCH((launch_pdl(flip_jobs_kernel, grid_cap(total, 256), 256, 0, s,
-                            reinterpret_cast<const uint16_t*>(Wop), p->d_pad, p->K, js, total)));
+      RN_LAUNCH((launch_pdl(flip_jobs_kernel, grid_cap(total / 8, 256), 256, 0, s,
+                            reinterpret_cast<const uint16_t*>(Wop), p->d_pad, p->K, js, (int)(total / 8))));
     js = FlipJobs{};
     total = 0;
     return LSGD_OK;
   };
   for (size_t i = 0; i < p->wflip.size(); ++i) {
     if (!p->wflip[i]) continue;
-    if (js.n == kMaxFlipJobs) {
-      const lsgd_status st = flush();  // a deeper network: one launch per table
+    if (js.n == kMaxFlipJobs || total > (1LL << 30)) {
+      const lsgd_status st = flush();  // a deeper or wider network: one launch per table
       if (st != LSGD_OK) return st;
     }
     const ConvL& c = p->convs[i];
