@@ -65,6 +65,17 @@ __device__ __forceinline__ void sgd_elem(float& w, float& u, float g, float lr, 
   w = fmaf(-lr, st, w);
 }
 
+// The same with the variant chosen at run time.
+__device__ __forceinline__ void sgd_elem_any(float& w, float& u, float g, float lr, float m, float lam,
+                                             bool nest, bool sgn) {
+  if (m == 0.f)
+    sgd_elem<false, false>(w, u, g, lr, 0.f, lam, sgn);
+  else if (nest)
+    sgd_elem<true, true>(w, u, g, lr, m, lam, sgn);
+  else
+    sgd_elem<true, false>(w, u, g, lr, m, lam, sgn);
+}
+
 // The K-way average's arithmetic (Eq. 2 right), shared by the stand-alone average and the
 // weight-gradient + update + average kernel so that both give the same bits.  Replicas are added
 // in order with Knuth's error-free TwoSum (s + x = t + e exactly) and the errors summed in c;

@@ -150,7 +150,7 @@ template <typename TD>
 __global__ void __launch_bounds__(1024) softmax_xent_kernel(
     const float* __restrict__ logits, int ld, int C, const int32_t* __restrict__ labels, int B,
     TD* __restrict__ dz, int ld_dz, float* __restrict__ loss_mean, float* __restrict__ loss_sum,
-    float* __restrict__ row_out) {
+    float* __restrict__ row_out, const __grid_constant__ LogitParts parts) {
   pdl_begin();
   extern __shared__ float row_loss[];  // [B]
   const int g = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -169,8 +169,23 @@ __global__ void __launch_bounds__(1024) softmax_xent_kernel(
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int c = lane + 32 * i;
-          zv[r][i] = (j < B && c < C) ? z[c] : -INFINITY;
+          zv[r][i] = (j < B && c < C && !parts.splits) ? z[c] : -INFINITY;
         }
+      }
+      if (parts.splits && j0 < B && lane < C) {
+        // the logits' partial products (one row to a warp), sixteen splits requested at a time
+        const float* p = parts.part + (int64_t)g * parts.part_gs + (int64_t)j0 * parts.part_rs + lane;
+        float v = 0.f;
+        for (int s0 = 0; s0 < parts.splits; s0 += 16) {
+          float q[16];
+#pragma unroll
+          for (int s = 0; s < 16; ++s)
+            q[s] = s0 + s < parts.splits ? p[(int64_t)(s0 + s) * parts.part_ss] : 0.f;
+#pragma unroll
+          for (int s = 0; s < 16; ++s)
+            if (s0 + s < parts.splits) v += q[s];
+        }
+        zv[0][0] = v + (parts.bias ? parts.bias[(int64_t)g * parts.bias_gs + lane] : 0.f);
       }
 #pragma unroll
       for (int r = 0; r < RPW; ++r) {
@@ -347,6 +362,94 @@ __global__ void __launch_bounds__(256) colsum_kernel(const TD* __restrict__ dz, 
         if (sgd.u) sgd.u[i] = u;
         if (sgd.wb) sgd.wb[i] = f2bf(w);
       }
+    }
+  }
+}
+
+// A narrow fp32 top layer's update (softmax regression's whole backward): one thread per input column with
+// all its outputs' sums, its column of the activations loaded sixteen rows ahead; block 0 of a replica also
+// sums the bias as colsum_kernel does.  The chains are those of the GEMM, the column sums and the update
+// that it replaces, so the bits are too.  Bound by latency: those three launches took 4.3, 2.1 and 2.6 us
+// and their gaps for 10 x 3072 of 32 rows, K = 4 (a step of softmax regression 34 -> 27 us with the loss
+// kernel's own sums of the split logits); this one takes 6.3.
+constexpr int kNarrowThreads = 128;
+__global__ void __launch_bounds__(kNarrowThreads) narrow_update_kernel(
+    const float* __restrict__ dz, int ld_dz, const float* __restrict__ act, int ld_act, int B, int out,
+    int in, int64_t gs, int64_t w_off, int64_t b_off, SgdParams sgd) {
+  pdl_begin();
+  extern __shared__ float dzs[];  // [B][kNarrowMaxOut]
+  __shared__ float part[8][kNarrowMaxOut];
+  const int g = blockIdx.y, t = threadIdx.x, i = blockIdx.x * kNarrowThreads + t;
+  const float* a = act + (int64_t)g * B * ld_act + i;
+  constexpr int NB = 16;
+  float x[NB];
+#pragma unroll
+  for (int r = 0; r < NB; ++r) x[r] = i < in && r < B ? a[(int64_t)r * ld_act] : 0.f;
+  for (int e = t; e < B * kNarrowMaxOut; e += kNarrowThreads) {
+    const int j = e / kNarrowMaxOut, o = e % kNarrowMaxOut;
+    dzs[e] = o < out ? dz[((int64_t)g * B + j) * ld_dz + o] : 0.f;
+  }
+  __syncthreads();
+  const bool mom = sgd.mom != 0.f;
+  auto apply = [&](int64_t k, float w, float u, float gr) {
+    sgd_elem_any(w, u, gr, sgd.lr, sgd.mom, sgd.wd, sgd.nesterov != 0, sgd.sign != 0);
+    sgd.w[k] = w;
+    if (mom) sgd.u[k] = u;
+  };
+  // what the update reads is requested before the sums (behind them, between stores that may alias, each
+  // element would wait for its own round trip: 7.7 us)
+  const int64_t wk = (int64_t)g * gs + w_off + i;
+  float wv[kNarrowMaxOut], uv[kNarrowMaxOut];
+#pragma unroll
+  for (int o = 0; o < kNarrowMaxOut; ++o) {
+    const bool in_range = i < in && o < out;
+    wv[o] = in_range ? sgd.w[wk + (int64_t)o * in] : 0.f;
+    uv[o] = in_range && mom ? sgd.u[wk + (int64_t)o * in] : 0.f;
+  }
+  float acc[kNarrowMaxOut];
+#pragma unroll
+  for (int o = 0; o < kNarrowMaxOut; ++o) acc[o] = 0.f;
+  for (int j0 = 0; j0 < B; j0 += NB) {
+    float c[NB];
+#pragma unroll
+    for (int r = 0; r < NB; ++r) {
+      c[r] = x[r];
+      const int j = j0 + NB + r;
+      x[r] = i < in && j < B ? a[(int64_t)j * ld_act] : 0.f;
+    }
+#pragma unroll
+    for (int r = 0; r < NB; ++r) {
+      if (j0 + r >= B) break;
+      const float4* d = reinterpret_cast<const float4*>(dzs + (j0 + r) * kNarrowMaxOut);
+#pragma unroll
+      for (int q = 0; q < kNarrowMaxOut / 4; ++q) {
+        if (4 * q >= out) break;
+        const float4 v = d[q];
+        acc[4 * q] = fmaf(v.x, c[r], acc[4 * q]);
+        acc[4 * q + 1] = fmaf(v.y, c[r], acc[4 * q + 1]);
+        acc[4 * q + 2] = fmaf(v.z, c[r], acc[4 * q + 2]);
+        acc[4 * q + 3] = fmaf(v.w, c[r], acc[4 * q + 3]);
+      }
+    }
+  }
+  if (i < in) {
+#pragma unroll
+    for (int o = 0; o < kNarrowMaxOut; ++o)
+      if (o < out) apply(wk + (int64_t)o * in, wv[o], uv[o], acc[o]);
+  }
+  if (blockIdx.x == 0) {
+    // bias: eight row slices, then the slices in order
+    const int o = t % kNarrowMaxOut, sl = t / kNarrowMaxOut;
+    float s = 0.f;
+    for (int j = sl; j < B; j += 8) s += dzs[j * kNarrowMaxOut + o];
+    part[sl][o] = s;
+    __syncthreads();
+    if (sl == 0 && o < out) {
+      float b = 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) b += part[q][o];
+      const int64_t k = (int64_t)g * gs + b_off + o;
+      apply(k, sgd.w[k], mom ? sgd.u[k] : 0.f, b);
     }
   }
 }
@@ -771,21 +874,23 @@ cudaError_t launch_gather_rows(void* dst, bool dst_bf16, int ld_dst, const float
 
 cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_t* labels, int G,
                                 int B, void* dz, bool dz_bf16, int ld_dz, float* loss_mean,
-                                float* loss_sum, float* row_loss, cudaStream_t stream) {
+                                float* loss_sum, float* row_loss, cudaStream_t stream,
+                                const LogitParts& parts) {
   if (G <= 0 || B <= 0) return cudaSuccess;
-  if (B > 8192 || C < 1) return cudaErrorInvalidValue;
+  if (B > 8192 || C < 1 || (parts.splits && (C > 32 || B > 32 || !parts.part))) return cudaErrorInvalidValue;
   // one warp per row, up to 32 warps (8 for at most 32 classes, where a row is one pass of a
-  // warp and the block's reduction barriers would dominate); the row losses in shared memory
-  const int threads = 32 * std::min(C > 32 ? 32 : 8, B);
+  // warp and the block's reduction barriers would dominate; 32 where each row is first summed from its
+  // partial products)
+  const int threads = 32 * std::min(C > 32 || parts.splits ? 32 : 8, B);
   const size_t smem = (size_t)B * sizeof(float);
   if (dz_bf16)
     launch_pdl(softmax_xent_kernel<uint16_t>, G, threads, smem, stream,
         logits, ld, C, labels, B, reinterpret_cast<uint16_t*>(dz), ld_dz, loss_mean, loss_sum,
-        row_loss);
+        row_loss, parts);
   else
     launch_pdl(softmax_xent_kernel<float>, G, threads, smem, stream,
         logits, ld, C, labels, B, reinterpret_cast<float*>(dz), ld_dz, loss_mean, loss_sum,
-        row_loss);
+        row_loss, parts);
   return cudaGetLastError();
 }
 
@@ -842,6 +947,29 @@ cudaError_t launch_colsum_update(const void* dz, bool dz_bf16, int ld, int G, in
   else
     launch_pdl(colsum_kernel<float, true>, grid, block, 0, stream, reinterpret_cast<const float*>(dz), ld, B,
                                                            out, nullptr, gs, sgd);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_narrow_update(const float* dz, int ld_dz, const float* act, int ld_act, int G, int B,
+                                 int out, int in, int64_t gs, int64_t w_off, int64_t b_off,
+                                 const SgdParams& sgd, cudaStream_t stream) {
+  if (G <= 0 || out <= 0 || in <= 0) return cudaSuccess;
+  if (out > kNarrowMaxOut || B < 1 || B > kNarrowMaxRows || G > 65535 || !sgd.w ||
+      (sgd.mom != 0.f && !sgd.u))
+    return cudaErrorInvalidValue;
+  const size_t smem = (size_t)B * kNarrowMaxOut * sizeof(float);
+  static int attr_dev = -1;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (attr_dev != dev) {
+    e = cudaFuncSetAttribute(narrow_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kNarrowMaxRows * kNarrowMaxOut * 4);
+    if (e != cudaSuccess) return e;
+    attr_dev = dev;
+  }
+  launch_pdl(narrow_update_kernel, dim3((in + kNarrowThreads - 1) / kNarrowThreads, G), kNarrowThreads, smem,
+             stream, dz, ld_dz, act, ld_act, B, out, in, gs, w_off, b_off, sgd);
   return cudaGetLastError();
 }
 

@@ -56,9 +56,27 @@ cudaError_t launch_gather_rows(void* dst, bool dst_bf16, int ld_dst, const float
 // Softmax cross-entropy over logits [G][B][ld]; dz = (softmax - onehot) / B into [G][B][ld_dz]
 // (skipped when dz == NULL); loss_mean[g] = mean row loss, loss_sum[g] = sum, row_loss[g B + j]
 // = row loss (each may be NULL).
+// With parts (C and B at most 32) the logits come as split partial products instead, added in split order as the
+// kernels that would have summed them do: sum over s of part[g part_gs + s part_ss + j part_rs + c], plus
+// bias[g bias_gs + c].
+struct LogitParts {
+  const float* part;
+  int splits;  // 0: none
+  int64_t part_gs, part_ss, part_rs;
+  const float* bias;
+  int64_t bias_gs;
+};
 cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_t* labels, int G,
                                 int B, void* dz, bool dz_bf16, int ld_dz, float* loss_mean,
-                                float* loss_sum, float* row_loss, cudaStream_t stream);
+                                float* loss_sum, float* row_loss, cudaStream_t stream,
+                                const LogitParts& parts = {});
+// A narrow fp32 top layer's local update (out <= 16, at most kNarrowMaxRows rows): the gradients
+// gW[o][i] = sum over j of dz[g][j][o] act[g][j][i] in row order and gb[o] as launch_colsum's, applied as
+// launch_sgd_update would to replica g's w_off / b_off within sgd.w and sgd.u (replica stride gs).
+constexpr int kNarrowMaxOut = 16, kNarrowMaxRows = 1024;
+cudaError_t launch_narrow_update(const float* dz, int ld_dz, const float* act, int ld_act, int G, int B,
+                                 int out, int in, int64_t gs, int64_t w_off, int64_t b_off,
+                                 const SgdParams& sgd, cudaStream_t stream);
 // Least squares: z [G][B][ld] (column 0), r = z - t; loss = r^2 / 2; dz = r / B.
 cudaError_t launch_lsq_loss(const float* z, int ld, const float* targets, int G, int B, void* dz,
                             bool dz_bf16, int ld_dz, float* loss_mean, float* loss_sum,
@@ -120,7 +138,8 @@ enum GemmEpilogue {
   EPI_STORE = 0,      // C = acc
   EPI_BIAS = 1,       // C = acc + bias[n]
   EPI_BIAS_RELU = 2,  // C = max(acc + bias[n], 0)
-  EPI_MASK = 3        // C = mask(m, n) > 0 ? acc : 0   (ReLU derivative from the stored activation)
+  EPI_MASK = 3,       // C = mask(m, n) > 0 ? acc : 0   (ReLU derivative from the stored activation)
+  EPI_SGD = 4         // launch_gemm_simt, fp32: the local update with gradient acc, through GemmArgs::sgd
 };
 
 struct GemmArgs {
@@ -147,6 +166,8 @@ struct GemmArgs {
   bool bias_colsum;
   SgdParams bsgd;
   float* bias_grad;
+  // EPI_SGD: the parameters (and momentum) where C's layout has its elements; C and ws are not used
+  SgdParams sgd;
   // implicit 3x3 convolution (zero padding 1): C[p][n] = sum over taps t and k < cv_ck of
   // in[shift_t(p)][k] B[n][t][k].  A is a rank-5 map over the NHWC input {cv_ck, W, H, B, G} whose
   // box is {cv_ck, Wout * s, rows * s, images, 1} with element strides {1, s, s, 1, 1}; B a rank-3
@@ -159,6 +180,9 @@ struct GemmArgs {
   // ws[g][split][m][n] and a second kernel adding them in split order before the epilogue
   float* ws;
   int64_t ws_floats;
+  // non-null (EPI_BIAS): a product that is split leaves its partial sums in ws, unsummed and without the
+  // bias, and *splits_left is their number (1: C is complete)
+  int* splits_left;
 };
 // Persistent implicit-GEMM 3x3 convolution (zero padding 1): out[g][p][n] (fp32, replica stride
 // out_gs) = sum over taps t and k < ck of in[g][shift_t(p)][k] w[g][n][t][k].  in_map: the rank-5

@@ -331,7 +331,7 @@ lsgd_status make_tc_maps(lsgd_ctx* c) {
 // nothing between its own backward and that launch reads its weights (the layers below read only
 // theirs), so the result is the same.
 bool defer_top_update(const lsgd_ctx* c) {
-  return c->fused && !c->head && c->layers.size() >= 3;
+  return c->fused && c->bf16 && !c->head && c->layers.size() >= 3;
 }
 
 lsgd_status alloc_dense(lsgd_ctx* c) {
@@ -377,7 +377,11 @@ lsgd_status tc_gemm(lsgd_ctx* c, const lsgd::TcGemmArgs& g) {
 }
 
 // Forward of every dense layer for `groups` groups.  Weights come from replica (w_g0 + g * w_gmul).
-lsgd_status dense_forward(lsgd_ctx* c, int groups, int w_g0, int w_gmul, bool skip_last = false) {
+// parts (optional): the top layer's product may stay in split partial sums, described there, for the
+// loss kernel to add: where each of its warps has one row of at most 32 logits, 8.0 us for both against
+// 4.3 + 7.0 (K = 4, 24 splits; with 256 rows it is 13.4 against 4.3 + 8, the sums being one CTA's).
+lsgd_status dense_forward(lsgd_ctx* c, int groups, int w_g0, int w_gmul, bool skip_last = false,
+                          lsgd::LogitParts* parts = nullptr) {
   const int B = c->cfg.B_loc;
   const int L = (int)c->layers.size();
   const void* Wop = c->bf16 ? (const void*)c->Wb : (const void*)c->W;
@@ -450,11 +454,23 @@ lsgd_status dense_forward(lsgd_ctx* c, int groups, int w_g0, int w_gmul, bool sk
     g.bias_gs = (int64_t)w_gmul * c->d_pad;
     g.ws = c->simt_ws;
     g.ws_floats = c->simt_ws_floats;
+    int left = 1;
+    if (parts && last && epi == lsgd::EPI_BIAS && Ly.out <= 32 && B <= 32) g.splits_left = &left;
     lsgd_status st = gemm(c, g);
     if (st != LSGD_OK) return st;
+    if (left > 1)
+      *parts = lsgd::LogitParts{c->simt_ws, left, (int64_t)left * B * Ly.out, (int64_t)B * Ly.out, Ly.out,
+                                g.bias, g.bias_gs};
   }
   (void)esz;
   return LSGD_OK;
+}
+
+// The top layer's update runs on narrow_update_kernel.
+bool narrow_top(const lsgd_ctx* c) {
+  const DenseLayer& top = c->layers.back();
+  return !c->bf16 && !c->lsq && top.b_off >= 0 && top.out <= lsgd::kNarrowMaxOut &&
+         c->cfg.B_loc <= lsgd::kNarrowMaxRows;
 }
 
 // The classifier-head kernels' view of the last layer (forward + loss and backward share it).
@@ -545,6 +561,8 @@ lsgd_status dense_backward(lsgd_ctx* c, bool avg) {
   for (int l = l_top; l >= 0; --l) {
     const DenseLayer& Ly = c->layers[l];
     const void* dz = c->dz[cur];
+    // a narrow fp32 top layer: both its gradients and their update in one launch
+    const bool narrow = l == L - 1 && narrow_top(c);
     // read before this layer's data gradient sets bias_done for the layer below
     const bool bias_by_dgrad_above = bias_done == l;
     if (l > 0) {
@@ -619,7 +637,12 @@ lsgd_status dense_backward(lsgd_ctx* c, bool avg) {
       span(LSGD_PH_BACKWARD);
     }
     // weight gradient G_W[o][i] = sum_j dz[j][o] act[j][i] (or, fused, the update it drives)
-    if (Ly.tc) {
+    if (narrow) {
+      LSGD_LAUNCH(c, lsgd::launch_narrow_update((const float*)dz, c->ld_dz, (const float*)c->act[l],
+                                                Ly.ld_in, K, B, Ly.out, Ly.in, c->d_pad, Ly.w_off,
+                                                Ly.b_off, sgd_at(0), c->stream));
+      span(LSGD_PH_UPDATE);
+    } else if (Ly.tc) {
       lsgd::TcGemmArgs t{};
       t.M = Ly.out;
       t.N = Ly.in;
@@ -702,13 +725,14 @@ lsgd_status dense_backward(lsgd_ctx* c, bool avg) {
       g.c_rs = Ly.in;
       g.c_gs = c->d_pad;
       g.c_bf16 = false;
-      g.epi = lsgd::EPI_STORE;
+      g.epi = c->fused ? lsgd::EPI_SGD : lsgd::EPI_STORE;
+      if (c->fused) g.sgd = sgd_at(Ly.w_off);
       lsgd_status st = gemm(c, g);
       if (st != LSGD_OK) return st;
       span(LSGD_PH_UPDATE);
     }
     // the bias sums: unless the head's kernel (layer L - 2) or the data-gradient GEMM above did them
-    if (Ly.b_off >= 0 && !(c->head && l == L - 2) && !bias_by_dgrad_above) {
+    if (Ly.b_off >= 0 && !narrow && !(c->head && l == L - 2) && !bias_by_dgrad_above) {
       if (c->fused)
         LSGD_LAUNCH(c, lsgd::launch_colsum_update(dz, c->bf16, c->ld_dz, K, B, Ly.out, c->d_pad,
                                                   sgd_at(Ly.b_off), c->stream));
@@ -724,7 +748,8 @@ lsgd_status dense_backward(lsgd_ctx* c, bool avg) {
 }
 
 // Loss of the last layer's output for `groups` groups; dz into dz[0] unless eval.
-lsgd_status dense_loss(lsgd_ctx* c, int groups, bool eval, float* loss_mean) {
+lsgd_status dense_loss(lsgd_ctx* c, int groups, bool eval, float* loss_mean,
+                       const lsgd::LogitParts& parts = {}) {
   const int B = c->cfg.B_loc;
   void* dz = eval ? nullptr : c->dz[0];
   if (c->lsq) {
@@ -733,7 +758,7 @@ lsgd_status dense_loss(lsgd_ctx* c, int groups, bool eval, float* loss_mean) {
   } else {
     LSGD_LAUNCH(c, lsgd::launch_softmax_xent(c->logits, c->ld_logits, c->C, c->yb, groups, B, dz,
                                              c->bf16, c->ld_dz, loss_mean, nullptr, c->row_loss,
-                                             c->stream));
+                                             c->stream, parts));
   }
   return LSGD_OK;
 }
@@ -750,7 +775,7 @@ lsgd_status do_update(lsgd_ctx* c) {
 // Whether a step that ends with the global average can run it inside its update launches:
 // dense bf16 model with the fused update on the tensor cores, plain averaging.
 bool can_fuse_average(const lsgd_ctx* c) {
-  return c->fused && !c->resnet && c->cfg.compress == LSGD_COMPRESS_NONE &&
+  return c->fused && c->bf16 && c->cfg.compress == LSGD_COMPRESS_NONE &&
          c->cfg.global_momentum <= 0.0;
 }
 
@@ -771,7 +796,8 @@ lsgd_status step_body(lsgd_ctx* c, int64_t e_start, bool avg = false) {
     e_bwd = prof_mark(c);
     prof_span(c, LSGD_PH_FORWARD, e_in, e_bwd);
   } else {
-    st = dense_forward(c, K, 0, 1, c->head);
+    lsgd::LogitParts parts{};
+    st = dense_forward(c, K, 0, 1, c->head, &parts);
     if (st != LSGD_OK) return st;
     const int64_t e_fwd = prof_mark(c);
     prof_span(c, LSGD_PH_FORWARD, e_in, e_fwd);
@@ -784,7 +810,7 @@ lsgd_status step_body(lsgd_ctx* c, int64_t e_start, bool avg = false) {
       LSGD_LAUNCH(c, lsgd::launch_head_forward(h, c->stream));
       c->loss_slot_now = loss_slot;
     } else {
-      st = dense_loss(c, K, false, loss_slot);
+      st = dense_loss(c, K, false, loss_slot, parts);
     }
     if (st != LSGD_OK) return st;
     const int64_t e_loss = prof_mark(c);
@@ -986,9 +1012,10 @@ lsgd_status lsgd_create(const lsgd_config* cfg, const lsgd_allocator* alloc, voi
     st = alloc_dense(c);
     if (st == LSGD_OK) st = init_dense_params(c);
     if (st == LSGD_OK) st = make_tc_maps(c);
-    if (st == LSGD_OK && c0.fused_update && c->bf16) {
+    // fp32: always (same bits; the gradient array is not written)
+    if (st == LSGD_OK && (c0.fused_update || !c->bf16)) {
       c->fused = true;
-      for (const DenseLayer& L : c->layers) c->fused = c->fused && L.tc;
+      for (const DenseLayer& L : c->layers) c->fused = c->fused && (L.tc || !c->bf16);
     }
     if (st == LSGD_OK) {
       const DenseLayer& top = c->layers.back();
