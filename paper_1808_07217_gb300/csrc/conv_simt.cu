@@ -51,19 +51,23 @@ Tile tile_of(int B, int H, int W, int px_log2) {
 // output gradient as input and w_t[ci][co] = w[co][8 - t][ci] (flip); a stride-2 layer's reads the
 // output gradient with zeros between its pixels (up).
 //
-// A CTA computes 256 pixels x 16 channels, a thread 4 consecutive pixels x 8 channels (4 packed
-// pairs).  Eight input channels at a time, the tile's input with its halo is staged as one plane
-// per channel -- a warp's reads of its rows are then consecutive -- and their weights as
-// [channel][tap][16]; all lanes of a warp read the same weights.  Per channel and kernel row a
-// thread loads 6 inputs (9 at stride 2) in two or three loads and 24 weights in six, for 48 packed
-// multiply-adds.  The eight channels' products are summed by themselves and then added to the
-// running sum, which halves the length of the longest chain of roundings at 16 channels and keeps
-// it at 72 + Cin / 8 for any Cin.
+// A CTA computes 256 pixels x 16 channels, a thread 8 consecutive pixels x 4 channels (2 packed pairs).
+// Eight input channels at a time, the tile's input with its halo is staged as one plane per channel
+// and their weights as [channel][tap][16].  Per channel and kernel row a thread loads 10 inputs (17 at
+// stride 2) and 12 weights for 48 packed multiply-adds: 22 words through the shared-memory pipe's 32
+// lanes a cycle against 24 cycles of multiply-adds (4 pixels x 8 channels: 30 words, that pipe bound).
+// Four lanes share a pixel group and eight a weight group, so a load's lanes do not conflict.  A
+// slice's loads are all requested before the barrier that frees the staging buffers.  The eight
+// channels' products are summed by themselves and then added to the running sum, which halves the
+// length of the longest chain of roundings at 16 channels and keeps it at 72 + Cin / 8 for any Cin.
 // The 16-channel tile over 256 pixels reads each input once per 16 outputs; wider tiles of 32
 // channels leave too few CTAs on the later, smaller stages.
-// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.73 ms forward and data gradients
-// (7.3 ms with one thread per pixel that loaded a weight per multiply-add).
-constexpr int kFwThreads = 128, kFwPxLog2 = 8, kFwCo = 16, kFwCi = 8;
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.43 ms forward and data gradients (1.58 ms with
+// 4 pixels x 8 channels, weight stores in 16-way conflicts and the shortcut added element by element;
+// 7.3 ms with one thread per pixel that loaded a weight per multiply-add).
+constexpr int kFwThreads = 128, kFwPxLog2 = 8, kFwCo = 16, kFwCi = 8, kFwPx = 8;
+constexpr int kFwWPitch = kFwCo + 4;  // a tap's weights; 20 floats: eight channels by four taps, as a warp
+                                      // stores them, spread over eight groups of four banks (16: over two banks)
 
 struct ConvFwArgs {
   const void* in;
@@ -86,8 +90,8 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
   extern __shared__ __align__(16) float fw_sm[];
   const int plane = (a.pr * a.pitch) << a.t.ti;
   float* patch = fw_sm;                                   // [kFwCi][ti][pr][pitch]
-  float* ws = patch + kFwCi * plane;                      // [kFwCi][9][kFwCo]
-  int2* table = reinterpret_cast<int2*>(ws + kFwCi * 9 * kFwCo);  // per patch pixel: source, place
+  float* ws = patch + kFwCi * plane;                      // [kFwCi][9][kFwWPitch]
+  int2* table = reinterpret_cast<int2*>(ws + kFwCi * 9 * kFwWPitch);  // per patch pixel: source, place
   const int tid = threadIdx.x, g = blockIdx.z, co0 = blockIdx.y * kFwCo;
   int tile = blockIdx.x;
   const int x0 = (tile % a.t.nx) << a.t.tw;
@@ -110,132 +114,165 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
   const TA* in = reinterpret_cast<const TA*>(a.in) + (int64_t)g * a.B * a.Hi * a.Wi * a.Ci;
   const TA* w = reinterpret_cast<const TA*>(a.w) + (int64_t)g * a.w_gs;
 
-  const int pg = tid & 63, cog = tid >> 6;  // pixel group (a warp's are 32 in a row), channel half
-  const int gx = (pg << 2) & ((1 << a.t.tw) - 1), gr = (pg << 2) >> a.t.tw;
+  const int cog = tid & 3, px = (tid >> 2) * kFwPx;  // four channels; first pixel
+  const int gx = px & ((1 << a.t.tw) - 1), gr = px >> a.t.tw;
   const int gy = gr & ((1 << a.t.th) - 1), gi = gr >> a.t.th;
   const float* prow = patch + (gi * a.pr + gy * S) * a.pitch + gx * S;
-  const float* wrow = ws + 8 * cog;
+  const float* wrow = ws + 4 * cog;
 
-  u64 sum[4][4];
+  u64 sum[kFwPx][2];
 #pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) sum[p][q] = 0ull;
+  for (int p = 0; p < kFwPx; ++p) sum[p][0] = sum[p][1] = 0ull;
 
+  __syncthreads();  // the table
   for (int c0 = 0; c0 < a.Ci; c0 += kFwCi) {
     const int nc = min(kFwCi, a.Ci - c0);
-    __syncthreads();  // the table is written; the previous channels have been read
-    if ((a.Ci & 3) == 0) {
-      for (int e = tid; e < npx; e += kFwThreads) {
-        const int2 s = table[e];
+    // weights, consecutive threads on consecutive elements of the tensor; requested before the pixels
+    float wv[kFwCi * 9 * kFwCo / kFwThreads];
+    auto weight_at = [&](int i, int& co, int& t, int& c) {
+      const int e = tid + i * kFwThreads;
+      if (!a.flip)
+        c = e % kFwCi, t = (e / kFwCi) % 9, co = e / (9 * kFwCi);
+      else
+        co = e % kFwCo, t = (e / kFwCo) % 9, c = e / (9 * kFwCo);
+    };
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (4 * h >= nc) break;
-          const float4 v = s.x >= 0 ? load4(in + (int64_t)s.x * a.Ci + c0 + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
-          float* d = patch + 4 * h * plane + s.y;
-          d[0] = v.x;
-          d[plane] = v.y;
-          d[2 * plane] = v.z;
-          d[3 * plane] = v.w;
+    for (int i = 0; i < kFwCi * 9 * kFwCo / kFwThreads; ++i) {
+      int co, t, c;
+      weight_at(i, co, t, c);
+      wv[i] = 0.f;
+      if (c < nc && co0 + co < a.Co)
+        wv[i] = Elem<TA>::load(a.flip ? w + ((int64_t)(c0 + c) * 9 + 8 - t) * a.Co + co0 + co
+                                      : w + ((int64_t)(co0 + co) * 9 + t) * a.Ci + c0 + c);
+    }
+    bool read = false;  // whether every thread is past the previous channels
+    if ((a.Ci & 3) == 0) {
+      constexpr int NB = 3;
+      for (int e0 = tid; e0 < npx; e0 += NB * kFwThreads) {
+        int2 s[NB];
+        float4 v[NB][2];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+          const int e = e0 + i * kFwThreads;
+          s[i] = e < npx ? table[e] : make_int2(-1, -1);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            v[i][h] = s[i].x >= 0 && 4 * h < nc ? load4(in + (int64_t)s[i].x * a.Ci + c0 + 4 * h)
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if (!read) __syncthreads();
+        read = true;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+          if (s[i].y < 0) break;
+          float* d = patch + s[i].y;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            d[(4 * h) * plane] = v[i][h].x;
+            d[(4 * h + 1) * plane] = v[i][h].y;
+            d[(4 * h + 2) * plane] = v[i][h].z;
+            d[(4 * h + 3) * plane] = v[i][h].w;
+          }
         }
       }
     } else {
+      __syncthreads();
       for (int e = tid; e < npx; e += kFwThreads) {
         const int2 s = table[e];
         for (int c = 0; c < nc; ++c)
           patch[c * plane + s.y] = s.x >= 0 ? Elem<TA>::load(in + (int64_t)s.x * a.Ci + c0 + c) : 0.f;
       }
     }
-    // weights, consecutive threads on consecutive elements of the tensor
-    for (int e = tid; e < kFwCi * 9 * kFwCo; e += kFwThreads) {
+#pragma unroll
+    for (int i = 0; i < kFwCi * 9 * kFwCo / kFwThreads; ++i) {
       int co, t, c;
-      float v = 0.f;
-      if (!a.flip) {
-        c = e % kFwCi, t = (e / kFwCi) % 9, co = e / (9 * kFwCi);
-        if (c < nc && co0 + co < a.Co) v = Elem<TA>::load(w + ((int64_t)(co0 + co) * 9 + t) * a.Ci + c0 + c);
-      } else {
-        co = e % kFwCo, t = (e / kFwCo) % 9, c = e / (9 * kFwCo);
-        if (c < nc && co0 + co < a.Co) v = Elem<TA>::load(w + ((int64_t)(c0 + c) * 9 + 8 - t) * a.Co + co0 + co);
-      }
-      ws[(c * 9 + t) * kFwCo + co] = v;
+      weight_at(i, co, t, c);
+      ws[(c * 9 + t) * kFwWPitch + co] = wv[i];
     }
     __syncthreads();
-    u64 acc[4][4];
+    u64 acc[kFwPx][2];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[p][q] = 0ull;
+    for (int p = 0; p < kFwPx; ++p) acc[p][0] = acc[p][1] = 0ull;
     for (int c = 0; c < nc; ++c) {
 #pragma unroll
       for (int kh = 0; kh < 3; ++kh) {
         const float* r = prow + c * plane + kh * a.pitch;
-        constexpr int NV = 3 * S + 3;
-        u64 v[NV];
+        constexpr int NV = (kFwPx - 1) * S + 3;
+        float v[NV];
 #pragma unroll
         for (int i = 0; i + 4 <= NV; i += 4) {
           const float4 f = *reinterpret_cast<const float4*>(r + i);
-          v[i] = pack2(f.x, f.x);
-          v[i + 1] = pack2(f.y, f.y);
-          v[i + 2] = pack2(f.z, f.z);
-          v[i + 3] = pack2(f.w, f.w);
+          v[i] = f.x;
+          v[i + 1] = f.y;
+          v[i + 2] = f.z;
+          v[i + 3] = f.w;
         }
         if (S == 1) {
-          const float2 f = *reinterpret_cast<const float2*>(r + 4);
-          v[4] = pack2(f.x, f.x);
-          v[5] = pack2(f.y, f.y);
+          const float2 f = *reinterpret_cast<const float2*>(r + NV - 2);
+          v[NV - 2] = f.x;
+          v[NV - 1] = f.y;
         } else {
-          v[NV - 1] = pack2(r[8], r[8]);
+          v[NV - 1] = r[NV - 1];
         }
 #pragma unroll
         for (int kw = 0; kw < 3; ++kw) {
-          const ulonglong2* wp = reinterpret_cast<const ulonglong2*>(wrow + (c * 9 + kh * 3 + kw) * kFwCo);
-          const ulonglong2 w0 = wp[0], w1 = wp[1];
+          const ulonglong2 wq = *reinterpret_cast<const ulonglong2*>(wrow + (c * 9 + kh * 3 + kw) * kFwWPitch);
 #pragma unroll
-          for (int p = 0; p < 4; ++p) {
-            const u64 x = v[p * S + kw];
-            fma2(acc[p][0], x, w0.x);
-            fma2(acc[p][1], x, w0.y);
-            fma2(acc[p][2], x, w1.x);
-            fma2(acc[p][3], x, w1.y);
+          for (int p = 0; p < kFwPx; ++p) {
+            const u64 x = pack2(v[p * S + kw], v[p * S + kw]);
+            fma2(acc[p][0], x, wq.x);
+            fma2(acc[p][1], x, wq.y);
           }
         }
       }
     }
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) add2(sum[p][q], acc[p][q]);
+    for (int p = 0; p < kFwPx; ++p) {
+      add2(sum[p][0], acc[p][0]);
+      add2(sum[p][1], acc[p][1]);
+    }
   }
 
   const int b = b0 + gi, y = y0 + gy;
   if (b >= a.B || y >= a.Ho) return;
-  const int co = co0 + 8 * cog;
+  const int co = co0 + 4 * cog;
   const int64_t img = (int64_t)g * a.B + b;
+  const bool sc_row = a.sc_dout && y % a.sc_s == 0, whole = ((a.Co | a.sc_C) & 3) == 0;
+  auto sc_at = [&](int x) { return ((img * a.sc_H + y / a.sc_s) * a.sc_W + x / a.sc_s) * a.sc_C + co; };
+  float4 act[kFwPx], d[kFwPx];  // the shortcut's, requested together
 #pragma unroll
-  for (int p = 0; p < 4; ++p) {
+  for (int p = 0; p < kFwPx; ++p) {
+    const int x = x0 + gx + p;
+    const bool on = sc_row && whole && co < a.Co && x < a.Wo && x % a.sc_s == 0;
+    act[p] = d[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (on) {
+      act[p] = load4(reinterpret_cast<const TA*>(a.sc_act) + sc_at(x));
+      d[p] = load4(a.sc_dout + sc_at(x));
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < kFwPx; ++p) {
     const int x = x0 + gx + p;
     if (x >= a.Wo) break;
-    float o[8];
+    const float2 lo = unpack2(sum[p][0]), hi = unpack2(sum[p][1]);
+    float o[4] = {lo.x, lo.y, hi.x, hi.y};
+    o[0] = act[p].x > 0.f ? o[0] + d[p].x : o[0];
+    o[1] = act[p].y > 0.f ? o[1] + d[p].y : o[1];
+    o[2] = act[p].z > 0.f ? o[2] + d[p].z : o[2];
+    o[3] = act[p].w > 0.f ? o[3] + d[p].w : o[3];
+    if (sc_row && !whole && x % a.sc_s == 0) {
+      const int64_t e = sc_at(x);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2 f = unpack2(sum[p][q]);
-      o[2 * q] = f.x;
-      o[2 * q + 1] = f.y;
-    }
-    if (a.sc_dout && y % a.sc_s == 0 && x % a.sc_s == 0) {
-      const int64_t e = ((img * a.sc_H + y / a.sc_s) * a.sc_W + x / a.sc_s) * a.sc_C + co;
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 4; ++i)
         if (co + i < a.Co && Elem<TA>::load(reinterpret_cast<const TA*>(a.sc_act) + e + i) > 0.f)
           o[i] += a.sc_dout[e + i];
     }
     float* dst = a.out + ((img * a.Ho + y) * a.Wo + x) * a.Co + co;
     if ((a.Co & 3) == 0) {
       if (co < a.Co) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-      if (co + 4 < a.Co) *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 4; ++i)
         if (co + i < a.Co) dst[i] = o[i];
     }
   }
@@ -247,7 +284,7 @@ cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
   a.pr = ((1 << a.t.th) - 1) * S + 3;
   a.pc = ((1 << a.t.tw) - 1) * S + 3;
   a.pitch = (a.pc + 3) / 4 * 4;  // rows start on 16 bytes
-  const size_t smem = (size_t)kFwCi * ((a.pr * a.pitch) << a.t.ti) * 4 + kFwCi * 9 * kFwCo * 4 +
+  const size_t smem = (size_t)kFwCi * ((a.pr * a.pitch) << a.t.ti) * 4 + kFwCi * 9 * kFwWPitch * 4 +
                       (size_t)((a.pr * a.pc) << a.t.ti) * sizeof(int2);
   const dim3 grid(a.t.tiles, (a.Co + kFwCo - 1) / kFwCo, G);
   if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
@@ -277,7 +314,7 @@ cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
 // the four rows' sums are added in a fixed order.
 // An accumulator's chain is a tile range's pixels / 4 (a few hundred roundings; one thread used to
 // add 2,048).
-// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.86 ms (46.7 ms with 16 pixels staged
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.76 ms (46.7 ms with 16 pixels staged
 // between two barriers and a shared-memory load per multiply-add).
 constexpr int kWgThreads = 192, kWgPxLog2 = 7;
 
@@ -503,12 +540,12 @@ cudaError_t launch_conv3x3_simt(const ConvSimtArgs& c, cudaStream_t s) {
   return two ? launch_fw<float, 2>(a, c.G, s) : launch_fw<float, 1>(a, c.G, s);
 }
 
-// Ranges of one replica: about four CTAs per SM over the replicas and channel blocks, at least one
-// tile each.
+// Ranges of one replica: three CTAs per SM over the replicas and channel blocks -- all that are resident,
+// in one wave -- and at least one tile each.  (Four per SM ran as a wave and a third: 55 against 46 us at 64 channels, 41 against 38 at 16.)
 int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout) {
   const int blocks = ((cout + 15) / 16) * ((cin + 15) / 16);
   const int tiles = tile_of(B, hout, wout, kWgPxLog2).tiles;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 4LL * kNumSMs / ((int64_t)G * blocks)));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 3LL * kNumSMs / ((int64_t)G * blocks)));
 }
 
 cudaError_t launch_conv_wgrad_simt(const ConvSimtArgs& c, const void* dy, float* part, cudaStream_t s) {
