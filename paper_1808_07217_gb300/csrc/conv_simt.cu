@@ -3,7 +3,8 @@
 // The fp32 mode's convolutions (tensor cores cannot give fp32-exact products) and the SIMT form of
 // the bf16 ones.  All three products of a layer run as register-tiled shared-memory kernels on the
 // packed two-lane fp32 multiply-add (fma.rn.f32x2: two roundings, each that of fmaf, in one issue
-// slot), and all are bound by that pipe: per shared-memory load a thread does 8 to 12 of them.
+// slot).  They keep that pipe about half busy: the moves that put one input into both lanes, the staging
+// between barriers and the uneven last CTAs take the rest.
 #include <algorithm>
 
 #include "common.cuh"
@@ -62,12 +63,19 @@ Tile tile_of(int B, int H, int W, int px_log2) {
 // length of the longest chain of roundings at 16 channels and keeps it at 72 + Cin / 8 for any Cin.
 // The 16-channel tile over 256 pixels reads each input once per 16 outputs; wider tiles of 32
 // channels leave too few CTAs on the later, smaller stages.
-// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.43 ms forward and data gradients (1.58 ms with
+// KS = 2, where at most two CTAs per SM would leave the schedulers two warps each (a late stage: 256
+// CTAs): a second 128 threads take the odd groups of eight channels, and their sums are added at the
+// end.  64 channels of 8 x 8 pixels: 43 -> 38 us, a whole pass of two steps 6.50 -> 6.15 ms; at up to four
+// CTAs per SM it gains nothing more (6.16).  Plain fmaf, without the packing moves, is slower (52 us), and
+// so are copies of the next slice in flight during this one's products (6.96 ms at KS = 1).
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.37 ms forward and data gradients (1.58 ms with
 // 4 pixels x 8 channels, weight stores in 16-way conflicts and the shortcut added element by element;
 // 7.3 ms with one thread per pixel that loaded a weight per multiply-add).
 constexpr int kFwThreads = 128, kFwPxLog2 = 8, kFwCo = 16, kFwCi = 8, kFwPx = 8;
 constexpr int kFwWPitch = kFwCo + 4;  // a tap's weights; 20 floats: eight channels by four taps, as a warp
                                       // stores them, spread over eight groups of four banks (16: over two banks)
+
+constexpr int kFwMaxSmem = 100 * 1024;
 
 struct ConvFwArgs {
   const void* in;
@@ -84,22 +92,25 @@ struct ConvFwArgs {
   int sc_s, sc_H, sc_W, sc_C;
 };
 
-template <typename TA, int S>
-__global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __grid_constant__ ConvFwArgs a) {
+template <typename TA, int S, int KS>
+__global__ void __launch_bounds__(kFwThreads * KS, 4 / KS)
+    conv3x3_simt_kernel(const __grid_constant__ ConvFwArgs a) {
   pdl_begin();
   extern __shared__ __align__(16) float fw_sm[];
+  constexpr int NT = kFwThreads * KS, CI = kFwCi * KS, NW = CI * 9 * kFwCo / NT;
   const int plane = (a.pr * a.pitch) << a.t.ti;
-  float* patch = fw_sm;                                   // [kFwCi][ti][pr][pitch]
-  float* ws = patch + kFwCi * plane;                      // [kFwCi][9][kFwWPitch]
-  int2* table = reinterpret_cast<int2*>(ws + kFwCi * 9 * kFwWPitch);  // per patch pixel: source, place
-  const int tid = threadIdx.x, g = blockIdx.z, co0 = blockIdx.y * kFwCo;
+  float* patch = fw_sm;                                   // [CI][ti][pr][pitch]
+  float* ws = patch + CI * plane;                         // [CI][9][kFwWPitch]
+  int2* table = reinterpret_cast<int2*>(ws + CI * 9 * kFwWPitch);  // per patch pixel: source, place
+  const int tid = threadIdx.x, ht = tid % kFwThreads, half = tid / kFwThreads;
+  const int g = blockIdx.z, co0 = blockIdx.y * kFwCo;
   int tile = blockIdx.x;
   const int x0 = (tile % a.t.nx) << a.t.tw;
   tile /= a.t.nx;
   const int y0 = (tile % a.t.ny) << a.t.th;
   const int b0 = (tile / a.t.ny) << a.t.ti;
   const int npx = (a.pr * a.pc) << a.t.ti;
-  for (int e = tid; e < npx; e += kFwThreads) {
+  for (int e = tid; e < npx; e += NT) {
     const int px = e % a.pc, r = e / a.pc, py = r % a.pr, im = r / a.pr;
     int iy = y0 * S + py - 1, ix = x0 * S + px - 1;
     bool in = b0 + im < a.B && iy >= 0 && ix >= 0;
@@ -114,7 +125,7 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
   const TA* in = reinterpret_cast<const TA*>(a.in) + (int64_t)g * a.B * a.Hi * a.Wi * a.Ci;
   const TA* w = reinterpret_cast<const TA*>(a.w) + (int64_t)g * a.w_gs;
 
-  const int cog = tid & 3, px = (tid >> 2) * kFwPx;  // four channels; first pixel
+  const int cog = tid & 3, px = (ht >> 2) * kFwPx;  // four channels; first pixel
   const int gx = px & ((1 << a.t.tw) - 1), gr = px >> a.t.tw;
   const int gy = gr & ((1 << a.t.th) - 1), gi = gr >> a.t.th;
   const float* prow = patch + (gi * a.pr + gy * S) * a.pitch + gx * S;
@@ -125,30 +136,41 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
   for (int p = 0; p < kFwPx; ++p) sum[p][0] = sum[p][1] = 0ull;
 
   __syncthreads();  // the table
-  for (int c0 = 0; c0 < a.Ci; c0 += kFwCi) {
-    const int nc = min(kFwCi, a.Ci - c0);
-    // weights, consecutive threads on consecutive elements of the tensor; requested before the pixels
-    float wv[kFwCi * 9 * kFwCo / kFwThreads];
-    auto weight_at = [&](int i, int& co, int& t, int& c) {
-      const int e = tid + i * kFwThreads;
-      if (!a.flip)
-        c = e % kFwCi, t = (e / kFwCi) % 9, co = e / (9 * kFwCi);
-      else
-        co = e % kFwCo, t = (e / kFwCo) % 9, c = e / (9 * kFwCo);
-    };
+  const bool quads = (a.Ci & 3) == 0;
+  // weight i of this thread in a slice: consecutive threads on consecutive elements of the tensor
+  auto weight_at = [&](int i, int& co, int& t, int& c) {
+    const int e = tid + i * NT;
+    if (!a.flip)
+      c = e % CI, t = (e / CI) % 9, co = e / (9 * CI);
+    else
+      co = e % kFwCo, t = (e / kFwCo) % 9, c = e / (9 * kFwCo);
+  };
+  auto weight_src = [&](int c0, int co, int t, int c) {
+    return a.flip ? w + ((int64_t)(c0 + c) * 9 + 8 - t) * a.Co + co0 + co
+                  : w + ((int64_t)(co0 + co) * 9 + t) * a.Ci + c0 + c;
+  };
+  const int h0 = half * kFwCi;  // the half's channels of a slice
+  auto put = [&](int place, int c, const float4& v) {
+    float* d = patch + c * plane + place;
+    d[0] = v.x;
+    d[plane] = v.y;
+    d[2 * plane] = v.z;
+    d[3 * plane] = v.w;
+  };
+  for (int c0 = 0; c0 < a.Ci; c0 += CI) {
+    const int nc = min(CI, a.Ci - c0);
+    // all of a slice's loads, the weights' first, before the barrier
+    float wv[NW];
 #pragma unroll
-    for (int i = 0; i < kFwCi * 9 * kFwCo / kFwThreads; ++i) {
+    for (int i = 0; i < NW; ++i) {
       int co, t, c;
       weight_at(i, co, t, c);
       wv[i] = 0.f;
-      if (c < nc && co0 + co < a.Co)
-        wv[i] = Elem<TA>::load(a.flip ? w + ((int64_t)(c0 + c) * 9 + 8 - t) * a.Co + co0 + co
-                                      : w + ((int64_t)(co0 + co) * 9 + t) * a.Ci + c0 + c);
+      if (c < nc && co0 + co < a.Co) wv[i] = Elem<TA>::load(weight_src(c0, co, t, c));
     }
-    bool read = false;  // whether every thread is past the previous channels
-    if ((a.Ci & 3) == 0) {
+    if (quads) {
       constexpr int NB = 3;
-      for (int e0 = tid; e0 < npx; e0 += NB * kFwThreads) {
+      for (int e0 = ht; e0 - ht < npx; e0 += NB * kFwThreads) {
         int2 s[NB];
         float4 v[NB][2];
 #pragma unroll
@@ -157,34 +179,27 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
           s[i] = e < npx ? table[e] : make_int2(-1, -1);
 #pragma unroll
           for (int h = 0; h < 2; ++h)
-            v[i][h] = s[i].x >= 0 && 4 * h < nc ? load4(in + (int64_t)s[i].x * a.Ci + c0 + 4 * h)
-                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[i][h] = s[i].x >= 0 && h0 + 4 * h < nc ? load4(in + (int64_t)s[i].x * a.Ci + c0 + h0 + 4 * h)
+                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        if (!read) __syncthreads();
-        read = true;
+        if (e0 == ht) __syncthreads();
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
           if (s[i].y < 0) break;
-          float* d = patch + s[i].y;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            d[(4 * h) * plane] = v[i][h].x;
-            d[(4 * h + 1) * plane] = v[i][h].y;
-            d[(4 * h + 2) * plane] = v[i][h].z;
-            d[(4 * h + 3) * plane] = v[i][h].w;
-          }
+          put(s[i].y, h0, v[i][0]);
+          put(s[i].y, h0 + 4, v[i][1]);
         }
       }
     } else {
       __syncthreads();
-      for (int e = tid; e < npx; e += kFwThreads) {
+      for (int e = tid; e < npx; e += NT) {
         const int2 s = table[e];
         for (int c = 0; c < nc; ++c)
           patch[c * plane + s.y] = s.x >= 0 ? Elem<TA>::load(in + (int64_t)s.x * a.Ci + c0 + c) : 0.f;
       }
     }
 #pragma unroll
-    for (int i = 0; i < kFwCi * 9 * kFwCo / kFwThreads; ++i) {
+    for (int i = 0; i < NW; ++i) {
       int co, t, c;
       weight_at(i, co, t, c);
       ws[(c * 9 + t) * kFwWPitch + co] = wv[i];
@@ -193,7 +208,7 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
     u64 acc[kFwPx][2];
 #pragma unroll
     for (int p = 0; p < kFwPx; ++p) acc[p][0] = acc[p][1] = 0ull;
-    for (int c = 0; c < nc; ++c) {
+    for (int c = h0; c < min(nc, h0 + kFwCi); ++c) {
 #pragma unroll
       for (int kh = 0; kh < 3; ++kh) {
         const float* r = prow + c * plane + kh * a.pitch;
@@ -231,6 +246,24 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
       add2(sum[p][0], acc[p][0]);
       add2(sum[p][1], acc[p][1]);
     }
+  }
+
+  if constexpr (KS == 2) {
+    // the second half's sums to the first, where the staging buffers were
+    u64* other = reinterpret_cast<u64*>(fw_sm) + ht;
+    __syncthreads();
+    if (half) {
+#pragma unroll
+      for (int p = 0; p < kFwPx; ++p)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) other[(2 * p + q) * kFwThreads] = sum[p][q];
+    }
+    __syncthreads();
+    if (half) return;
+#pragma unroll
+    for (int p = 0; p < kFwPx; ++p)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) add2(sum[p][q], other[(2 * p + q) * kFwThreads]);
   }
 
   const int b = b0 + gi, y = y0 + gy;
@@ -278,27 +311,38 @@ __global__ void __launch_bounds__(kFwThreads, 4) conv3x3_simt_kernel(const __gri
   }
 }
 
+template <typename TA, int S, int KS>
+cudaError_t launch_fw_ks(const ConvFwArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
+  static int attr_dev = -1;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (attr_dev != dev) {
+    e = cudaFuncSetAttribute(conv3x3_simt_kernel<TA, S, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kFwMaxSmem);
+    if (e != cudaSuccess) return e;
+    attr_dev = dev;
+  }
+  return launch_pdl(conv3x3_simt_kernel<TA, S, KS>, grid, dim3(kFwThreads * KS), smem, s, a);
+}
+
 template <typename TA, int S>
 cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
   a.t = tile_of(a.B, a.Ho, a.Wo, kFwPxLog2);
   a.pr = ((1 << a.t.th) - 1) * S + 3;
   a.pc = ((1 << a.t.tw) - 1) * S + 3;
   a.pitch = (a.pc + 3) / 4 * 4;  // rows start on 16 bytes
-  const size_t smem = (size_t)kFwCi * ((a.pr * a.pitch) << a.t.ti) * 4 + kFwCi * 9 * kFwWPitch * 4 +
-                      (size_t)((a.pr * a.pc) << a.t.ti) * sizeof(int2);
   const dim3 grid(a.t.tiles, (a.Co + kFwCo - 1) / kFwCo, G);
   if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
-  static int attr_dev = -1;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (attr_dev != dev) {
-    e = cudaFuncSetAttribute(conv3x3_simt_kernel<TA, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             100 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_dev = dev;
+  auto smem = [&](int ks) {
+    return (size_t)ks * kFwCi * (((a.pr * a.pitch) << a.t.ti) + 9 * kFwWPitch) * 4 +
+           (size_t)((a.pr * a.pc) << a.t.ti) * sizeof(int2);
+  };
+  if constexpr (S == 1) {
+    if (a.Ci > kFwCi && (int64_t)grid.x * grid.y * grid.z <= 2 * kNumSMs && smem(2) <= kFwMaxSmem)
+      return launch_fw_ks<TA, S, 2>(a, grid, smem(2), s);
   }
-  return launch_pdl(conv3x3_simt_kernel<TA, S>, grid, dim3(kFwThreads), smem, s, a);
+  return launch_fw_ks<TA, S, 1>(a, grid, smem(1), s);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -1,6 +1,7 @@
 """The fp32-core convolutions against the oracle: the gradient of one ResNet step at geometries that
 cut their tiles (images narrower, wider and taller than a tile, odd sizes under stride 2, channel
-counts that are no multiple of the 16-channel block or of 4, a batch that leaves a partial tile)."""
+counts that are no multiple of the 16-channel block or of 4, a batch that leaves a partial tile, few
+CTAs and many)."""
 import numpy as np
 import pytest
 
@@ -13,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("hwc,base,B,K", [((32, 32, 3), 16, 6, 2), ((9, 7, 5), 12, 5, 3),
                                           ((35, 41, 16), 8, 3, 1), ((2, 3, 1), 4, 40, 2),
-                                          ((16, 8, 64), 4, 7, 1)])
+                                          ((16, 8, 64), 4, 7, 1),
+                                          ((16, 16, 3), 16, 320, 1)])  # more than two CTAs per SM
 def test_fp32_step_gradient(hwc, base, B, K):
     P = built_package()
     N, C = max(K * B, 64), 5
