@@ -102,7 +102,8 @@ typedef struct {
   int fused_update;      /* BF16 dense models on tcgen05: 1 = the weight-gradient epilogue (and the
                             bias-gradient sum) apply the local update directly, so the gradient is
                             never written to memory; bit-identical to 0, which runs the stand-alone
-                            update kernel over the whole K x d buffer.  Ignored elsewhere. */
+                            update kernel over the whole K x d buffer.  FP32 dense models always
+                            update in their gradient kernels (the same bits); ignored elsewhere. */
   int hier_block;        /* hierarchical local SGD (Sec. D): > 0 = after every H-step round the
                             hier_block consecutive replicas of each block are averaged, and every
                             hier_rounds-th round (and the run's last step) all K; must divide K.
@@ -305,9 +306,9 @@ typedef enum {
   LSGD_PH_INPUT = 0,    /* index sampling + row gather / cast (or the caller batch's copy) */
   LSGD_PH_FORWARD = 1,  /* forward GEMMs / convolutions */
   LSGD_PH_LOSS = 2,     /* softmax cross-entropy (or least-squares) loss and its gradient */
-  LSGD_PH_BACKWARD = 3, /* data / weight gradient products and bias sums (with fused_update: the
-                           data-gradient products and the bias sum + update launches) */
-  LSGD_PH_UPDATE = 4,   /* the local update kernel (with fused_update: the weight-gradient
+  LSGD_PH_BACKWARD = 3, /* data / weight gradient products and bias sums (with fused_update, and in
+                           FP32 dense models: the data-gradient products and the bias sum + update launches) */
+  LSGD_PH_UPDATE = 4,   /* the local update kernel (with fused_update, and in FP32 dense models: the weight-gradient
                            launches that apply the update in their epilogue) */
   LSGD_PH_AVERAGE = 5,  /* the K-way average kernel */
   LSGD_NUM_PHASES = 6
@@ -364,9 +365,9 @@ lsgd_status lsgd_batchnorm_stats(const float* y, int64_t P, int C, int G, float*
  *   dW[g][co][kh][kw][ci] = sum over b, oy, ox of dy[g][b][oy][ox][co] x[g][b][oy s + kh - 1][ox s + kw - 1][ci]
  * (x zero outside the image).  x [G][B][s Hout][s Wout][Cin] and dy [G][B][Hout][Wout][Cout] are
  * NHWC bf16 device arrays (16-byte aligned), dW [G][Cout][3][3][Cin] fp32 device, fully
- * overwritten.  The column matrix of every 64-pixel block is built in shared memory; one fp32
- * partial per CTA (a scratch buffer allocated and freed on `stream`) is summed in CTA order, so
- * the result is deterministic.  Cin 16, 32 or 64; Cout a multiple of 16 up to 64; Wout dividing
+ * overwritten.  The taps read shifted windows of input strips in shared memory (outputs narrower
+ * than 8 pixels run on the fp32 cores); one fp32 partial per CTA (a scratch buffer allocated and
+ * freed on `stream`) is summed in CTA order, so the result is deterministic.  Cin 16, 32 or 64; Cout a multiple of 16 up to 64; Wout dividing
  * 64 and Hout Wout a multiple of 64: LSGD_EINVAL otherwise, LSGD_ENOMEM if the scratch cannot be
  * allocated, LSGD_EUNSUPPORTED without tcgen05. */
 lsgd_status lsgd_conv_wgrad_bf16(const uint16_t* x, const uint16_t* dy, float* dW, int G, int B,
@@ -398,10 +399,10 @@ lsgd_status lsgd_conv3x3_bf16(int mode, const uint16_t* in, const uint16_t* W, f
  * statistics of its output (Sec. A.4; the first half of the conv -> BN -> ReLU unit of Sec. A.2's
  * ResNet-20), as the ResNet-20 training step computes them: y [G][B][Hout][Wout][Cout] fp32 as in
  * mode 0, and mean[G][Cout], rstd[G][Cout] = 1 / sqrt(biased variance + 1e-5) over the B Hout Wout
- * output positions of each group.  Each epilogue warp of the convolution keeps a running (count,
- * mean, sum of squared deviations) per channel, combining the two-pass moments of its 32 rows of
- * every 128-pixel tile in tile order by Chan et al.'s formula; a second kernel combines the
- * warps' partials in a fixed order, so the result is deterministic.  Same operands, alignment and shapes as mode 0 with
+ * output positions of each group.  The convolution's epilogue keeps running (count, mean,
+ * sum of squared deviations) partials per channel, combining the two-pass moments of its share of
+ * every tile in tile order by Chan et al.'s formula; a second kernel combines the partials in a
+ * fixed order, so the result is deterministic.  Same operands, alignment and shapes as mode 0 with
  * Cout <= 64; mean and rstd fp32 device arrays.  Scratch (the stem operands and the partials) is
  * allocated and freed on `stream`.  LSGD_EINVAL on bad arguments, LSGD_EUNSUPPORTED for shapes the
  * kernel does not take, LSGD_ENOMEM if the scratch cannot be allocated. */

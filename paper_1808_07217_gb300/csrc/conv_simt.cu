@@ -68,7 +68,7 @@ Tile tile_of(int B, int H, int W, int px_log2) {
 // end.  64 channels of 8 x 8 pixels: 43 -> 38 us, a whole pass of two steps 6.50 -> 6.15 ms; at up to four
 // CTAs per SM it gains nothing more (6.16).  Plain fmaf, without the packing moves, is slower (52 us), and
 // so are copies of the next slice in flight during this one's products (6.96 ms at KS = 1).
-// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.37 ms forward and data gradients (1.58 ms with
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 1.45 ms forward and data gradients (1.65 ms with
 // 4 pixels x 8 channels, weight stores in 16-way conflicts and the shortcut added element by element;
 // 7.3 ms with one thread per pixel that loaded a weight per multiply-add).
 constexpr int kFwThreads = 128, kFwPxLog2 = 8, kFwCo = 16, kFwCi = 8, kFwPx = 8;
@@ -358,7 +358,7 @@ cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
 // the four rows' sums are added in a fixed order.
 // An accumulator's chain is a tile range's pixels / 4 (a few hundred roundings; one thread used to
 // add 2,048).
-// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.76 ms (46.7 ms with 16 pixels staged
+// Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.78 ms (46.7 ms with 16 pixels staged
 // between two barriers and a shared-memory load per multiply-add).
 constexpr int kWgThreads = 192, kWgPxLog2 = 7;
 

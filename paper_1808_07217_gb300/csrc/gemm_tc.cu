@@ -6,9 +6,10 @@
 // replica, so the CTA for (n-tile, m-tile, replica g) loads its tiles at coordinate z = g.
 //
 // One CTA computes a 128 x BN fp32 tile in TMEM:
-//   warp 0 (one lane)  TMA producer: k-blocks of 64 bf16 (one 128-byte swizzle row) into a ring
-//                      of shared-memory stages, completion signalled on the stage's mbarrier;
-//   warp 1 (one lane)  MMA issuer: 4 x tcgen05.mma (M=128, N=BN, K=16) per stage, accumulate in
+//   warps 0, 3         TMA producers of A and of B: k-blocks of 64 bf16 (one 128-byte swizzle row)
+//                      into a ring of shared-memory stages, completion signalled on the stage's
+//                      mbarrier;
+//   warp 1             MMA issuer: 4 x tcgen05.mma (M=128, N=BN, K=16) per stage, accumulate in
 //                      TMEM; tcgen05.commit frees the stage and finally signals the epilogue;
 //   warp 2             allocates / frees the TMEM columns;
 //   warps 0-3          epilogue: tcgen05.ld of their 32 TMEM lanes (= tile rows), bias / ReLU /
@@ -651,7 +652,8 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
 // tiles blockIdx.x, blockIdx.x + gridDim.x, ... with the replica innermost (so the CTAs that
 // share a weight tile when every replica reads replica 0's, b_shared, run together and L2 serves
 // it), and two TMEM accumulators let one tile's epilogue overlap the next tile's products:
-//   warp 0      TMA producer: A (128 x 64) and B (PBN x 64) k-blocks into a PST-stage ring
+//   warps 0, 3  TMA producers: A (128 x 64) and 64 of B's columns, and the rest of B's PBN, of each
+//               k-block into a PST-stage ring
 //   warp 1      MMA issuer: tcgen05.mma (M = 128, N = PBN, K = 16), accumulator (tile & 1)
 //   warp 2      TMEM allocation (2 PBN columns)
 //   warps 4-7   epilogue (epilogue_rows: bias / ReLU / ReLU mask; column sums + bias

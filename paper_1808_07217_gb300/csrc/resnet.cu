@@ -1242,7 +1242,7 @@ bool implicit_conv_ok(int ck, int stride, int hout, int wout) {
   return (ck == 16 || ck == 32 || ck == 64) && (stride == 1 || stride == 2) &&
          conv_tile_shape(hout, wout, &rows, &images);
 }
-// The weight gradient builds its column matrix in shared memory (conv_wgrad_tc_kernel).
+// The weight gradient reads its taps from shared-memory strips of the input (conv_wgrad_tc_kernel).
 bool wgrad_tc(const ResNetPlan* p, const ConvL& c) {
   return conv_on_tc(p, c) && conv_wgrad_tc_ok(c.cin, c.cout, c.stride, c.hin, c.win, c.hout, c.wout);
 }
@@ -1836,8 +1836,7 @@ lsgd_status conv_wgrad(ResNetPlan* p, int i, const void* in, float* Gr, cudaStre
     return LSGD_OK;
   }
   if (wgrad_tc(p, c)) {
-    // dW [Cout][9 Cin] from dy and the input directly: the column matrix of each 64-pixel block
-    // is built in shared memory; one partial per CTA, summed in order
+    // dW [Cout][9 Cin] from dy and strips of the input; one partial per CTA, summed in order
     // with a buffer of its own the partials' sum waits for the end of the backward, where one
     // launch adds every layer's
     float* wp = (size_t)i < p->wpart.size() ? p->wpart[i] : nullptr;
