@@ -1886,9 +1886,15 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
 // epilogue at 107 us (141 with the shortcut) for a first-stage layer of 16 workers x 128 images.
 // A lane then also holds few channels (8, or 16 of 64), so running moments and sums stay in its
 // registers until the end of the kernel: no exchange per tile.
-// Measured there: forward with statistics 35 us, data gradient 32 (201 MB: 6.3 TB/s), with the
-// BatchNorm-backward epilogue 59 (402 MB: 6.8 TB/s), 90 with the shortcut, where conv_tc_kernel took
-// 65, 55, 102 and 135.
+// Measured there: forward with statistics 44 us (201 MB: 4.6 TB/s), data gradient with the
+// BatchNorm-backward epilogue 66 (402 MB: 6.1 TB/s), 104 with the shortcut, where conv_tc_kernel took
+// 65, 102 and 135.
+// 16 outputs or 64 inputs to a pixel: each kernel row has partial columns of its own (npart), added by the
+// epilogue, which hands them back as soon as they are in registers.  A tensor-core sum rounds with every
+// product added: one chain over the kernel rows was off by 8.5e-8 and 3.0e-7 (relative, 16 and 64
+// channels, forward; 4.8e-7 the 64-channel data gradient) where three are off by 4.9e-8, 1.1e-7 and
+// 1.7e-7, as conv_tc_kernel is.  It costs 7.41 -> 7.79 ms for two ResNet-20 steps: fewer tiles in TMEM.  The
+// partials are read eight registers at a time (sixteen spilled: 8.05 ms).
 // The BatchNorm-backward epilogue reads up to 192 bytes for every 64 it writes, and four warps that
 // went through a tile's rows one after another were bound by the latency of those reads (102 us, 158
 // with the shortcut): its sixteen warps (eight of an M = 64 tile) take 16 rows x 32 columns each, on
@@ -1950,6 +1956,32 @@ __device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, float (&v)[16]
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+// And for 16.
+__device__ __forceinline__ void tmem_ld_16x256_x2(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+// The partial accumulators np columns apart beyond the first, added in order.
+template <int NV>
+__device__ __forceinline__ void tmem_add_16x256(uint32_t at, int npart, int np, float (&v)[NV]) {
+#pragma unroll 1
+  for (int p = 1; p < npart; ++p) {
+#pragma unroll
+    for (int i = 0; i < NV / 8; ++i) {
+      float q[8];
+      tmem_ld_16x256_x2(at + (uint32_t)(p * np + 16 * i), q);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[8 * i + k] += q[k];
+    }
+  }
+}
 __device__ __forceinline__ bool bf_positive(const uint32_t (&w)[4], int k) {
   return bf2f((uint16_t)(k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu)) > 0.f;
 }
@@ -1962,7 +1994,7 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   const int ck = a.ck, ks = ck / 16, nst = a.nst, nacc = a.nacc;
-  const int np = 64 * a.nseg;                        // accumulator columns
+  const int np = 64 * a.nseg, npart = a.npart;       // a partial accumulator's columns; partials of a tile
   const int per_row = a.nj * ks, nmma = a.nkh * per_row;
   const uint32_t box_bytes = (uint32_t)a.box_rows * sp::ROWB, pitch = (box_bytes + 1023u) & ~1023u;
   const uint32_t slice_bytes = (uint32_t)np * 32u;   // one slice's weights
@@ -1976,7 +2008,7 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int g = blockIdx.y, cpr = gridDim.x;
   const int tpi = a.hg / a.tr, tiles = a.B * tpi;  // tiles per image, per replica
-  const uint32_t tmem_cols = conv_tmem_cols(nacc, np);
+  const uint32_t tmem_cols = conv_tmem_cols(nacc * npart, np);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < nst; ++i) {
@@ -2004,6 +2036,12 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
   const uint32_t tmem = *tmem_slot;
   pdl_begin();  // everything above touched only shared memory and TMEM
 
+  // an epilogue warp has read all that it reads of a tile's accumulators
+  auto give_back = [&](int ab) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&acc_empty[ab]);
+  };
   if (warp > 0) {
     // the weights: 16-byte chunk e = (slice, column n, half of its 16 channels)
     const uint16_t* w = a.w + (int64_t)g * a.w_gs;
@@ -2070,11 +2108,15 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t acc = tmem + (uint32_t)(ab * np);
+      uint32_t acc = tmem + (uint32_t)(ab * npart * np);
       const uint64_t st = a_desc0 + ((uint32_t)sl * pitch >> 4);
       uint64_t bd = b_desc0;
       uint32_t on = 0;
       for (int kh = 0; kh < a.nkh; ++kh) {
+        if (kh > 0 && npart > 1) {
+          acc += (uint32_t)np;
+          on = 0;
+        }
         uint64_t ad = st + (uint32_t)kh * (sp::ROWB >> 4);
 #pragma unroll 4
         for (int r = 0; r < per_row; ++r) {
@@ -2178,8 +2220,11 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         float v[16];  // v[4 k + 2 row + b]: column 32 i + 8 k + 2 m + b
-        tmem_ld_16x256_x4(
-            tmem + ((uint32_t)(quarter * 32 + 16 * h) << 16) + (uint32_t)(ab * np + 64 * seg + 32 * i), v);
+        const uint32_t at = tmem + ((uint32_t)(quarter * 32 + 16 * h) << 16) +
+                            (uint32_t)(ab * npart * np + 64 * seg + 32 * i);
+        tmem_ld_16x256_x4(at, v);
+        tmem_add_16x256(at, npart, np, v);
+        if (seg == a.nseg - 1) give_back(ab);
 #pragma unroll
         for (int row = 0; row < 2; ++row) {
           // dx (+ the shortcut's share) masked by the layer below's ReLU, and that layer's sums
@@ -2198,9 +2243,6 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
         }
       }
       if (!ok) break;
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[ab]);
       if (++ab == nacc) {
         ab = 0;
         ph ^= 1;
@@ -2258,7 +2300,11 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
       for (int hs = 0; hs < (M / 64) * a.nseg; ++hs) {
         const int h = a.nseg == 2 ? hs >> 1 : hs, seg = a.nseg == 2 ? hs & 1 : 0;
         float v[32];  // v[4 k + 2 row + b]: column 8 k + 2 m + b of image row `row`
-        tmem_ld_16x256_x8(tmem + ((uint32_t)(quarter * 32 + 16 * h) << 16) + (uint32_t)(ab * np + 64 * seg), v);
+        const uint32_t at =
+            tmem + ((uint32_t)(quarter * 32 + 16 * h) << 16) + (uint32_t)(ab * npart * np + 64 * seg);
+        tmem_ld_16x256_x8(at, v);
+        tmem_add_16x256(at, npart, np, v);
+        if (hs == (M / 64) * a.nseg - 1) give_back(ab);
         const int64_t pix0 = ((int64_t)img * a.ho + (y_first + 2 * h) * a.rs + seg) * a.wo + sx * ps;
 #pragma unroll
         for (int row = 0; row < 2; ++row) {
@@ -2286,9 +2332,6 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
           }
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[ab]);
       if (++ab == nacc) {
         ab = 0;
         ph ^= 1;
@@ -2806,7 +2849,6 @@ bool conv_sp_plan(ConvSpArgs& a, int sms, int* cpr, size_t* smem) {
   a.box_rows = (a.tr - 1) * a.S + a.nkh;
   const size_t pitch = ((size_t)a.box_rows * sp::ROWB + 1023) / 1024 * 1024;
   const size_t fixed = 1024 + (size_t)a.nkh * a.nj * (a.ck / 16) * 64 * a.nseg * 32 + sp::AUX;
-  a.nacc = a.nseg == 2 ? 2 : 4;
   int per_sm = 2;
   size_t st = sp::kTwoPerSm > fixed ? (sp::kTwoPerSm - fixed) / pitch : 0;
   if (st < 2 || a.bwd.y) {
@@ -2815,6 +2857,8 @@ bool conv_sp_plan(ConvSpArgs& a, int sms, int* cpr, size_t* smem) {
   }
   if (st < 2) return false;
   a.nst = (int)std::min<size_t>(st, sp::MAX_ST);
+  a.npart = a.N == 16 || a.ck == 64 ? a.nkh : 1;
+  a.nacc = std::min(4, 512 / per_sm / (64 * a.nseg * a.npart));
   *smem = fixed + a.nst * pitch;
   *cpr = std::max(1, std::min(a.B * (a.hg / a.tr), per_sm * sms / a.G));
   return true;

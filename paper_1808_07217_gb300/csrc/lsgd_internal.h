@@ -261,8 +261,8 @@ struct ConvSpArgs {
   ConvBwdFuse bwd;
   // set by the launcher: columns / 64; output rows per input row group; row stride; first kernel row
   // and their number; first pixel (0 = the one left of the super-pixel) and their number; group
-  // rows, output size; tile rows, box rows; ring stages and accumulators
-  int nseg, rs, S, kh0, nkh, j0, nj, hg, ho, wo, tr, box_rows, nst, nacc;
+  // rows, output size; tile rows, box rows; ring stages; partial sums of a tile and tiles' accumulators
+  int nseg, rs, S, kh0, nkh, j0, nj, hg, ho, wo, tr, box_rows, nst, npart, nacc;
 };
 // The partials per replica that launch_conv_sp writes to stats or bwd.part (a number > 0 without
 // either), or 0 if it does not take the convolution.
