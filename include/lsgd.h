@@ -365,11 +365,11 @@ lsgd_status lsgd_batchnorm_stats(const float* y, int64_t P, int C, int G, float*
  *   dW[g][co][kh][kw][ci] = sum over b, oy, ox of dy[g][b][oy][ox][co] x[g][b][oy s + kh - 1][ox s + kw - 1][ci]
  * (x zero outside the image).  x [G][B][s Hout][s Wout][Cin] and dy [G][B][Hout][Wout][Cout] are
  * NHWC bf16 device arrays (16-byte aligned), dW [G][Cout][3][3][Cin] fp32 device, fully
- * overwritten.  The taps read shifted windows of input strips in shared memory (outputs narrower
- * than 8 pixels run on the fp32 cores); one fp32 partial per CTA (a scratch buffer allocated and
- * freed on `stream`) is summed in CTA order, so the result is deterministic.  Cin 16, 32 or 64; Cout a multiple of 16 up to 64; Wout dividing
- * 64 and Hout Wout a multiple of 64: LSGD_EINVAL otherwise, LSGD_ENOMEM if the scratch cannot be
- * allocated, LSGD_EUNSUPPORTED without tcgen05. */
+ * overwritten.  The taps read shifted windows of input strips in shared memory; one fp32 partial per
+ * CTA (a scratch buffer allocated and freed on `stream`) is summed in CTA order, so the result is
+ * deterministic.  Cin 16, 32 or 64; Cout a multiple of 16 up to 64; Wout dividing 64 and Hout Wout a
+ * multiple of 64: LSGD_EINVAL otherwise, LSGD_ENOMEM if the scratch cannot be allocated,
+ * LSGD_EUNSUPPORTED without tcgen05. */
 lsgd_status lsgd_conv_wgrad_bf16(const uint16_t* x, const uint16_t* dy, float* dW, int G, int B,
                                  int Hout, int Wout, int Cin, int Cout, int stride, void* stream);
 

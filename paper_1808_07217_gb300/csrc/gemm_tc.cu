@@ -2408,6 +2408,13 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
 // 3 x 64 channels) in TMEM; it writes its partial dW, and a second kernel adds the CTAs' partials
 // in order.  Rows m beyond the third kernel row multiply whatever lies behind the strip and are
 // never read.
+//
+// Outputs narrower than 8 pixels have no 16 pixels in a row or two, so their tiles run down the image
+// columns instead (ConvWgradGeom::cols): a strip row is one column of the input under the tile's
+// kp / Wout rows, a box of its own (columns start at whole swizzle atoms: `pitch`), the output-gradient
+// tile is Wout columns likewise, and kernel rows and columns change places.  On the fp32 cores, which
+// staged 8-pixel rows and left tensor cores idle, 16 workers x 128 images of 64 x 1 pixels and 64 x 64
+// channels took 4,332 us, of 16 x 4 pixels 1,094 (a gathered column matrix 31 and 33); so 20 and 23.
 //   warp 0      TMA producer (strip(s) + output-gradient tile per stage)
 //   warp 1      MMA issuer: per 16 pixels and kernel column one tcgen05.mma (two for 64 channels)
 //   warp 2      TMEM allocation
@@ -2431,7 +2438,8 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
   const ConvWgradGeom& gm = a.geom;
   const int cin = a.cin, nst = gm.stages;
   const uint32_t rowb = (uint32_t)cin * 2;               // bytes of one pixel
-  const uint32_t strip_bytes = (uint32_t)gm.rows * gm.wp * rowb, strip_pitch = up1k(strip_bytes);
+  const uint32_t row_bytes = (uint32_t)gm.pitch * rowb;  // one strip row
+  const uint32_t strip_pitch = up1k(gm.rows * row_bytes);
   const uint32_t tile_b = (uint32_t)gm.kp * a.nb * 2;
   const uint32_t stage_pitch = gm.strips * strip_pitch + up1k(tile_b);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + nst * stage_pitch + gm.pad);
@@ -2477,10 +2485,20 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
       if (!mbar_wait_warp(&empty[s], ph)) break;
       uint8_t* st = base + s * stage_pitch;
       if (el) {
-        mbar_expect_tx(&full[s], gm.strips * strip_bytes + tile_b);
-        tma_load_5d(st, &a.x_map, &full[s], 0, -1, y * a.stride - 1, b, g);
-        if (gm.strips == 2) tma_load_5d(st + strip_pitch, &a.x_map, &full[s], 0, 0, y * a.stride - 1, b, g);
-        tma_load_3d(st + gm.strips * strip_pitch, &a.dy_map, &full[s], 0, p0, g);
+        mbar_expect_tx(&full[s], (uint32_t)(gm.strips * gm.rows * gm.wp) * rowb + tile_b);
+        uint8_t* tile = st + gm.strips * strip_pitch;
+        if (!gm.cols) {
+          tma_load_5d(st, &a.x_map, &full[s], 0, -1, y * a.stride - 1, b, g);
+          if (gm.strips == 2) tma_load_5d(st + strip_pitch, &a.x_map, &full[s], 0, 0, y * a.stride - 1, b, g);
+          tma_load_3d(tile, &a.dy_map, &full[s], 0, p0, g);
+        } else {
+          for (int r = 0; r < gm.rows; ++r)
+            for (int i = 0; i < gm.strips; ++i)
+              tma_load_5d(st + i * strip_pitch + r * row_bytes, &a.x_map, &full[s], 0, r - 1,
+                          y * a.stride - 1 + i, b, g);
+          for (int x = 0; x < a.wout; ++x)
+            tma_load_5d(tile + (uint32_t)(x * gm.inner * a.nb) * 2, &a.dy_map, &full[s], 0, x, y, b, g);
+        }
       }
       p0 += gm.kp;
       y += R;
@@ -2502,17 +2520,17 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
     const uint32_t idesc0 = make_idesc(m0, a.nb, true, true), idesc1 = make_idesc(64, a.nb, true, true);
     const uint32_t ux = rowb >> 4;  // one strip pixel in the descriptors' 16-byte units
     // along k: eight pixels to the next core group (a whole output row where rows are 8 wide);
-    // along m: one strip row to the next kernel row
-    const uint32_t row_px = (uint32_t)gm.wp * a.stride;  // strip pixels from one output row to the next
+    // along m: one strip row to the next kernel row (columns: kernel column)
+    const uint32_t row_px = (uint32_t)gm.pitch * a.stride;  // strip pixels from one output row to the next
     const uint64_t a_desc0 =
-        smem_desc_swz(smem_u32(base), gm.wp * rowb, (a.wout == 8 ? row_px : 8u) * rowb, rowb);
+        smem_desc_swz(smem_u32(base), row_bytes, (gm.inner == 8 ? row_px : 8u) * rowb, rowb);
     const uint64_t b_desc0 = smem_desc_swz(smem_u32(base) + gm.strips * strip_pitch, 16u * a.nb,
                                            16u * a.nb, 2u * a.nb);
-    // kernel column kw: which strip and how many pixels into it
+    // kernel column kw (columns: kernel row): which strip and how many pixels into it
     const uint32_t col1 = a.stride == 1 ? ux : strip_pitch >> 4, col2 = a.stride == 1 ? 2 * ux : ux;
-    const uint32_t mt_off = 2u * gm.wp * ux;  // kernel row 2 of 64 channels
+    const uint32_t mt_off = 2u * gm.pitch * ux;  // the third row group of 64 channels
     const uint32_t acc_kw = (uint32_t)(mt_n * a.nb);
-    const int lw = 31 - __clz(a.wout);
+    const int lw = 31 - __clz(gm.inner);
     bool ok = true;
     int s = 0;
     uint32_t ph = 0, acc = 0;
@@ -2528,7 +2546,7 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
       for (int k = 0; k < 8; ++k) {
         if (16 * k >= gm.kp) break;
         // the 16 pixels from 16 k on: their output row and the column in it
-        const uint64_t ad = ad0 + (((16u * k) >> lw) * row_px + ((16u * k) & (a.wout - 1))) * ux;
+        const uint64_t ad = ad0 + (((16u * k) >> lw) * row_px + ((16u * k) & (gm.inner - 1))) * ux;
         const uint64_t bd = bd0 + (uint32_t)(2 * a.nb * k);
         if (el) {
           mma_bf16(tmem, ad, bd, idesc0, acc);
@@ -2556,20 +2574,20 @@ __global__ void __launch_bounds__(cw::THREADS, 1) conv_wgrad_tc_kernel(
   if (nt > 0 && __all_sync(0xffffffffu, mbar_wait(acc_full, 0) ? 1 : 0)) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     float* out = a.part + ((int64_t)g * cpr + q) * a.cout * 9 * cin;
-    for (int kw = 0; kw < 3; ++kw)
+    for (int t = 0; t < 3; ++t)  // the tap along the strip's rows; th across them
       for (int mt = 0; mt < mt_n; ++mt) {
         // TMEM lane -> row m: all 128 lanes of an M = 128 accumulator, the first 16 of each warp's
         // 32 of an M = 64 one
         const bool half = cin == 16 || mt == 1;
         const int m = half ? warp * 16 + lane : warp * 32 + lane;
-        const int kh = 2 * mt + m / cin, ci = m % cin;
-        const bool row_ok = kh < 3 && (!half || lane < 16);
+        const int th = 2 * mt + m / cin, ci = m % cin, tap = gm.cols ? t * 3 + th : th * 3 + t;
+        const bool row_ok = th < 3 && (!half || lane < 16);
         for (int c0 = 0; c0 < a.cout; c0 += 16) {
           float v[16];
-          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((kw * mt_n + mt) * a.nb + c0), v);
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((t * mt_n + mt) * a.nb + c0), v);
           if (row_ok) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) out[((int64_t)(c0 + i) * 9 + kh * 3 + kw) * cin + ci] = v[i];
+            for (int i = 0; i < 16; ++i) out[((int64_t)(c0 + i) * 9 + tap) * cin + ci] = v[i];
           }
         }
       }
@@ -3014,24 +3032,26 @@ bool conv_wgrad_tc_ok(int cin, int cout, int stride, int hin, int win, int hout,
   return (hout * wout) % 64 == 0 && win == wout * stride && hin == hout * stride;
 }
 
-// Outputs at least 8 wide: 16 pixels are then within a row, or two whole rows (narrower ones run
-// on the fp32 cores).
+// Rows at least 8 wide: 16 pixels are then within a row, or two whole rows.  Narrower ones: 16 pixels are
+// within a column of the tile's kp / wout (16 to 128) rows.
 bool conv_wgrad_geom(int cin, int cout, int stride, int hout, int wout, ConvWgradGeom* gm) {
-  if (wout < 8) return false;
   const int nb = conv_wgrad_nb(cout);
+  gm->cols = wout < 8;
   gm->strips = stride;
-  gm->wp = stride == 1 ? wout + 2 : wout + 1;
   uint32_t cols = 32;
   while (cols < (uint32_t)(3 * (cin == 64 ? 2 : 1) * nb)) cols <<= 1;
   gm->tmem_cols = cols;
   // 128-pixel tiles where an image has them: fewer stage handshakes, less halo
   for (int kp = (hout * wout) % 128 == 0 ? 128 : 64; kp >= 64; kp -= 64) {
     gm->kp = kp;
-    gm->rows = (kp / wout - 1) * stride + 3;
-    // the unread rows of the last strip's operand end at most (fourth kernel row) one strip row
+    gm->inner = gm->cols ? kp / wout : wout;
+    gm->rows = (kp / gm->inner - 1) * stride + 3;
+    gm->wp = gm->inner + (stride == 1 ? 2 : 1);
+    gm->pitch = gm->cols ? (gm->wp + 7) / 8 * 8 : gm->wp;
+    // the unread rows of the last strip's operand end at most (fourth row group) one strip row
     // behind the strip; the tile follows it, and this pad where the tile is smaller
-    gm->pad = (int)up1k((uint32_t)gm->wp * cin * 2);
-    const size_t stage = gm->strips * (size_t)up1k((uint32_t)(gm->rows * gm->wp * cin * 2)) +
+    gm->pad = (int)up1k((uint32_t)gm->pitch * cin * 2);
+    const size_t stage = gm->strips * (size_t)up1k((uint32_t)(gm->rows * gm->pitch * cin * 2)) +
                          up1k((uint32_t)(kp * nb * 2));
     const size_t fixed = 1024 + gm->pad + (2 * cw::MAX_ST + 1) * 8 + 16;
     const size_t n2 = (cw::kTwoPerSm - fixed) / stage, n1 = (cw::kOnePerSm - fixed) / stage;
@@ -3039,40 +3059,52 @@ bool conv_wgrad_geom(int cin, int cout, int stride, int hout, int wout, ConvWgra
     gm->per_sm = n2 >= 3 && 2 * cols <= 512 ? 2 : 1;
     gm->stages = (int)std::min<size_t>(cw::MAX_ST, gm->per_sm == 2 ? n2 : n1);
     gm->smem = fixed + gm->stages * stage;
-    if (gm->stages >= 2 && gm->rows <= 256) return true;
+    // (the pixels that a strip row spans and its rows are TMA box extents)
+    if (gm->stages >= 2 && gm->rows <= 256 && (gm->wp - 1) * stride + 1 <= 256) return true;
   }
   return false;
 }
 
 int conv_wgrad_ctas(int cin, int cout, int stride, int hout, int wout, int B, int G) {
   ConvWgradGeom gm;
-  if (!conv_wgrad_geom(cin, cout, stride, hout, wout, &gm))
-    return conv_wgrad_simt_ranges(G, B, hout, wout, cin, cout);
+  if (!conv_wgrad_geom(cin, cout, stride, hout, wout, &gm)) return 1;  // launch_conv_wgrad_tc rejects it
   const int64_t tiles = (int64_t)B * hout * wout / gm.kp;
   return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)kNumSMs * gm.per_sm / std::max(G, 1)));
 }
 
-bool make_tma_map_strip(CUtensorMap* map, const void* base, int cin, int win, int hin, int B, int G,
-                        int stride, const ConvWgradGeom& gm) {
+namespace {
+// A box of box_c channels x (span_w, span_h) pixels, every step_w-th / step_h-th of them, of an NHWC bf16
+// array [G][B][H][W][C].
+bool encode_nhwc(CUtensorMap* map, const void* base, int C, int W, int H, int B, int G, int box_c, int span_w,
+                 int span_h, int step_w, int step_h) {
   std::call_once(g_encode_once, load_encode);
-  if (!g_encode || (cin != 16 && cin != 32 && cin != 64) || (reinterpret_cast<uintptr_t>(base) & 15))
+  if (!g_encode || (box_c != 16 && box_c != 32 && box_c != 64) || (reinterpret_cast<uintptr_t>(base) & 15) ||
+      span_w > 256 || span_h > 256)
     return false;
-  const int span = (gm.wp - 1) * stride + 1;  // columns a strip row spans
-  if (span > 256 || gm.rows > 256) return false;
   const uint64_t e = 2;
-  cuuint64_t dims[5] = {(cuuint64_t)cin, (cuuint64_t)win, (cuuint64_t)hin, (cuuint64_t)B,
-                        (cuuint64_t)G};
-  cuuint64_t strides[4] = {(cuuint64_t)cin * e, (cuuint64_t)win * cin * e,
-                           (cuuint64_t)hin * win * cin * e, (cuuint64_t)B * hin * win * cin * e};
-  cuuint32_t box[5] = {(cuuint32_t)cin, (cuuint32_t)span, (cuuint32_t)gm.rows, 1, 1};
-  cuuint32_t estr[5] = {1, (cuuint32_t)stride, 1, 1, 1};
-  const CUtensorMapSwizzle sw = cin == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                          : (cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                                       : CU_TENSOR_MAP_SWIZZLE_32B);
+  cuuint64_t dims[5] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B, (cuuint64_t)G};
+  cuuint64_t strides[4] = {(cuuint64_t)C * e, (cuuint64_t)W * C * e, (cuuint64_t)H * W * C * e,
+                           (cuuint64_t)B * H * W * C * e};
+  cuuint32_t box[5] = {(cuuint32_t)box_c, (cuuint32_t)span_w, (cuuint32_t)span_h, 1, 1};
+  cuuint32_t estr[5] = {1, (cuuint32_t)step_w, (cuuint32_t)step_h, 1, 1};
+  const CUtensorMapSwizzle sw = box_c == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                            : (box_c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                           : CU_TENSOR_MAP_SWIZZLE_32B);
   CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims,
                         strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+}  // namespace
+
+bool make_conv_wgrad_maps(ConvWgradArgs* a, const ConvWgradGeom& gm, const void* x, const void* dy, int B) {
+  const int span = (gm.wp - 1) * a->stride + 1;  // pixels that a strip row spans
+  if (gm.cols)
+    return encode_nhwc(&a->x_map, x, a->cin, a->win, a->hin, B, a->G, a->cin, 1, span, 1, a->stride) &&
+           encode_nhwc(&a->dy_map, dy, a->cout, a->wout, a->hout, B, a->G, a->nb, 1, gm.inner, 1, 1);
+  return encode_nhwc(&a->x_map, x, a->cin, a->win, a->hin, B, a->G, a->cin, span, gm.rows, a->stride, 1) &&
+         make_tma_map(&a->dy_map, dy, true, a->cout, a->P, a->G, a->cout, (uint64_t)a->P * a->cout, a->nb,
+                      gm.kp, 2 * a->nb);
 }
 
 cudaError_t launch_conv_wgrad_tc(const ConvWgradArgs& a, cudaStream_t stream) {

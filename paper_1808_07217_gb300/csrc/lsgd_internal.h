@@ -270,14 +270,15 @@ int conv_sp_parts(const ConvSpArgs& a);
 cudaError_t launch_conv_sp(const ConvSpArgs& a, const void* in, cudaStream_t stream);
 // Weight gradient of a 3x3 convolution (zero padding 1, stride 1 or 2) on the tensor cores:
 // part[g][q][co][t Cin + ci] = the sum over CTA q's output pixels of dy[g][p][co] x[g][src_t(p)][ci],
-// src_t(p) the input pixel under tap t of output pixel p (zero outside the image).  x_map:
-// make_tma_map_strip over the NHWC input; dy_map: rank-3 bf16 map over [G][P][Cout] with box
-// {nb, kp} and a 2 nb-byte swizzle.  Cin 16 / 32 / 64, Cout a multiple of 16 up to 64, Wout dividing
-// 64, Hout Wout a multiple of 64.
+// src_t(p) the input pixel under tap t of output pixel p (zero outside the image).  Cin 16 / 32 / 64,
+// Cout a multiple of 16 up to 64, Wout dividing 64, Hout Wout a multiple of 64.
 struct ConvWgradGeom {
   int kp;       // output pixels per tile: whole rows of one image
-  int rows, wp; // the input strip's rows and its width in pixels
-  int strips;   // 1, or 2 at stride 2 (odd and even columns)
+  int cols;     // 1: the tile is walked down its columns (kernel rows and columns change places)
+  int inner;    // output pixels of a row (columns: of a column) of the tile
+  int rows, wp; // the input strip's rows (columns: columns) and the pixels of each
+  int pitch;    // pixels from one strip row to the next
+  int strips;   // 1, or 2 at stride 2 (odd and even columns; columns: rows)
   int stages, per_sm, pad;
   uint32_t tmem_cols;
   size_t smem;
@@ -289,18 +290,18 @@ struct ConvWgradArgs {
   int cin, cout, stride, hin, win, hout, wout, G, P;
   int cpr;      // CTAs (partials) per replica, from conv_wgrad_ctas
   float* part;  // [G][cpr][cout][9 cin]
-  int nb;       // the MMAs' N and the output-gradient tile's channels (conv_wgrad_nb; dy_map's box)
+  int nb;       // the MMAs' N and the output-gradient tile's channels (conv_wgrad_nb)
   ConvWgradGeom geom;  // set by the launcher
 };
 bool conv_wgrad_tc_ok(int cin, int cout, int stride, int hin, int win, int hout, int wout);
-// The kernel's launch shape; false: the shape (accepted by conv_wgrad_tc_ok) runs on the fp32 cores.
+// The kernel's launch shape (true for every shape that conv_wgrad_tc_ok accepts).
 bool conv_wgrad_geom(int cin, int cout, int stride, int hout, int wout, ConvWgradGeom* gm);
-// Partials per replica of either.
+// Partials per replica.
 int conv_wgrad_ctas(int cin, int cout, int stride, int hout, int wout, int B, int G);
-// One tile's input strip: rank-5 map {Cin, Win, Hin, B, G}, every `stride`-th column, all rows,
-// swizzled at the 2 Cin-byte pixel.
-bool make_tma_map_strip(CUtensorMap* map, const void* base, int cin, int win, int hin, int B, int G,
-                        int stride, const ConvWgradGeom& gm);
+// x_map and dy_map of `a` (sizes and nb set) over x [G][B][hin][win][cin] and dy [G][B][hout][wout][cout],
+// 16-byte aligned: one tile's input strip(s), every `stride`-th column (columns: row) of it, swizzled at
+// the 2 cin-byte pixel, and its output gradients, swizzled at 2 nb bytes.
+bool make_conv_wgrad_maps(ConvWgradArgs* a, const ConvWgradGeom& gm, const void* x, const void* dy, int B);
 cudaError_t launch_conv_wgrad_tc(const ConvWgradArgs& a, cudaStream_t stream);
 // The tile geometry of an implicit convolution with an Hout x Wout output: whole output rows,
 // 128 pixels per tile.  False when the shape does not tile that way.

@@ -1161,36 +1161,22 @@ cudaError_t launch_conv_wgrad_impl(const uint16_t* x, const uint16_t* dy, float*
     return cudaErrorInvalidValue;
   const int cpr = conv_wgrad_ctas(cin, cout, stride, hout, wout, B, G);
   ConvWgradGeom gm;
-  cudaError_t e;
-  if (conv_wgrad_geom(cin, cout, stride, hout, wout, &gm)) {
-    ConvWgradArgs a{};
-    a.nb = conv_wgrad_nb(cout);
-    if (!make_tma_map_strip(&a.x_map, x, cin, win, hin, B, G, stride, gm) ||
-        !make_tma_map(&a.dy_map, dy, true, cout, P, G, cout, (uint64_t)P * cout, a.nb, gm.kp, 2 * a.nb))
-      return cudaErrorInvalidValue;
-    a.cin = cin;
-    a.cout = cout;
-    a.stride = stride;
-    a.hin = hin;
-    a.win = win;
-    a.hout = hout;
-    a.wout = wout;
-    a.G = G;
-    a.P = (int)P;
-    a.cpr = cpr;
-    a.part = part;
-    e = launch_conv_wgrad_tc(a, s);
-  } else {
-    ConvSimtArgs a{};
-    a.bf16 = true;
-    a.G = G;
-    a.B = B;
-    a.hin = hin, a.win = win, a.cin = cin;
-    a.hout = hout, a.wout = wout, a.cout = cout;
-    a.stride = stride;
-    a.in = x;
-    e = launch_conv_wgrad_simt(a, dy, part, s);
-  }
+  ConvWgradArgs a{};
+  a.nb = conv_wgrad_nb(cout);
+  a.cin = cin;
+  a.cout = cout;
+  a.stride = stride;
+  a.hin = hin;
+  a.win = win;
+  a.hout = hout;
+  a.wout = wout;
+  a.G = G;
+  a.P = (int)P;
+  a.cpr = cpr;
+  a.part = part;
+  if (!conv_wgrad_geom(cin, cout, stride, hout, wout, &gm) || !make_conv_wgrad_maps(&a, gm, x, dy, B))
+    return cudaErrorInvalidValue;
+  const cudaError_t e = launch_conv_wgrad_tc(a, s);
   if (e != cudaSuccess) return e;
   // the partials' sum, cropped to the first cin_out channels of every tap
   if (defer && deferred && sum_partials_v4_ok(part, 9 * cin, 9 * cin_out, dW, dW_gs, cin, cin_out)) {

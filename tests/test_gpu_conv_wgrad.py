@@ -63,7 +63,7 @@ def test_conv_wgrad_matches_fp64(P, shape):
     want, scale = _reference(x.float().cpu().numpy().astype(np.float64),
                              dy.float().cpu().numpy().astype(np.float64), s)
     got = dW.cpu().numpy().astype(np.float64)
-    err = np.abs(got - want) / scale
+    err = np.abs(got - want) / np.maximum(scale, 1e-30)  # a tap that never meets the image: exactly zero
     assert np.isfinite(got).all()
     assert err.max() <= 1e-5, err.max()
 
@@ -100,6 +100,34 @@ def test_conv_wgrad_rejects_unsupported_shapes(P):
 @pytest.mark.parametrize("shape", [(2, 3, 2, 64, 16, 16, 1), (1, 2, 4, 64, 64, 64, 2),   # widest rows
                                    (2, 3, 2, 32, 32, 16, 1), (1, 5, 4, 16, 64, 32, 2),   # 64-pixel tiles
                                    (3, 2, 16, 8, 16, 48, 1), (1, 9, 16, 8, 32, 64, 2),   # two rows per step
-                                   (2, 3, 16, 4, 16, 32, 1), (1, 2, 32, 2, 32, 16, 2)])  # narrower than 8
+                                   # narrower than 8: tiles of 64 and of 128 pixels down the columns
+                                   (2, 3, 16, 4, 16, 32, 1), (1, 2, 32, 2, 32, 16, 2), (3, 5, 64, 1, 64, 48, 1),
+                                   (2, 3, 128, 1, 32, 32, 1), (1, 3, 128, 1, 16, 16, 2), (2, 7, 64, 2, 16, 64, 1),
+                                   (1, 2, 96, 2, 32, 16, 2), (1, 3, 160, 4, 64, 64, 1), (2, 2, 32, 4, 64, 32, 2),
+                                   (1, 5, 48, 4, 32, 48, 2), (20, 9, 64, 1, 64, 64, 2)])
 def test_conv_wgrad_tile_edges(P, shape):
     test_conv_wgrad_matches_fp64(P, shape)
+
+
+def test_conv_wgrad_of_narrow_outputs_runs_on_the_tensor_cores(P):
+    # the same pixels, channels and products as 64 x 1, 16 x 4 and 8 x 8 images.  Narrow rows cost more
+    # loads per tile, at most ten for an 8-pixel row's two; the fp32 cores take fifty times the 8 x 8 time.
+    import torch
+
+    def us(Hout, Wout, G=16, B=128, C=64):
+        x = torch.ones((G, B, Hout, Wout, C), device="cuda", dtype=torch.bfloat16)
+        dW = torch.empty((G, C, 3, 3, C), device="cuda")
+        times = []
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(10):
+                P.lsgd_conv_wgrad_bf16(x, x, dW, G, B, Hout, Wout, C, C, 1)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        return min(times)
+
+    wide = us(8, 8)
+    assert us(64, 1) <= 5 * wide
+    assert us(16, 4) <= 5 * wide
