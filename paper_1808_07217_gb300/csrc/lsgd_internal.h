@@ -246,8 +246,8 @@ cudaError_t launch_conv_tc(const ConvArgs& a, cudaStream_t stream, int* ctas_per
 int conv_tc_ctas(const ConvArgs& a);
 // The same convolutions where an image row is 512 channel values (wi ck = 512) and the output's
 // pixels over one 64-value super-pixel of it give 64 columns (conv_sp_kernel): input [G][B][hi][wi][ck]
-// bf16, weights w [N][9][ck] bf16 per replica (stride w_gs), output [G][B][ho][wo][N] fp32, 32-byte
-// aligned.  phases: the input is the output gradient of a stride-2 layer and w its four parity
+// bf16, weights w [N][9][ck] bf16 per replica (stride w_gs), output [G][B][ho][wo][N] fp32, 16-byte
+// aligned (32 with bwd).  phases: the input is the output gradient of a stride-2 layer and w its four parity
 // phases' weights (stride w_ps between phases, flip_phase_weights_kernel); the output has twice the
 // rows and columns.  stats and bwd as in ConvArgs (part_off unused; bwd.sc_stride 2 only with phases).
 struct ConvSpArgs {

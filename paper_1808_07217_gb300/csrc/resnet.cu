@@ -1322,10 +1322,11 @@ size_t conv_wt_elems(int G, int cin, int cout, int stride) {
 }
 
 // The partials per replica of a convolution on conv_sp_kernel (conv_sp_parts), 0 where it does not take it (its
-// shape, or buffers that its 32-byte accesses of the output and 16-byte ones of the weights reject).
+// shape, or buffers that its 16-byte accesses of output and weights -- 32 with the BatchNorm backward, all in
+// buffers of the step -- reject).
 int conv_sp_takes(const ConvSpArgs& a) {
   auto al = [](const void* p, uintptr_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; };
-  if (!al(a.out, 32) || a.out_gs % 8 || !al(a.w, 16) || a.w_gs % 8 || a.w_ps % 8) return 0;
+  if (!al(a.out, a.bwd.y ? 32 : 16) || a.out_gs % 8 || !al(a.w, 16) || a.w_gs % 8 || a.w_ps % 8) return 0;
   if (a.bwd.y && (!al(a.bwd.y, 32) || !al(a.bwd.mask, 32) || (a.bwd.sc_dout && (!al(a.bwd.sc_dout, 32) ||
                                                                                !al(a.bwd.sc_out, 32)))))
     return 0;

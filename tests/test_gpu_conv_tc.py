@@ -270,3 +270,34 @@ def test_conv_output_alignment_does_not_change_results(P):
     P.lsgd_conv3x3_bf16(P.CONV_FORWARD, x, w, y16, G, B, H, H, Cin, Cout, 1)
     torch.cuda.synchronize()
     assert torch.equal(y, y16)
+
+
+@pytest.mark.parametrize("mode,H,Cin,Cout,s", [(0, 32, 16, 16, 1), (0, 32, 16, 32, 2), (0, 32, 3, 16, 1),
+                                               (0, 16, 32, 32, 1), (0, 8, 64, 64, 1), (1, 32, 16, 16, 1),
+                                               (1, 32, 16, 32, 2), (1, 8, 64, 64, 1)])
+def test_conv_output_alignment_does_not_change_the_512_value_rows(P, mode, H, Cin, Cout, s):
+    # the same for the super-pixel kernel, whose order of sums is not the tap kernel's: it has to take
+    # every output that the entry point takes
+    import torch
+
+    G, B, Ho = 3, 4, H // s
+    ishape, oshape = ((G, B, H, H, Cin), (G, B, Ho, Ho, Cout))[::1 if mode == 0 else -1]
+    gen = torch.Generator(device="cuda").manual_seed(19)
+    x = _bf16_randn(torch, ishape, gen)
+    w = _bf16_randn(torch, (G, Cout, 3, 3, Cin), gen)
+    out = torch.empty(oshape, device="cuda")
+    buf = torch.full((out.numel() + 8,), float("nan"), device="cuda")
+    out16 = buf[4:-4].view(oshape)
+    assert out16.data_ptr() % 32 == 16
+    for o in (out, out16):
+        P.lsgd_conv3x3_bf16(mode, x, w, o, G, B, H, H, Cin, Cout, s)
+    torch.cuda.synchronize()
+    assert torch.equal(out, out16)
+    assert torch.isnan(buf[:4]).all() and torch.isnan(buf[-4:]).all()
+    if mode == 0:
+        stats = [torch.empty((G, Cout), device="cuda") for _ in range(4)]
+        P.lsgd_conv3x3_bn_bf16(x, w, out, stats[0], stats[1], G, B, H, H, Cin, Cout, s)
+        P.lsgd_conv3x3_bn_bf16(x, w, out16, stats[2], stats[3], G, B, H, H, Cin, Cout, s)
+        torch.cuda.synchronize()
+        assert torch.equal(out, out16)
+        assert torch.equal(stats[0], stats[2]) and torch.equal(stats[1], stats[3])
