@@ -385,7 +385,7 @@ lsgd_status lsgd_conv_wgrad_bf16(const uint16_t* x, const uint16_t* dy, float* d
  *          iy = oy s + kh - 1, ix = ox s + kw - 1 and co of in[g][b][oy][ox][co] W[g][co][kh][kw][ci]
  *          with in = dy [G][B][Hout][Wout][Cout] and out = dx [G][B][Hin][Win][Cin]; stride 1 as
  *          a convolution with the flipped, transposed weights, stride 2 as four parity phases.
- * bf16 operands, fp32 accumulation; `out` fp32, fully overwritten.  Device pointers, in and W
+ * bf16 operands, fp32 accumulation; `out` fp32, fully overwritten.  Device pointers, all three
  * 16-byte aligned, asynchronous on `stream`; scratch (the padded stem operands or the flipped
  * weights) is allocated and freed on `stream`.  LSGD_EINVAL on bad arguments, LSGD_EUNSUPPORTED
  * for shapes the kernel does not take (it needs 16, 32 or 64 channels per tap, Cout and Cin (mode

@@ -2288,7 +2288,7 @@ cudaError_t launch_batchnorm_stats(const float* y, int64_t P, int C, int G, floa
   const int64_t nq = (P + kStatChunk - 1) / kStatChunk;
   if (nq > 65535) return cudaErrorInvalidValue;
   const int lanes = std::max(1, 256 / C);
-  if (vec4_ok(C))
+  if (vec4_ok(C) && (reinterpret_cast<uintptr_t>(y) & 15) == 0)
     launch_pdl(bn_stats_partial_v4_kernel, dim3((unsigned)nq, (unsigned)G), 256, 0, s, y, P, C,
         (int)nq, kStatChunk, part);
   else

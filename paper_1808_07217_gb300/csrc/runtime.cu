@@ -1827,8 +1827,8 @@ lsgd_status lsgd_conv3x3_bf16(int mode, const uint16_t* in, const uint16_t* W, f
   if (!in || !W || !out || (mode != 0 && mode != 1) || G < 1 || G > 65535 || B < 1 || Hin < 1 ||
       Win < 1 || Cin < 1 || Cout < 1 || (stride != 1 && stride != 2))
     return fail(nullptr, LSGD_EINVAL, "lsgd_conv3x3_bf16: bad arguments");
-  if (((uintptr_t)in & 15) || ((uintptr_t)W & 15))
-    return fail(nullptr, LSGD_EINVAL, "lsgd_conv3x3_bf16: operands must be 16-byte aligned");
+  if (((uintptr_t)in & 15) || ((uintptr_t)W & 15) || ((uintptr_t)out & 15))
+    return fail(nullptr, LSGD_EINVAL, "lsgd_conv3x3_bf16: operands and output must be 16-byte aligned");
   if (!lsgd::tc_available()) return fail(nullptr, LSGD_EUNSUPPORTED, "tcgen05 not available");
   if (!lsgd::conv3x3_tc_route(mode, B, Hin, Win, Cin, Cout, stride))
     return fail(nullptr, LSGD_EUNSUPPORTED,
@@ -1854,8 +1854,8 @@ lsgd_status lsgd_conv3x3_bn_bf16(const uint16_t* x, const uint16_t* W, float* y,
   if (!x || !W || !y || !mean || !rstd || G < 1 || G > 65535 || B < 1 || Hin < 1 || Win < 1 ||
       Cin < 1 || Cout < 1 || (stride != 1 && stride != 2))
     return fail(nullptr, LSGD_EINVAL, "lsgd_conv3x3_bn_bf16: bad arguments");
-  if (((uintptr_t)x & 15) || ((uintptr_t)W & 15))
-    return fail(nullptr, LSGD_EINVAL, "lsgd_conv3x3_bn_bf16: operands must be 16-byte aligned");
+  if (((uintptr_t)x & 15) || ((uintptr_t)W & 15) || ((uintptr_t)y & 15))
+    return fail(nullptr, LSGD_EINVAL, "lsgd_conv3x3_bn_bf16: operands and output must be 16-byte aligned");
   if (!lsgd::tc_available()) return fail(nullptr, LSGD_EUNSUPPORTED, "tcgen05 not available");
   if (!lsgd::conv3x3_tc_route(0, B, Hin, Win, Cin, Cout, stride) || Cout > 64)
     return fail(nullptr, LSGD_EUNSUPPORTED,

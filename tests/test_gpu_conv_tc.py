@@ -301,3 +301,21 @@ def test_conv_output_alignment_does_not_change_the_512_value_rows(P, mode, H, Ci
         torch.cuda.synchronize()
         assert torch.equal(out, out16)
         assert torch.equal(stats[0], stats[2]) and torch.equal(stats[1], stats[3])
+
+
+def test_conv_rejects_outputs_that_are_not_16_byte_aligned(P):
+    # the kernels store 16 bytes at a time: the host refuses before anything is launched
+    import torch
+
+    G, B, H, C = 1, 2, 32, 16
+    x = torch.zeros((G, B, H, H, C), device="cuda", dtype=torch.bfloat16)
+    w = torch.zeros((G, C, 3, 3, C), device="cuda", dtype=torch.bfloat16)
+    out = torch.zeros(G * B * H * H * C + 4, device="cuda")
+    m, r = torch.zeros((G, C), device="cuda"), torch.zeros((G, C), device="cuda")
+    for off in (1, 2, 3):
+        for call in (lambda: P.lsgd_conv3x3_bf16(P.CONV_FORWARD, x, w, out[off:], G, B, H, H, C, C, 1),
+                     lambda: P.lsgd_conv3x3_bf16(P.CONV_DGRAD, x, w, out[off:], G, B, H, H, C, C, 1),
+                     lambda: P.lsgd_conv3x3_bn_bf16(x, w, out[off:], m, r, G, B, H, H, C, C, 1)):
+            with pytest.raises(P.LsgdError) as e:
+                call()
+            assert e.value.status == P.EINVAL

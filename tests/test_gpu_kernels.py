@@ -184,3 +184,18 @@ def test_batchnorm_stats(P, torch, G, n, C):
     np.testing.assert_allclose(rstd.cpu().numpy(), r, rtol=1e-4)
     with pytest.raises(P.LsgdError):
         P.lsgd_batchnorm_stats(y, n, 300, G, mean, rstd)
+
+
+def test_batchnorm_stats_of_a_view_that_is_not_16_byte_aligned(P, torch):
+    # element loads instead of 16-byte ones: another order of the same fp32 sums, over at most 1,024 values
+    G, n, C = 2, 3000, 16
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    buf = torch.randn(G * n * C + 4, device="cuda", generator=gen) * 2.0 + 5.0
+    for off in range(4):
+        y = buf[off:off + G * n * C].view(G, n, C)
+        mean = torch.empty((G, C), device="cuda")
+        rstd = torch.empty((G, C), device="cuda")
+        P.lsgd_batchnorm_stats(y, n, C, G, mean, rstd)
+        yn = y.double().cpu().numpy()
+        np.testing.assert_allclose(mean.cpu().numpy(), yn.mean(axis=1), rtol=1e-5)
+        np.testing.assert_allclose(rstd.cpu().numpy(), 1.0 / np.sqrt(yn.var(axis=1) + 1e-5), rtol=1e-4)
