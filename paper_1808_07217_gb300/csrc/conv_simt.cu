@@ -356,11 +356,11 @@ cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
 // walks its row four pixels at a time: one load per pixel of dy and of x (two at stride 2; the
 // columns that the three kernel columns share stay in registers), 24 packed multiply-adds.  At the end
 // the four rows' sums are added in a fixed order.
-// An accumulator's chain is a tile range's pixels / 4 (a few hundred roundings; one thread used to
-// add 2,048).
+// An accumulator's chain is a tile range's pixels / 4: at most 32 kWgRangeTiles = 2,048 roundings, however
+// many replicas share the launch.
 // Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.78 ms (46.7 ms with 16 pixels staged
 // between two barriers and a shared-memory load per multiply-add).
-constexpr int kWgThreads = 192, kWgPxLog2 = 7;
+constexpr int kWgThreads = 192, kWgPxLog2 = 7, kWgRangeTiles = 64;
 
 struct ConvWgArgs {
   const void* x;
@@ -586,10 +586,14 @@ cudaError_t launch_conv3x3_simt(const ConvSimtArgs& c, cudaStream_t s) {
 
 // Ranges of one replica: three CTAs per SM over the replicas and channel blocks -- all that are resident,
 // in one wave -- and at least one tile each.  (Four per SM ran as a wave and a third: 55 against 46 us at 64 channels, 41 against 38 at 16.)
+// At most kWgRangeTiles tiles each, in as many waves as that takes, so that many replicas or a large batch
+// do not lengthen the fp32 chains: K = 64, B = 128, 16 x 16 pixels of 32 channels would otherwise be one range
+// of 256 tiles, 8,192 roundings.
 int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout) {
   const int blocks = ((cout + 15) / 16) * ((cin + 15) / 16);
   const int tiles = tile_of(B, hout, wout, kWgPxLog2).tiles;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 3LL * kNumSMs / ((int64_t)G * blocks)));
+  const int64_t wave = std::min<int64_t>(tiles, 3LL * kNumSMs / ((int64_t)G * blocks));
+  return (int)std::max<int64_t>(wave, (tiles + kWgRangeTiles - 1) / kWgRangeTiles);
 }
 
 cudaError_t launch_conv_wgrad_simt(const ConvSimtArgs& c, const void* dy, float* part, cudaStream_t s) {
