@@ -361,6 +361,7 @@ cudaError_t launch_fw(ConvFwArgs a, int G, cudaStream_t s) {
 // Measured, ResNet-20 in fp32, K = 4, B = 64, per step: 0.78 ms (46.7 ms with 16 pixels staged
 // between two barriers and a shared-memory load per multiply-add).
 constexpr int kWgThreads = 192, kWgPxLog2 = 7, kWgRangeTiles = 64;
+constexpr int64_t kSmemPerSm = 228 * 1024;  // of which each CTA takes 1 KB besides its own
 
 struct ConvWgArgs {
   const void* x;
@@ -532,15 +533,20 @@ __global__ void __launch_bounds__(kWgThreads, 3) conv_wgrad_simt_kernel(const __
   }
 }
 
-template <typename TA, int S>
-cudaError_t launch_wg(ConvWgArgs a, int G, cudaStream_t s) {
+// The staging's geometry at stride S, and its shared memory.
+size_t wg_staging(ConvWgArgs& a, int S) {
   a.pr = ((1 << a.t.th) - 1) * S + 3;
   a.pc = ((1 << a.t.tw) - 1) * S + 3;
   // odd row pitches: the two half-warps of a warp, a row apart, then read different banks
   a.xpitch = a.pc | 1;
   a.dpitch = (1 << a.t.tw) | 1;
   const size_t floats = (size_t)((a.dpitch << (a.t.th + a.t.ti)) + (a.pr << a.t.ti) * a.xpitch) * 16;
-  const size_t smem = std::max<size_t>(2 * floats, 3 * 48 * 16) * 4;
+  return std::max<size_t>(2 * floats, 3 * 48 * 16) * 4;
+}
+
+template <typename TA, int S>
+cudaError_t launch_wg(ConvWgArgs a, int G, cudaStream_t s) {
+  const size_t smem = wg_staging(a, S);
   const dim3 grid(a.nq, ((a.Co + 15) / 16) * a.ci_blocks, G);
   if (grid.y > 65535 || grid.z > 65535 || smem > 160 * 1024) return cudaErrorInvalidValue;
   static int attr_dev = -1;
@@ -584,15 +590,20 @@ cudaError_t launch_conv3x3_simt(const ConvSimtArgs& c, cudaStream_t s) {
   return two ? launch_fw<float, 2>(a, c.G, s) : launch_fw<float, 1>(a, c.G, s);
 }
 
-// Ranges of one replica: three CTAs per SM over the replicas and channel blocks -- all that are resident,
-// in one wave -- and at least one tile each.  (Four per SM ran as a wave and a third: 55 against 46 us at 64 channels, 41 against 38 at 16.)
+// Ranges of one replica: as many CTAs over the replicas and channel blocks as are resident, in one wave -- per
+// SM three, or the two or one whose staging its shared memory holds (stride 2, and outputs one or two rows
+// high) -- and at least one tile each.  (Four per SM ran as a wave and a third: 55 against 46 us at 64
+// channels, 41 against 38 at 16.  Three at stride 2, where two fit: 36.6 against 30.1 us for 16 x 16 pixels,
+// 42.5 against 34.2 for 8 x 8, K = 4, B = 64.)
 // At most kWgRangeTiles tiles each, in as many waves as that takes, so that many replicas or a large batch
 // do not lengthen the fp32 chains: K = 64, B = 128, 16 x 16 pixels of 32 channels would otherwise be one range
 // of 256 tiles, 8,192 roundings.
-int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout) {
-  const int blocks = ((cout + 15) / 16) * ((cin + 15) / 16);
-  const int tiles = tile_of(B, hout, wout, kWgPxLog2).tiles;
-  const int64_t wave = std::min<int64_t>(tiles, 3LL * kNumSMs / ((int64_t)G * blocks));
+int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout, int stride) {
+  ConvWgArgs a{};
+  a.t = tile_of(B, hout, wout, kWgPxLog2);
+  const int blocks = ((cout + 15) / 16) * ((cin + 15) / 16), tiles = a.t.tiles;
+  const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(3, kSmemPerSm / (wg_staging(a, stride) + 1024)));
+  const int64_t wave = std::min<int64_t>(tiles, per_sm * kNumSMs / ((int64_t)G * blocks));
   return (int)std::max<int64_t>(wave, (tiles + kWgRangeTiles - 1) / kWgRangeTiles);
 }
 
@@ -607,7 +618,7 @@ cudaError_t launch_conv_wgrad_simt(const ConvSimtArgs& c, const void* dy, float*
   a.Hi = c.hin, a.Wi = c.win, a.Ci = c.cin, a.Ho = c.hout, a.Wo = c.wout, a.Co = c.cout;
   a.ci_blocks = (c.cin + 15) / 16;
   a.t = tile_of(c.B, c.hout, c.wout, kWgPxLog2);
-  a.nq = conv_wgrad_simt_ranges(c.G, c.B, c.hout, c.wout, c.cin, c.cout);
+  a.nq = conv_wgrad_simt_ranges(c.G, c.B, c.hout, c.wout, c.cin, c.cout, c.stride);
   if (c.bf16)
     return c.stride == 2 ? launch_wg<uint16_t, 2>(a, c.G, s) : launch_wg<uint16_t, 1>(a, c.G, s);
   return c.stride == 2 ? launch_wg<float, 2>(a, c.G, s) : launch_wg<float, 1>(a, c.G, s);

@@ -331,7 +331,7 @@ struct ConvSimtArgs {
 };
 cudaError_t launch_conv3x3_simt(const ConvSimtArgs& a, cudaStream_t stream);
 // Weight-gradient partials part [G][conv_wgrad_simt_ranges()][cout][9][cin], to be added in order.
-int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout);
+int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout, int stride);
 cudaError_t launch_conv_wgrad_simt(const ConvSimtArgs& a, const void* dy, float* part,
                                    cudaStream_t stream);
 

@@ -1870,7 +1870,7 @@ lsgd_status conv_wgrad(ResNetPlan* p, int i, const void* in, float* Gr, cudaStre
         p->d_pad, 0, 0, s)));
     return LSGD_OK;
   }
-  const int nq = conv_wgrad_simt_ranges(K, p->B, c.hout, c.wout, c.cin, c.cout);
+  const int nq = conv_wgrad_simt_ranges(K, p->B, c.hout, c.wout, c.cin, c.cout, c.stride);
   const int J = 9 * c.cin;
   ConvSimtArgs ca = simt_args(p, c, K);
   ca.in = in;
@@ -2442,7 +2442,7 @@ lsgd_status resnet_alloc(ResNetPlan* p, const std::function<void*(size_t)>& allo
     p->rstd.push_back((float*)alloc((size_t)K * c.cout * 4));
     const int64_t P = (int64_t)B * c.hout * c.wout;
     const int64_t nq_s = (P + kRnChunk - 1) / kRnChunk;
-    const int64_t nq_w = conv_wgrad_simt_ranges(K, B, c.hout, c.wout, c.cin, c.cout);
+    const int64_t nq_w = conv_wgrad_simt_ranges(K, B, c.hout, c.wout, c.cin, c.cout, c.stride);
     part = std::max(part, (size_t)(K * nq_s * c.cout * 2));
     part = std::max(part, (size_t)(K * nq_w * c.cout * 9 * c.cin));
     float* wp = nullptr;

@@ -16,8 +16,8 @@ ConvSimtArgs simt(int bf16, int G, int B, int hout, int wout, int cin, int cout,
 
 extern "C" {
 
-int t_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout) {
-  return conv_wgrad_simt_ranges(G, B, hout, wout, cin, cout);
+int t_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout, int stride) {
+  return conv_wgrad_simt_ranges(G, B, hout, wout, cin, cout, stride);
 }
 
 int t_wgrad_simt(int G, int B, int hout, int wout, int cin, int cout, int stride, const float* x,

@@ -24,9 +24,24 @@ def test_chain_is_bounded(H, C):
     for K in (1, 2, 5, 16, 31, 64, 500):
         for B in (1, 7, 128, 1024, 8192):
             tiles = _tiles(B, H, H)
-            nq = L.t_wgrad_simt_ranges(K, B, H, H, C, C)
-            assert 1 <= nq <= tiles
-            assert -(-tiles // nq) * 128 // 4 <= LONGEST, (K, B, nq)
+            for stride in (1, 2):
+                nq = L.t_wgrad_simt_ranges(K, B, H, H, C, C, stride)
+                assert 1 <= nq <= tiles
+                assert -(-tiles // nq) * 128 // 4 <= LONGEST, (K, B, stride, nq)
+
+
+@pytest.mark.parametrize("H,W,C,stride,per_sm", [(32, 32, 16, 1, 3), (8, 8, 64, 1, 3), (1, 1, 16, 1, 2),
+                                                 (16, 16, 32, 2, 2), (8, 8, 64, 2, 2), (1, 1, 16, 2, 1)])
+def test_one_wave_where_the_chains_allow(H, W, C, stride, per_sm):
+    # CTAs that an SM holds: its 228 KB of shared memory over two staging buffers of 128 output pixels and
+    # the input under them, 64 bytes each, and 1 KB; 192 threads of at most 113 registers leave three
+    L = internal()
+    blocks = (C // 16) ** 2
+    B = 16000 if H == 1 else 4096 // H
+    for K in (1, 3, 4):
+        wave = per_sm * 152 // (K * blocks)
+        assert wave < _tiles(B, H, W) <= 64 * wave
+        assert L.t_wgrad_simt_ranges(K, B, H, W, C, C, stride) == wave
 
 
 @pytest.mark.gpu
@@ -41,7 +56,7 @@ def test_equal_terms_at_many_workers():
     v = np.float32(1 + 0.49 / 2048)
     x = torch.full((G, B, H, H, C), float(v), device="cuda")
     dy = torch.ones((G, B, H, H, C), device="cuda")
-    nq = L.t_wgrad_simt_ranges(G, B, H, H, C, C)
+    nq = L.t_wgrad_simt_ranges(G, B, H, H, C, C, 1)
     part = torch.full((G, nq, C, 3, 3, C), float("nan"), device="cuda")
     assert L.t_wgrad_simt(G, B, H, H, C, C, 1, ptr(x), ptr(dy), ptr(part), ctypes.c_void_p(0)) == 0
     torch.cuda.synchronize()
