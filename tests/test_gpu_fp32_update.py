@@ -15,18 +15,23 @@ from _gpu_common import built_package, dense_cfgs, dense_segments, max_rel_per_t
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("rule", ["plain", "heavy_ball", "nesterov"])
-@pytest.mark.parametrize("widths,K,B", [((516, 1), 2, 5),            # one output; split logits
-                                        ((129, 16), 3, 32),          # the widest narrow layer
-                                        ((513, 17), 2, 33),          # past it: the 32-wide tiles
-                                        ((260, 36, 3), 2, 1024),     # the narrow kernel's largest batch
-                                        ((260, 36, 3), 2, 1025),     # one more
-                                        ((1284, 516, 10), 16, 24),   # tiles of 128, ragged at both edges
-                                        ((321, 203, 7), 4, 9)])      # rows that are not 16-byte aligned
+CASES = pytest.mark.parametrize("widths,K,B", [
+    ((516, 1), 2, 5),            # one output; split logits
+    ((129, 16), 3, 32),          # the widest narrow layer
+    ((513, 17), 2, 33),          # past it: the 32-wide tiles
+    ((260, 36, 3), 2, 1024),     # the narrow kernel's largest batch
+    ((260, 36, 3), 2, 1025),     # one more
+    ((1284, 516, 10), 16, 24),   # tiles of 128, ragged at both edges
+    ((321, 203, 7), 4, 9)])      # rows that are not 16-byte aligned
+RULES = {"plain": dict(momentum=0.0), "heavy_ball": dict(momentum=0.9, weight_decay=1e-3),
+         "nesterov": dict(momentum=0.9, nesterov=True, weight_decay=1e-3)}
+
+
+@pytest.mark.parametrize("rule", list(RULES))
+@CASES
 def test_one_step_matches_the_oracle(widths, K, B, rule):
     P = built_package()
-    mom = {"plain": dict(momentum=0.0), "heavy_ball": dict(momentum=0.9, weight_decay=1e-3),
-           "nesterov": dict(momentum=0.9, nesterov=True, weight_decay=1e-3)}[rule]
+    mom = RULES[rule]
     N = 2 * K * B
     classes = max(widths[-1], 2)
     X, y = synthdata.gaussian_mixture_cached(N, widths[0], classes, 31)
@@ -47,5 +52,50 @@ def test_one_step_matches_the_oracle(widths, K, B, rule):
     segs = dense_segments(widths)
     for k in range(K):
         assert max_rel_per_tensor(P.lsgd_params(ctx, k), Wo[k], segs) <= 1e-5
+        if mom["momentum"]:  # u = 0.9 U + gradient, the largest of a tensor at least half the gradient's
+            assert max_rel_per_tensor(P.lsgd_momentum(ctx, k), Uo[k], segs) <= 2e-4
     np.testing.assert_allclose(P.lsgd_losses(ctx, 1, K)[0], lo[0], rtol=1e-5, atol=1e-6)
     P.lsgd_destroy(ctx)
+
+
+@pytest.mark.parametrize("rule", list(RULES))
+@CASES
+def test_one_step_has_the_bits_of_the_stand_alone_update(widths, K, B, rule):
+    # a step from zero momentum without decay leaves the gradient itself as the momentum; the stand-alone
+    # update on it and the case's own state is then the step's result, bit for bit
+    import torch
+
+    P = built_package()
+    mom, N = RULES[rule], 2 * K * B
+    X, y = synthdata.gaussian_mixture_cached(N, widths[0], max(widths[-1], 2), 31)
+    y = (y % widths[-1]).astype(np.int32)
+    rng = np.random.default_rng(10)
+    _, o = dense_cfgs(P, widths=widths, K=K, B=B, H=2, T=2, N=N, precision=P.FP32, seed=5)
+    W = np.tile(oracle.init_params(o, oracle.INIT_HE), (K, 1)).astype(np.float32)
+    U = (0.1 * rng.standard_normal(W.shape)).astype(np.float32)
+
+    def step(U0, **kw):
+        g, _ = dense_cfgs(P, widths=widths, K=K, B=B, H=2, T=2, N=N, precision=P.FP32, seed=5, **kw)
+        ctx = P.lsgd_create(g)
+        P.lsgd_set_dataset(ctx, X, y)
+        for k in range(K):
+            P.lsgd_set_params(ctx, k, W[k])
+            if kw["momentum"] and U0 is not None:
+                P.lsgd_set_momentum(ctx, k, U0[k])
+        P.lsgd_run(ctx, 1)
+        out = [np.stack([f(ctx, k) for k in range(K)]) for f in (P.lsgd_params, P.lsgd_momentum)]
+        P.lsgd_destroy(ctx)
+        return out
+
+    G = step(None, momentum=0.9)[1]
+    W1, U1 = step(U, **mom)
+    n = W.size + (-W.size) % 4
+    w, u, g = (torch.zeros(n, device="cuda") for _ in range(3))
+    for t, a in ((w, W), (u, U), (g, G)):
+        t[:W.size] = torch.from_numpy(a.reshape(-1)).cuda()
+    has_u = mom["momentum"] != 0
+    P.lsgd_sgd_update(w, u if has_u else None, g, None, n, 0.1, mom["momentum"], mom.get("nesterov", False),
+                      mom.get("weight_decay", 0.0))
+    assert np.array_equal(w[:W.size].cpu().numpy().reshape(W.shape), W1)
+    if has_u:
+        assert np.array_equal(u[:W.size].cpu().numpy().reshape(W.shape), U1)
