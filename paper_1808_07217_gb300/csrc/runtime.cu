@@ -721,7 +721,7 @@ lsgd_status dense_backward(lsgd_ctx* c, bool avg) {
       g.b_cs = 1;
       g.b_gs = (int64_t)B * Ly.ld_in;
       g.b_bf16 = c->bf16;
-      g.C = c->G + Ly.w_off;
+      g.C = c->fused ? nullptr : c->G + Ly.w_off;
       g.c_rs = Ly.in;
       g.c_gs = c->d_pad;
       g.c_bf16 = false;
@@ -968,7 +968,9 @@ lsgd_status lsgd_create(const lsgd_config* cfg, const lsgd_allocator* alloc, voi
 
   const size_t n_rep = (size_t)K * c->d_pad;
   c->W = (float*)dalloc(c, n_rep * 4);
-  c->G = (float*)dalloc(c, n_rep * 4);
+  // dense fp32 models update in their gradient kernels: nothing holds their gradients
+  const bool grads = c->bf16 || c->resnet;
+  if (grads) c->G = (float*)dalloc(c, n_rep * 4);
   if (c0.momentum != 0.0) c->U = (float*)dalloc(c, n_rep * 4);
   if (c->bf16) c->Wb = (uint16_t*)dalloc(c, n_rep * 2);
   if (!c->bf16 && !c->resnet) {
@@ -995,7 +997,7 @@ lsgd_status lsgd_create(const lsgd_config* cfg, const lsgd_allocator* alloc, voi
       return bail(LSGD_ENOMEM);
     }
   }
-  if (!c->W || !c->G || (c0.momentum != 0.0 && !c->U) || (c->bf16 && !c->Wb) || !c->idx ||
+  if (!c->W || (grads && !c->G) || (c0.momentum != 0.0 && !c->U) || (c->bf16 && !c->Wb) || !c->idx ||
       !c->yb || !c->tb || !c->loss_hist || !c->row_loss || !c->flag) {
     fail(nullptr, LSGD_ENOMEM, "device allocation failed");
     return bail(LSGD_ENOMEM);
@@ -1012,7 +1014,7 @@ lsgd_status lsgd_create(const lsgd_config* cfg, const lsgd_allocator* alloc, voi
     st = alloc_dense(c);
     if (st == LSGD_OK) st = init_dense_params(c);
     if (st == LSGD_OK) st = make_tc_maps(c);
-    // fp32: always (same bits; the gradient array is not written)
+    // fp32: always (the bits of the stand-alone update on the same gradient)
     if (st == LSGD_OK && (c0.fused_update || !c->bf16)) {
       c->fused = true;
       for (const DenseLayer& L : c->layers) c->fused = c->fused && (L.tc || !c->bf16);

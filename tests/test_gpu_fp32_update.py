@@ -99,3 +99,26 @@ def test_one_step_has_the_bits_of_the_stand_alone_update(widths, K, B, rule):
     assert np.array_equal(w[:W.size].cpu().numpy().reshape(W.shape), W1)
     if has_u:
         assert np.array_equal(u[:W.size].cpu().numpy().reshape(W.shape), U1)
+
+
+def test_no_gradient_array():
+    # the gradients are never in memory: one array of parameters, and the activations, are all that is asked for
+    import torch
+
+    P = built_package()
+    asked = []
+
+    def _alloc(user, nbytes, stream):
+        asked.append(int(nbytes))
+        return torch.cuda.caching_allocator_alloc(int(nbytes), 0, stream)
+
+    def _free(user, p, stream):
+        torch.cuda.caching_allocator_delete(p)
+
+    a = P.Allocator(P.ALLOC_FN(_alloc), P.FREE_FN(_free), None)
+    K, widths = 3, (2048, 2048, 10)
+    g, _ = dense_cfgs(P, widths=widths, K=K, B=4, H=1, T=1, N=64, precision=P.FP32)
+    ctx = P.lsgd_create(g, allocator=a)
+    params = 4 * K * sum(i * o for i, o in zip(widths[:-1], widths[1:]))
+    assert sum(n >= params for n in asked) == 1
+    P.lsgd_destroy(ctx)
