@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kFwThreads * KS, 4 / KS)
 
 template <typename TA, int S, int KS>
 cudaError_t launch_fw_ks(const ConvFwArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -549,7 +549,7 @@ cudaError_t launch_wg(ConvWgArgs a, int G, cudaStream_t s) {
   const size_t smem = wg_staging(a, S);
   const dim3 grid(a.nq, ((a.Co + 15) / 16) * a.ci_blocks, G);
   if (grid.y > 65535 || grid.z > 65535 || smem > 160 * 1024) return cudaErrorInvalidValue;
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

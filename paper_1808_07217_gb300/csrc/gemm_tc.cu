@@ -2635,7 +2635,7 @@ cudaError_t launch_one_tile(const TcGemmArgs& a, dim3 grid, int nk, cudaStream_t
   int sms = 0;
   const int dev = device_sms(&sms);
   if (dev < 0) return cudaErrorInvalidDevice;
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   if (attr_dev != dev) {
     cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
     if (e != cudaSuccess) return e;
@@ -2830,7 +2830,7 @@ cudaError_t launch_conv_tc(const ConvArgs& a, cudaStream_t stream, int* ctas_per
   ConvArgs la = a;
   la.ring_bytes = (int)ring;
   la.st32 = (reinterpret_cast<uintptr_t>(a.out) & 31) == 0 && a.out_gs % 8 == 0 ? 1 : 0;
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   if (attr_dev != dev) {
     e = cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)cv::SMEM_MAX);
@@ -2927,14 +2927,14 @@ cudaError_t launch_conv_sp(const ConvSpArgs& a, const void* in, cudaStream_t str
     return cudaErrorInvalidValue;
   const int mode = la.stats ? 1 : (la.bwd.y ? 2 : 0);
   const bool a32 = (out & 31) == 0;
-  static int attr_dev[2][5] = {{-1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1}};
+  static std::atomic<int> attr_dev[2][5];  // device + 1; several threads may launch
   auto run = [&](auto kernel, int threads) -> cudaError_t {
-    int& ad = attr_dev[la.tr == 16][a32 ? mode : 3 + mode];
-    if (ad != dev) {
+    std::atomic<int>& ad = attr_dev[la.tr == 16][a32 ? mode : 3 + mode];
+    if (ad != dev + 1) {
       const cudaError_t e =
           cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp::kOnePerSm);
       if (e != cudaSuccess) return e;
-      ad = dev;
+      ad = dev + 1;
     }
     return launch_pdl(kernel, dim3(cpr, la.G), dim3(threads), smem, stream, la);
   };
@@ -2981,7 +2981,7 @@ cudaError_t launch_wgrad_update(const WgradUpdateArgs& a, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   constexpr size_t smem = sizeof(WuSmem) + 1024;
   static_assert(smem <= 232448, "shared memory per CTA");
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   if (attr_dev != dev) {
     e = cudaFuncSetAttribute(wgrad_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
@@ -3137,7 +3137,7 @@ cudaError_t launch_conv_wgrad_tc(const ConvWgradArgs& a, cudaStream_t stream) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   if (attr_dev != dev) {
     e = cudaFuncSetAttribute(conv_wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              232448);
@@ -3173,7 +3173,7 @@ cudaError_t launch_pt(const TcGemmArgs& a, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   constexpr size_t smem = sizeof(PtSmem) + 1024;
   static_assert(smem <= 232448, "shared memory per CTA");
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   if (attr_dev != dev) {
     e = cudaFuncSetAttribute(gemm_pt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

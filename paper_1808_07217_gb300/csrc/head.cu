@@ -394,7 +394,7 @@ cudaError_t head_launch(const HeadArgs& h, bool backward, cudaStream_t stream) {
     return launch_pdl(head_forward_kernel<CMAX>, grid, dim3(kHeadThreads), (size_t)h.C * h.in * 2, stream, h);
   }
   const size_t smem = (size_t)(h.B + 8 * kHeadCols) * CMAX * sizeof(float);
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

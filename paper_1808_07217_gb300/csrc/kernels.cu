@@ -958,7 +958,7 @@ cudaError_t launch_narrow_update(const float* dz, int ld_dz, const float* act, i
       (sgd.mom != 0.f && !sgd.u))
     return cudaErrorInvalidValue;
   const size_t smem = (size_t)B * kNarrowMaxOut * sizeof(float);
-  static int attr_dev = -1;
+  static std::atomic<int> attr_dev{-1};  // several threads may launch
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

@@ -2,6 +2,8 @@
 counts, error handling (bad arguments, call order, failed allocation, non-finite parameters)."""
 import ctypes
 import os
+import subprocess
+import sys
 import tempfile
 
 import numpy as np
@@ -267,3 +269,40 @@ def test_default_allocator_and_launch_count(P):
     # bias gradient), the first layer's weight-gradient GEMM, the update
     assert per_step == 7
     P.lsgd_destroy(ctx)
+
+
+def test_first_launches_from_several_threads(P):
+    # every launcher raises its kernel's shared-memory limit before its first launch: in a process of its own,
+    # eight threads make the first calls at once, each on its own stream, and get one thread's results
+    code = """
+import sys, threading
+sys.path[:0] = [%r]
+import torch, paper_1808_07217_gb300 as P
+P.lib()
+G, B, H, C = 2, 4, 32, 16
+gen = torch.Generator(device="cuda").manual_seed(1)
+x = torch.randn((G, B, H, H, C), generator=gen, device="cuda").bfloat16()
+w = torch.randn((G, C, 3, 3, C), generator=gen, device="cuda").bfloat16()
+a = x.reshape(G, 128, 512)
+torch.cuda.synchronize()
+def work(out):
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        y, dx = torch.empty((G, B, H, H, C), device="cuda"), torch.empty((G, B, H, H, C), device="cuda")
+        dw, z = torch.empty((G, C, 3, 3, C), device="cuda"), torch.empty((G, 128, 128), device="cuda")
+        P.lsgd_conv3x3_bf16(P.CONV_FORWARD, x, w, y, G, B, H, H, C, C, 1)
+        P.lsgd_conv3x3_bf16(P.CONV_DGRAD, x, w, dx, G, B, H, H, C, C, 1)
+        P.lsgd_conv_wgrad_bf16(x, x, dw, G, B, H, H, C, C, 1)
+        P.lsgd_grouped_gemm_bf16(a, False, a, False, z, 128, 128, 512, G)
+    s.synchronize()
+    out.extend([y, dx, dw, z])
+outs = [[] for _ in range(9)]
+ts = [threading.Thread(target=work, args=(o,)) for o in outs[:8]]
+[t.start() for t in ts]
+[t.join() for t in ts]
+work(outs[8])
+assert all(len(o) == 4 and all(torch.equal(p, q) for p, q in zip(o, outs[8])) for o in outs)
+print("equal")
+""" % os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "equal" in r.stdout, r.stderr[-2000:]
