@@ -1557,8 +1557,11 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
       mbar_expect_tx(w_full, 9 * wtap);
       for (int t = 0; t < 9; ++t) tma_load_3d(wsm + t * wtap, &a.w_map, w_full, t * ck, 0, g);
     }
-    // a tile's first image and row; the next one is cpr tiles on
+    // a tile's first image and row; the next one is cpr tiles on: step_b images and step_y rows (walked
+    // image by image that is 512 steps for a single replica of 512 images of 16 x 16 pixels, 32 -> 64
+    // channels at stride 2: forward 10.0 us against 7.2)
     const int rows_img = a.hout, row_step = cpr * (BM / a.wout);
+    const int step_b = row_step / rows_img, step_y = row_step - step_b * rows_img;
     int b0 = (int)blockIdx.x * BM / per_img, y = (int)blockIdx.x * BM % per_img / a.wout;
     int q = 0, sl = 0;
     uint32_t ph = 1;
@@ -1584,8 +1587,9 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
           ph ^= 1;
         }
       }
-      y += row_step;
-      while (y >= rows_img) {
+      y += step_y;
+      b0 += step_b;
+      if (y >= rows_img) {
         y -= rows_img;
         ++b0;
       }
@@ -2040,6 +2044,18 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
   const uint32_t tmem = *tmem_slot;
   pdl_begin();  // everything above touched only shared memory and TMEM
 
+  // from tile t of image b to the CTA's next one, cpr tiles on (walked image by image, a single replica's
+  // 304 CTAs are as many steps per tile of 8 x 8 pixels: 512 images of 64 channels, forward 18.1 us against
+  // 11.2)
+  const int step_b = cpr / tpi, step_t = cpr - step_b * tpi;
+  auto next_tile = [&](int& b, int& t) {
+    t += step_t;
+    b += step_b;
+    if (t >= tpi) {
+      t -= tpi;
+      ++b;
+    }
+  };
   // an epilogue warp has read all that it reads of a tile's accumulators
   auto give_back = [&](int ab) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -2101,11 +2117,7 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
         sl = 0;
         ph ^= 1;
       }
-      t += cpr;
-      while (t >= tpi) {
-        t -= tpi;
-        ++b;
-      }
+      next_tile(b, t);
     }
     // copies in flight land before the CTA can exit
     for (int j = (q > nst ? q - nst : 0); j < q; ++j) mbar_wait(&full[j % nst], (j / nst) & 1);
@@ -2183,11 +2195,7 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
     };
     for (int tile = blockIdx.x; tile < tiles; tile += cpr) {
       const int img = b, tt = t;
-      t += cpr;
-      while (t >= tpi) {
-        t -= tpi;
-        ++b;
-      }
+      next_tile(b, t);
       bool ok = true;
       for (int seg = 0; seg < a.nseg; ++seg) {
         uint4 mk[2], so[2];
@@ -2308,11 +2316,7 @@ __global__ void __launch_bounds__(sp::kThreads<M, MODE>, MODE == 2 ? 1 : 2) conv
     uint32_t ph = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += cpr) {
       const int img = b, y_first = t * a.tr + quarter * (M / 32);  // this warp's first group row
-      t += cpr;
-      while (t >= tpi) {
-        t -= tpi;
-        ++b;
-      }
+      next_tile(b, t);
       if (!mbar_wait_warp(&acc_full[ab], ph)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
