@@ -283,22 +283,28 @@ __global__ void bn_act_fwd_kernel(const float* __restrict__ y, const float* __re
   }
 }
 
-constexpr int kMergeBatch = 8;  // partials per lane requested together
+constexpr int kMergeBatch = 8;  // partials per thread requested together
+constexpr int kMergeCh = 8;     // channels of a merging block: neighbours in a partial's row
 
 // The convolution epilogue's statistics partials (count, mean, M2; one per epilogue warp and CTA)
-// merged by Chan et al.'s formula: one warp per (replica, channel); lane l merges partials l,
-// l + 32, ... in order, then the fixed butterfly of bn_stats_finalize_kernel combines the lanes.
-__global__ void bn_merge_partials_kernel(const float4* __restrict__ stats, int nparts, int G, int C,
-                                         float* __restrict__ mean, float* __restrict__ rstd) {
+// merged by Chan et al.'s formula: one block per replica and kMergeCh channels (C a multiple of them);
+// chain l of a channel merges partials l, l + 32, ... in order, then the fixed butterfly of
+// bn_stats_finalize_kernel combines the 32 chains.  Eight threads read a partial's eight channels, one
+// line.  (With a warp per channel every lane read a line of its own: slow, and more so where the previous
+// convolution's CTAs leave few SMs free and the blocks gather there: convolution and merge of 1 x 512 images
+// of 16 x 16 pixels, 32 -> 64 channels at stride 2, 47 us against 18.)
+__global__ void __launch_bounds__(32 * kMergeCh) bn_merge_partials_kernel(
+    const float4* __restrict__ stats, int nparts, int C, float* __restrict__ mean, float* __restrict__ rstd) {
   pdl_begin();
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (wid >= G * C) return;
-  const int g = wid / C, c = wid % C;
-  const float4* src = stats + (int64_t)g * nparts * C + c;
+  __shared__ float chain[kMergeCh][3][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ch = threadIdx.x % kMergeCh, l = threadIdx.x / kMergeCh, first = blockIdx.x * kMergeCh;
+  const int g = first / C;
+  const float4* src = stats + (int64_t)g * nparts * C + first % C + ch;
   float n = 0.f, mu = 0.f, M2 = 0.f;
   // a batch of loads at a time, merged in order (one after another, eight round trips took 7.3 us
   // for 240 partials)
-  for (int q0 = lane; q0 < nparts; q0 += 32 * kMergeBatch) {
+  for (int q0 = l; q0 < nparts; q0 += 32 * kMergeBatch) {
     float4 v[kMergeBatch];
 #pragma unroll
     for (int i = 0; i < kMergeBatch; ++i)
@@ -307,6 +313,13 @@ __global__ void bn_merge_partials_kernel(const float4* __restrict__ stats, int n
     for (int i = 0; i < kMergeBatch; ++i)
       if (q0 + 32 * i < nparts) chan_merge(n, mu, M2, v[i].x, v[i].y, v[i].z);
   }
+  chain[ch][0][l] = n;
+  chain[ch][1][l] = mu;
+  chain[ch][2][l] = M2;
+  __syncthreads();
+  n = chain[warp][0][lane];
+  mu = chain[warp][1][lane];
+  M2 = chain[warp][2][lane];
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const float n2 = __shfl_xor_sync(0xffffffffu, n, o);
@@ -325,8 +338,8 @@ __global__ void bn_merge_partials_kernel(const float4* __restrict__ stats, int n
     M2 = Ma;
   }
   if (lane == 0) {
-    mean[wid] = mu;
-    rstd[wid] = 1.0f / sqrtf(M2 / n + kBnEps);
+    mean[first + warp] = mu;
+    rstd[first + warp] = 1.0f / sqrtf(M2 / n + kBnEps);
   }
 }
 
@@ -524,22 +537,23 @@ __global__ void bn_bwd_finalize_kernel(const float* __restrict__ part, int C, in
   }
 }
 
-// The same sums from the data-gradient convolution's epilogue partials (ConvBwdFuse): one warp
-// per (replica, channel); lane l adds partials l, l + 32, ... in order, then a fixed butterfly.
-__global__ void bn_bwd_merge_kernel(const float2* __restrict__ part, int nparts, int C, int G,
-                                    float* __restrict__ s12, float* __restrict__ Gr, int64_t g_off,
-                                    int64_t b_off, int64_t d_gs) {
+// The same sums from the data-gradient convolution's epilogue partials (ConvBwdFuse), read as
+// bn_merge_partials_kernel reads its: chain l adds partials l, l + 32, ... in order, then a fixed butterfly.
+__global__ void __launch_bounds__(32 * kMergeCh) bn_bwd_merge_kernel(
+    const float2* __restrict__ part, int nparts, int C, float* __restrict__ s12, float* __restrict__ Gr,
+    int64_t g_off, int64_t b_off, int64_t d_gs) {
   pdl_begin();
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (wid >= G * C) return;
-  const int g = wid / C, c = wid % C;
+  __shared__ float chain[kMergeCh][2][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ch = threadIdx.x % kMergeCh, l = threadIdx.x / kMergeCh, first = blockIdx.x * kMergeCh;
+  const int g = first / C, c = first % C + warp;
+  const float2* src = part + (int64_t)g * nparts * C + first % C + ch;
   float a = 0.f, b = 0.f;
-  for (int q0 = lane; q0 < nparts; q0 += 32 * kMergeBatch) {
+  for (int q0 = l; q0 < nparts; q0 += 32 * kMergeBatch) {
     float2 v[kMergeBatch];
 #pragma unroll
     for (int i = 0; i < kMergeBatch; ++i)
-      v[i] = q0 + 32 * i < nparts ? __ldg(part + ((int64_t)g * nparts + q0 + 32 * i) * C + c)
-                                  : make_float2(0.f, 0.f);
+      v[i] = q0 + 32 * i < nparts ? __ldg(src + (int64_t)(q0 + 32 * i) * C) : make_float2(0.f, 0.f);
 #pragma unroll
     for (int i = 0; i < kMergeBatch; ++i)
       if (q0 + 32 * i < nparts) {
@@ -547,14 +561,19 @@ __global__ void bn_bwd_merge_kernel(const float2* __restrict__ part, int nparts,
         b += v[i].y;
       }
   }
+  chain[ch][0][l] = a;
+  chain[ch][1][l] = b;
+  __syncthreads();
+  a = chain[warp][0][lane];
+  b = chain[warp][1][lane];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
   }
   if (lane == 0) {
-    s12[(int64_t)wid * 2] = a;
-    s12[(int64_t)wid * 2 + 1] = b;
+    s12[(int64_t)(first + warp) * 2] = a;
+    s12[(int64_t)(first + warp) * 2 + 1] = b;
     Gr[(int64_t)g * d_gs + g_off + c] = b;
     Gr[(int64_t)g * d_gs + b_off + c] = a;
   }
@@ -1722,8 +1741,8 @@ lsgd_status forward_impl(ResNetPlan* p, const float* W, const void* Wop, int w_g
       st = bn_stats(p, c, p->y[i], p->mean[i], p->rstd[i], G, s, launches);
       if (st != LSGD_OK) return st;
     } else {
-      RN_LAUNCH((launch_pdl(bn_merge_partials_kernel, (G * c.cout * 32 + 127) / 128, 128, 0, s,
-          cst, nparts, G, c.cout, p->mean[i], p->rstd[i])));
+      RN_LAUNCH((launch_pdl(bn_merge_partials_kernel, G * c.cout / kMergeCh, 32 * kMergeCh, 0, s,
+          cst, nparts, c.cout, p->mean[i], p->rstd[i])));
     }
     const bool second = i > 0 && i % 2 == 0;
     const TA* sc = second ? reinterpret_cast<const TA*>(p->act[i - 2]) : nullptr;
@@ -1780,8 +1799,8 @@ lsgd_status bn_backward(ResNetPlan* p, const ConvL& c, int i, const float* dout,
   const int nq = (int)((P + chunk - 1) / chunk);
   const int lanes = std::max(1, 256 / c.cout);
   if (fused_parts > 0) {
-    RN_LAUNCH((launch_pdl(bn_bwd_merge_kernel, (K * c.cout * 32 + 127) / 128, 128, 0, s, p->bpart,
-        fused_parts, c.cout, K, p->s12, Gr, c.g_off, c.b_off, p->d_pad)));
+    RN_LAUNCH((launch_pdl(bn_bwd_merge_kernel, K * c.cout / kMergeCh, 32 * kMergeCh, 0, s, p->bpart,
+        fused_parts, c.cout, p->s12, Gr, c.g_off, c.b_off, p->d_pad)));
   } else if (vec4_ok(c.cout))
     RN_LAUNCH((launch_pdl(bn_bwd_partial_v4_kernel<TA>, dim3(nq, K), 256, 0, s, dout,
         reinterpret_cast<const TA*>(out), p->y[i], p->mean[i], p->rstd[i], P, c.cout, nq, chunk,
@@ -2259,8 +2278,8 @@ lsgd_status conv3x3_bn_bf16(const uint16_t* in, const uint16_t* w, float* y, flo
                                x16 ? x16 + conv_x16_elems(G, B, hin, win) : nullptr, s, e,
                                &launches, stats, &nparts);
   if (st == LSGD_OK) {
-    launch_pdl(bn_merge_partials_kernel, (G * cout * 32 + 127) / 128, 128, 0, s, stats, nparts, G,
-               cout, mean, rstd);
+    launch_pdl(bn_merge_partials_kernel, G * cout / kMergeCh, 32 * kMergeCh, 0, s, stats, nparts, cout,
+               mean, rstd);
     const cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) {
       e = std::string("statistics merge: ") + cudaGetErrorString(ce);
