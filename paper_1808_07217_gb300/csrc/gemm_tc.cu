@@ -2897,11 +2897,10 @@ bool conv_sp_plan(ConvSpArgs& a, int sms, int* cpr, size_t* smem) {
   const size_t fixed = 1024 + (size_t)a.nkh * a.nj * (a.ck / 16) * 64 * a.nseg * 32 + sp::AUX;
   // Two CTAs per SM, where each still has two stages, overlap one's products with the other's epilogue; but
   // both lay out the weights (up to 73 KB), and alone a CTA has two accumulator sets for that.  So one where
-  // it gets at most eight tiles: forward of 512 images of 8 x 8 pixels, 64 channels, for 1 replica 11.1 -> 9.3
-  // us, for 4 9.9 -> 8.8; of 16 x 128 images of 16 x 16, 32 -> 64 at stride 2 (13 tiles) it would be 11.4 -> 12.7.
-  // With statistics only at 64 channels, where the layout is longest (4 replicas 15.6 -> 12.9): elsewhere
-  // the partials, one per CTA and warp, stay as they are.
-  const bool few = (int64_t)a.G * a.B * (a.hg / a.tr) <= 8LL * sms && (!a.stats || a.ck == 64);
+  // it gets at most eight tiles: forward of 1 x 512 images of 32 x 32 pixels, 16 channels, 11.7 -> 10.2 us,
+  // data gradient of 16 x 16 pixels, 32 -> 64 at stride 2, 14.2 -> 11.0; forward of 16 x 128 images of that (13
+  // tiles) would be 11.4 -> 12.7.  Not with statistics: their partials, one per CTA and warp, stay as they are.
+  const bool few = (int64_t)a.G * a.B * (a.hg / a.tr) <= 8LL * sms && !a.stats;
   int per_sm = 2;
   size_t st = sp::kTwoPerSm > fixed ? (sp::kTwoPerSm - fixed) / pitch : 0;
   if (st < 2 || a.bwd.y || few) {

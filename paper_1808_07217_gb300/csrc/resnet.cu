@@ -1352,6 +1352,15 @@ int conv_sp_takes(const ConvSpArgs& a) {
   return conv_sp_parts(a);
 }
 
+// 64 channels are one pixel to a super-pixel, and the super-pixel kernel's products have 64 rows where the
+// tap kernel's have 128: it is the faster one only through its statistics epilogue, where an SM gets more than
+// eight tiles of eight image rows.  8 x 8 pixels, tap kernel against this one, forward and with statistics: 1 x
+// 128 images 5.4 / 9.7 us against 6.7 / 11.3, 4 x 128 7.3 / 12.9 against 8.9 / 12.9, 16 x 128 16.7 / 30.9 against
+// 18.3 / 24.6.  (Both forms take the same kernel, and so give the same bits.)
+bool conv_sp_pays_forward(int G, int B, int hin, int cin) {
+  return cin < 64 || (int64_t)G * B * ((hin + 7) / 8) > 8LL * kNumSMs;
+}
+
 lsgd_status conv_fwd_tc(const uint16_t* x, const uint16_t* w, int64_t w_gs, float* y, int G, int B,
                         int hin, int win, int cin, int cout, int stride, uint16_t* x16,
                         uint16_t* wstem, cudaStream_t s, std::string& err, int64_t* launches,
@@ -1399,7 +1408,8 @@ lsgd_status conv_fwd_tc(const uint16_t* x, const uint16_t* w, int64_t w_gs, floa
     ca.ck = 16;
   } else {
     const ConvSpArgs sa = sp_args(w, w_gs, cin);
-    if (const int n = conv_sp_takes(sa)) {
+    const int n = conv_sp_pays_forward(G, B, hin, cin) ? conv_sp_takes(sa) : 0;
+    if (n) {
       if (nparts && stats) *nparts = n;
       CV_CALL(launch_conv_sp(sa, x, s));
       return LSGD_OK;
@@ -1457,7 +1467,10 @@ lsgd_status conv_dgrad_tc(const uint16_t* dy, const uint16_t* w, int64_t w_gs, f
     sa.out = dx;
     sa.out_gs = P * cin;
     if (bf) sa.bwd = *bf;
-    if (const int n = conv_sp_takes(sa)) {
+    // 64 channels without the BatchNorm backward, whose loads the super-pixel kernel hides better: the tap
+    // kernel (8 x 8 pixels: 1 x 128 images 7.2 us against 8.5, 4 x 128 9.7 against 11.3, 16 x 128 23.5 against 24.3)
+    const int n = bf || cout < 64 ? conv_sp_takes(sa) : 0;
+    if (n) {
       sa.bwd.part_gs = n;
       if (nparts && bf) *nparts = n;
       CV_CALL(launch_conv_sp(sa, dy, s));

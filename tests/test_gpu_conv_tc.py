@@ -90,6 +90,11 @@ FORWARD = [  # (G, B, Hin, Win, Cin, Cout, stride): ResNet-20's forward convolut
     (5, 7, 16, 16, 32, 32, 1),     # eight-row tiles, CTAs with unequal shares
     (2, 3, 32, 64, 16, 16, 1),     # rows wider than eight super-pixels: the tap kernel
     (2, 4, 8, 32, 16, 16, 1),      # eight image rows
+    (16, 76, 8, 8, 64, 64, 1),     # 64 channels at and past eight tiles per SM: tap kernel, super-pixels
+    (16, 78, 8, 8, 64, 64, 1),
+    (61, 5, 32, 32, 16, 16, 1),    # two tiles' CTAs of a replica, uneven steps to the next tile
+    (1, 700, 8, 8, 64, 64, 1),     # one replica: a CTA's next tile is hundreds of images on
+    (1, 332, 16, 16, 32, 64, 2),
 ]
 
 
@@ -200,6 +205,8 @@ BN_SHAPES = [  # (G, B, Hin, Win, Cin, Cout, stride): forward convolutions of Re
     (3, 6, 16, 16, 32, 64, 2),     # stage-3 entry: 64 channels, four 16-channel chunks
     (2, 6, 8, 8, 64, 64, 1),       # stage 3
     (16, 16, 32, 32, 16, 16, 1),   # many groups
+    (7, 180, 8, 8, 64, 64, 1),     # stage 3 on super-pixels
+    (1, 332, 16, 16, 32, 64, 2),   # one group: over a thousand partials
 ]
 
 
@@ -274,13 +281,13 @@ def test_conv_output_alignment_does_not_change_results(P):
 
 @pytest.mark.parametrize("mode,H,Cin,Cout,s", [(0, 32, 16, 16, 1), (0, 32, 16, 32, 2), (0, 32, 3, 16, 1),
                                                (0, 16, 32, 32, 1), (0, 8, 64, 64, 1), (1, 32, 16, 16, 1),
-                                               (1, 32, 16, 32, 2), (1, 8, 64, 64, 1)])
+                                               (1, 32, 16, 32, 2), (1, 16, 32, 64, 2)])
 def test_conv_output_alignment_does_not_change_the_512_value_rows(P, mode, H, Cin, Cout, s):
     # the same for the super-pixel kernel, whose order of sums is not the tap kernel's: it has to take
     # every output that the entry point takes
     import torch
 
-    G, B, Ho = 3, 4, H // s
+    G, B, Ho = 3, 410 if H == 8 else 4, H // s  # (64 channels: past eight tiles per SM)
     ishape, oshape = ((G, B, H, H, Cin), (G, B, Ho, Ho, Cout))[::1 if mode == 0 else -1]
     gen = torch.Generator(device="cuda").manual_seed(19)
     x = _bf16_randn(torch, ishape, gen)
@@ -319,3 +326,35 @@ def test_conv_rejects_outputs_that_are_not_16_byte_aligned(P):
             with pytest.raises(P.LsgdError) as e:
                 call()
             assert e.value.status == P.EINVAL
+
+
+def test_one_worker_costs_what_sixteen_do(P):
+    # the same images as one replica or as sixteen: the kernels' persistent CTAs and the partials' merge do
+    # the same work.  A replica's CTAs walking to the next tile image by image, or its partials merged by a
+    # warp per channel, cost two to four times.
+    import torch
+
+    def us(G, B, H, Cin, Cout, s, bn):
+        x = torch.ones((G, B, H, H, Cin), device="cuda", dtype=torch.bfloat16)
+        w = torch.ones((G, Cout, 3, 3, Cin), device="cuda", dtype=torch.bfloat16)
+        y = torch.empty((G, B, H // s, H // s, Cout), device="cuda")
+        m, r = torch.empty((G, Cout), device="cuda"), torch.empty((G, Cout), device="cuda")
+        times = []
+        for _ in range(7):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(10):
+                if bn:
+                    P.lsgd_conv3x3_bn_bf16(x, w, y, m, r, G, B, H, H, Cin, Cout, s)
+                else:
+                    P.lsgd_conv3x3_bf16(P.CONV_FORWARD, x, w, y, G, B, H, H, Cin, Cout, s)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        return min(times)
+
+    for H, Cin, Cout, s, bn in [(32, 16, 32, 2, False), (8, 64, 64, 1, False), (16, 32, 64, 2, False),
+                                (16, 32, 64, 2, True)]:
+        one, sixteen = us(1, 2048, H, Cin, Cout, s, bn), us(16, 128, H, Cin, Cout, s, bn)
+        print(H, Cin, Cout, s, bn, f"{one:.1f} {sixteen:.1f}")
+        assert one <= 1.6 * sixteen, (H, Cin, Cout, s, bn, one, sixteen)
