@@ -400,9 +400,10 @@ lsgd_status lsgd_conv3x3_bf16(int mode, const uint16_t* in, const uint16_t* W, f
  * ResNet-20), as the ResNet-20 training step computes them: y [G][B][Hout][Wout][Cout] fp32 as in
  * mode 0, and mean[G][Cout], rstd[G][Cout] = 1 / sqrt(biased variance + 1e-5) over the B Hout Wout
  * output positions of each group.  The convolution's epilogue keeps running (count, mean,
- * sum of squared deviations) partials per channel, combining the two-pass moments of its share of
- * every tile in tile order by Chan et al.'s formula; a second kernel combines the partials in a
- * fixed order, so the result is deterministic.  Same operands, alignment and shapes as mode 0 with
+ * sum of squared deviations) partials per channel over its share of the tiles, in tile order
+ * (Welford's update per value, or Chan et al.'s formula on each tile's two-pass moments); a second
+ * kernel combines the partials by Chan et al.'s formula in a fixed order, so the result is
+ * deterministic.  Same operands, alignment and shapes as mode 0 with
  * Cout <= 64; mean and rstd fp32 device arrays.  Scratch (the stem operands and the partials) is
  * allocated and freed on `stream`.  LSGD_EINVAL on bad arguments, LSGD_EUNSUPPORTED for shapes the
  * kernel does not take, LSGD_ENOMEM if the scratch cannot be allocated. */

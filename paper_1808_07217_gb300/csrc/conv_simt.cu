@@ -597,7 +597,8 @@ cudaError_t launch_conv3x3_simt(const ConvSimtArgs& c, cudaStream_t s) {
 // 42.5 against 34.2 for 8 x 8, K = 4, B = 64.)
 // At most kWgRangeTiles tiles each, in as many waves as that takes, so that many replicas or a large batch
 // do not lengthen the fp32 chains: K = 64, B = 128, 16 x 16 pixels of 32 channels would otherwise be one range
-// of 256 tiles, 8,192 roundings.
+// of 256 tiles, 8,192 roundings.  (The ranges, and so the last bits of a replica's gradient, depend on how
+// many replicas share the launch, as the tensor-core kernel's do.)
 int conv_wgrad_simt_ranges(int G, int B, int hout, int wout, int cin, int cout, int stride) {
   ConvWgArgs a{};
   a.t = tile_of(B, hout, wout, kWgPxLog2);

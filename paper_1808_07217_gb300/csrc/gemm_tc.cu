@@ -1890,14 +1890,14 @@ __global__ void __launch_bounds__(cv::THREADS, 2) conv_tc_kernel(const __grid_co
 // epilogue at 107 us (141 with the shortcut) for a first-stage layer of 16 workers x 128 images.
 // A lane then also holds few channels (8, or 16 of 64), so running moments and sums stay in its
 // registers until the end of the kernel: no exchange per tile.
-// Measured there: forward with statistics 44 us (201 MB: 4.6 TB/s), data gradient with the
+// Measured there: forward with statistics 41 us (201 MB: 4.9 TB/s), data gradient with the
 // BatchNorm-backward epilogue 66 (402 MB: 6.1 TB/s), 104 with the shortcut, where conv_tc_kernel took
 // 65, 102 and 135.
 // 16 outputs or 64 inputs to a pixel: each kernel row has partial columns of its own (npart), added by the
 // epilogue, which hands them back as soon as they are in registers.  A tensor-core sum rounds with every
 // product added: one chain over the kernel rows was off by 8.5e-8 and 3.0e-7 (relative, 16 and 64
 // channels, forward; 4.8e-7 the 64-channel data gradient) where three are off by 4.9e-8, 1.1e-7 and
-// 1.7e-7, as conv_tc_kernel is.  It costs 7.41 -> 7.79 ms for two ResNet-20 steps: fewer tiles in TMEM.  The
+// 1.7e-7, as conv_tc_kernel is.  It cost 7.41 -> 7.79 ms for two ResNet-20 steps: fewer tiles in TMEM.  The
 // partials are read eight registers at a time (sixteen spilled: 8.05 ms).
 // The BatchNorm-backward epilogue reads up to 192 bytes for every 64 it writes, and four warps that
 // went through a tile's rows one after another were bound by the latency of those reads (102 us, 158

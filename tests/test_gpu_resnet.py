@@ -174,9 +174,9 @@ def test_resnet20_conv_weight_gradients_per_layer(P, hwc, B):
     # initialisation these gradients are differences of nearly equal BatchNorm terms, so bf16
     # rounding alone moves them by 10-30 %: the bar is that the GPU lies closer to the oracle's
     # bf16 gradient than the oracle's own fp32 gradient does, layer by layer (a wrong tap or
-    # channel would put it at ~100 %).  At 32 x 32 every 3 x 3 convolution but the stem builds
-    # its column matrix in shared memory; at 16 x 16 the last stage's 4 x 4 images take the
-    # column-matrix GEMM instead.
+    # channel would put it at ~100 %).  At 32 x 32 every 3 x 3 convolution's weight gradient reads
+    # strips of its input; at 16 x 16 the last stage's 4 x 4 images take the column-matrix GEMM
+    # instead.
     N, K = 96, 2
     X, y = synthdata.gaussian_mixture(N, hwc[0] * hwc[1] * hwc[2], 10, seed=11)
     kw = dict(hwc=hwc, base=16, blocks=3, classes=10, K=K, B=B, H=4, T=4, N=N, base_lr=0.05,
